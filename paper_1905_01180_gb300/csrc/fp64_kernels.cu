@@ -960,13 +960,28 @@ gkba_status fp64_prepare_model(gkba_ctx* c) {
     GKBA_TRY(launch_end(c, t));
     t = launch_begin(c, K_PREP, 0.0, 0.0);
     k_build_vK64<<<grid1(N4, 256), 256, 0, c->stream>>>(c->N, c->v, c->vK64);
-    return launch_end(c, t);
+    GKBA_TRY(launch_end(c, t));
+    if (!c->oz) return GKBA_OK;
+    // stage S4 reads only the digit images of vK
+    GKBA_TRY(oz_prepare(c));
+    GKBA_TRY(oz_slice(c, c->vK64, n * n * n, 0, c->N, n * n * n, 1, c->vKimg));
+    GKBA_CUDA(c, cudaStreamSynchronize(c->stream));
+    cudaFree(c->vK64);
+    c->vK64 = nullptr;
+    return GKBA_OK;
 }
 
 gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz,
                          const double* B, long long ldb, long long sBz, double* out,
                          long long sOz, int M, int Nc, long long Ktot, int nz, int splitk,
                          long long Kc, StageMap map, double flops, double bytes) {
+    if (c->oz && !splitk) {
+        const int nzB = sBz ? nz : 1;
+        if (oz_img_bytes(Nc, Ktot) * nzB <= c->ozimg_bytes) {
+            GKBA_TRY(oz_slice(c, B, ldb, sBz, Nc, Ktot, nzB, c->ozimg));
+            return oz_gemm(c, cls, A, lda, sAz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
+        }
+    }
     dim3 grid((Nc + G64_BN - 1) / G64_BN, (M + G64_BM - 1) / G64_BM, nz);
     if (grid.y > 65535u) return fail(c, GKBA_EINVAL, "stage GEMM: M=%d too large", M);
     auto t = launch_begin(c, cls, flops, bytes);
@@ -1394,22 +1409,33 @@ gkba_status fp64_chain_x3(gkba_ctx* c, int nb, const double* A1, const StageMap*
     return GKBA_OK;
 }
 
-gkba_status contract_batch_fp64(gkba_ctx* c, int nb) {
+// Stage S4, D[(u,c,j)][i], split over K, and the reduction of its partial sums.
+gkba_status fp64_final(gkba_ctx* c, int nb) {
     const int N = c->N;
     const long long N2 = (long long)N * N, N3 = N2 * N, N4 = N3 * N;
-    double* X13 = (double*)c->X13;
-    const double fl_cr = 4.0 * (double)N4 * N;
-    GKBA_TRY(fp64_chain_x3(c, nb, c->wS64));
+    const double* X13 = (const double*)c->X13;
+    const double fl = 4.0 * (double)N4 * N * nb, by = 8.0 * (2 * N4 * nb + N4);
     const long long R = 2LL * N * nb;
-    const long long Kc = 8192;
-    const int nz = (int)((N3 + Kc - 1) / Kc);
-    {
-        StageMap m{0, 0, 1, 0, R, (int)R, 1, N};
-        GKBA_TRY(gemm64_stage(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, (double*)c->part, N * R,
-                              (int)R, N, N3, nz, 1, Kc, m, fl_cr * nb,
-                              8.0 * (2 * N4 * nb + N4)));
+    const StageMap m{0, 0, 1, 0, R, (int)R, 1, N};
+    const long long max_z = (long long)(c->part_bytes / (N * R * 8));
+    int nz;
+    if (c->oz) {
+        nz = oz_items(c, (int)R, N, N3, max_z);
+        GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m,
+                         fl, by));
+    } else {
+        // chunks that fill one wave of blocks when one unit has few output tiles
+        const long long Kc = nb > 1 ? 8192 : gemm64_splitk_chunk(c, (int)R, N, N3, max_z);
+        nz = (int)((N3 + Kc - 1) / Kc);
+        GKBA_TRY(gemm64_stage(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, (double*)c->part, N * R, (int)R, N, N3, nz, 1,
+                              Kc, m, fl, by));
     }
     return reduce_partials_launch(c, nb, nz, N * R, R, c->part, false, c->Su);
+}
+
+gkba_status contract_batch_fp64(gkba_ctx* c, int nb) {
+    GKBA_TRY(fp64_chain_x3(c, nb, c->wS64));
+    return fp64_final(c, nb);
 }
 
 // Self-energy of a structured interaction for nb units (G_u, Gb_u device

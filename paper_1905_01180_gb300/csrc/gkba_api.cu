@@ -107,7 +107,8 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const double part_per_unit = !gen ? 0.0
                                  : tc ? (std::ceil((double)Np * Np * Np / kTcItemK) * Np * 2.0 * Np * 4)
                                       : (std::ceil(N3 / 8192.0) * N * 2.0 * N * 8);
-    const double per_unit = 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
+    const double img_bytes = c->oz ? 1.25 * (double)oz_img_bytes(2 * (int)N, 2 * N) : 0.0;
+    const double per_unit = img_bytes + 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
     size_t cap = c->ws_cap;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
@@ -145,7 +146,13 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
         if (c->history == GKBA_HISTORY_TIME_LINEAR)
             part_bytes = std::max(part_bytes, (size_t)(1024LL * N * 2LL * N * 8));
     }
+    // partial sums of oz_gemm: at most two items per SM of 128 rows, or one item
+    if (c->oz) part_bytes = (size_t)N * 8 * std::max(2LL * c->num_sms * 128, 2LL * N * ub);
     const size_t oPart = cv.take(part_bytes);
+    // digit images of one stage's per-unit operands (the widest: S2 and S3); the
+    // time-linear accumulator's one long operand pads its windows differently
+    const size_t ozimg_bytes = c->oz ? (size_t)(img_bytes * ub) + ((size_t)64 << 10) : 0;
+    const size_t oImg = cv.take(ozimg_bytes);
     const size_t oB1 = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 2 * Np * Np * ub * 4) : (size_t)(2LL * NN * ub * 8));
     const size_t oG = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 4 * Np * Np * ub * 4) : (size_t)(4LL * NN * ub * 8));
     const size_t oG3 = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 4 * Np * Np * ub * 4) : (size_t)(4LL * NN * ub * 8));
@@ -170,6 +177,8 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     c->X2 = b + oX2;
     c->part = b + oPart;
     c->part_bytes = part_bytes;
+    c->ozimg = b + oImg;
+    c->ozimg_bytes = ozimg_bytes;
     c->formsB1 = b + oB1;
     c->formsG = b + oG;
     c->formsG3 = b + oG3;
@@ -425,7 +434,7 @@ void free_ctx(gkba_ctx* c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     void* ptrs[] = {c->tl_acc, c->tl_s, c->tl_W, c->tl_Wn, c->tl_uf,
                     c->h, c->d, c->v, c->vm, c->vjp, c->rhot_hist, c->U_hist, c->adj_ws, c->vomega,
-                    c->vgrad, c->hfK, c->wS64, c->vK64, c->wS32, c->vO32, c->xsw, c->vKhi, c->vKlo,
+                    c->vgrad, c->hfK, c->wS64, c->vK64, c->vKimg, c->wS32, c->vO32, c->xsw, c->vKhi, c->vKlo,
                     c->rho_hist, c->T_a, c->T_b, c->hhf_n, c->hhf_t, c->k1, c->k2, c->Ia, c->Ib,
                     c->U, c->ex0, c->ex1, c->ex2, c->tmp0, c->tmp1, c->dscal, c->dint, c->ws,
                     c->stage};
@@ -624,6 +633,8 @@ gkba_status gkba_init(gkba_ctx** out, const gkba_config* cfg, const double* h, c
     } else if (c->prec == GKBA_FP64) {
         ALLOC(c->wS64, N4 * 8);
         ALLOC(c->vK64, N4 * 8);
+        c->oz = N >= kOzMinN;
+        if (c->oz) ALLOC(c->vKimg, oz_img_bytes(N, (long long)N4 / N));
         if (c->history == GKBA_HISTORY_TIME_LINEAR) {
             ALLOC(c->tl_acc, 2 * N4 * 8);
             ALLOC(c->tl_s, 2 * N4 * 8);

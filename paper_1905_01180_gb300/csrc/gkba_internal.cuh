@@ -81,7 +81,9 @@ struct gkba_ctx {
 
     // FP64 contraction operands (natural N)
     double* wS64 = nullptr;  // [j][m][q][s] = w_mqsj
-    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn
+    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn (null when vKimg holds its digits)
+    bool oz = false;         // stage GEMMs on the FP16 tensor cores (oz_gemm.cu)
+    void* vKimg = nullptr;   // digit images of vK (oz)
 
     // split-TF32 contraction operands (padded Np, zero padding)
     float* wS32 = nullptr;    // raw FP32 [j][m][q][s]
@@ -131,6 +133,8 @@ struct gkba_ctx {
     void* formsB1 = nullptr;     // per-unit B operand of S1
     void* formsG = nullptr;      // per-unit B operand of S2/S3
     void* formsG3 = nullptr;     // per-unit B operand of S3 when its slot differs (sep_A)
+    void* ozimg = nullptr;       // digit images of one stage's B operands (oz)
+    size_t ozimg_bytes = 0;
     double2* vjp = nullptr;      // adjoint scratch: 10 blocks of vjp_units N*N units
     int vjp_units = 0;
     // trajectory record of gkba_step for the adjoint (steps adj_from .. n-1)
@@ -225,6 +229,23 @@ gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, l
                          const double* B, long long ldb, long long sBz, double* out,
                          long long sOz, int M, int Nc, long long Ktot, int nz, int splitk,
                          long long Kc, StageMap map, double flops, double bytes);
+
+// The same GEMM on the FP16 tensor cores, FP64 in and out (oz_gemm.cu).  B is
+// given as digit images: oz_img_bytes(Nc, K) bytes per z, written by oz_slice.
+// K is split into nitem ranges of whole windows (out += item * sOitem);
+// oz_items proposes a number of them for M x Nc outputs, at most max_items.
+size_t oz_img_bytes(int Nc, long long K);
+gkba_status oz_prepare(gkba_ctx* c);
+gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz, int Nc, long long K, int nz,
+                     void* img);
+int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items);
+gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const void* img,
+                    int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
+                    long long sOitem, StageMap map, double flops, double bytes);
+// Bases from which the FP64 stage GEMMs run there (a row tile holds 128 of N^3 rows).
+constexpr int kOzMinN = 6;
+// Stage S4 of the FP64 chain on the X3 of nb units in X13, with its reduction: S_u -> c->Su.
+gkba_status fp64_final(gkba_ctx* c, int nb);
 
 // Complex batched GEMM: C[b] = alpha * op(A[b]) * op(B[b]) + beta * C[b] (+ I if add_identity),
 // op = 'N' or 'C' (conjugate transpose); square n x n matrices, per-batch strides in elements.

@@ -184,15 +184,7 @@ gkba_status tl_apply(gkba_ctx* c, const double2* W, double2* I_out) {
     const StageMap mx3{N3, 1, N2, N4, N, N, N, N};
     GKBA_TRY(gemm64_stage(c, K_TL, c->tl_s, 2 * N, 0, Urc, 2 * N, 0, X13, 0, (int)N3, 2 * N, 2 * N,
                           1, 0, 0, mx3, fl, by));
-    // stage S4 on one unit: D[(c, j)][i] = sum_(n,r,p) X3[c][j][(n,r,p)] vK[i][(n,r,p)],
-    // split-K into chunks that fill one wave of blocks (one unit has few output tiles)
-    const long long R = 2LL * N;
-    const long long Kc = gemm64_splitk_chunk(c, (int)R, N, N3, (long long)(c->part_bytes / (N * R * 8)));
-    const int nz = (int)((N3 + Kc - 1) / Kc);
-    const StageMap m4{0, 0, 1, 0, R, (int)R, 1, N};
-    GKBA_TRY(gemm64_stage(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, (double*)c->part, N * R, (int)R, N,
-                          N3, nz, 1, Kc, m4, 4.0 * (double)N4 * N, 8.0 * 3 * N4));
-    GKBA_TRY(reduce_partials_launch(c, 1, nz, N * R, R, c->part, false, c->Su));
+    GKBA_TRY(fp64_final(c, 1));  // stage S4 on one unit
     // I = S Ucal^+ = S W
     return zgemm_batched(c, K_RED, N, 'N', 'N', make_double2(1.0, 0.0), c->Su, 0, W, 0,
                          make_double2(0.0, 0.0), I_out, 0, 1, 0);
