@@ -4,17 +4,20 @@
 //
 // The error-free splitting is that of Ozaki, Ogita, Oishi and Rump (Numer.
 // Algorithms 59, 2012), with integer digits and one scale per row and K window.
-// With E the largest biased exponent of the row's window, x = X 2^(E - 1076),
-// |X| < 2^54, and X = sum_{i=0..6} d_i 2^(8 (6 - i)) with d_i in [-128, 127]
-// (|d_0| <= 64): every digit is an FP16 integer.  The products of two windows
-// are grouped by level l = i + j, weight 2^(96 - 8 l); a level's sum over a
-// window of at most 96 K is an integer below 7 96 2^14 < 2^24, exact in the
-// tensor core's FP32 accumulator.  Levels 0 .. 7 are kept (34 of the 49 digit
-// products); the dropped ones are below 2^-60 of the window's largest product,
-// less than the rounding of X (2^-55 of the row's largest element).
+// With E the largest biased exponent of the row's window (at least 64),
+// x = X 2^(E - 1076), |X| < 2^54, and X = sum_{i=0..6} d_i 2^(8 (6 - i)) with
+// d_i in [-128, 127] (|d_0| <= 64): every digit is an FP16 integer.  The products
+// of two windows are grouped by level l = i + j, weight 2^(96 - 8 l); a level's
+// sum over a window of at most 96 K is an integer below 7 96 2^14 < 2^24, exact
+// in the tensor core's FP32 accumulator.  Levels 0 .. 7 are kept (34 of the 49
+// digit products); the dropped ones are below 2^-60 of the window's largest
+// product, less than the rounding of X (2^-54 of the row's largest element).
+// Elements below 2^-1012 count as zero (the floor of E).
 #pragma once
 
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #if defined(__CUDACC__)
 #define GKBA_OZ_HD __host__ __device__ __forceinline__
@@ -28,60 +31,120 @@ constexpr int kOzSlices = 7;   // digits of an element
 constexpr int kOzLevels = 8;   // digit-product levels kept
 constexpr int kOzMaxKw = 96;   // longest K window (exact level sums, see above)
 
-// Biased exponent of an FP64 bit pattern's high word; subnormals count as 1.
-GKBA_OZ_HD int oz_exponent(uint32_t hi) {
-    const int e = (int)((hi >> 20) & 0x7FFu);
-    return e > 1 ? e : 1;
-}
+constexpr uint32_t kOzExpMask = 0x7FF00000u;
+constexpr uint32_t kOzExpMin = 64u << 20;     // floor of E: zeros need a shift of 64
+constexpr int kOzNonFinite = 0x10000;         // window exponent of a row with Inf or NaN
 
-// Digits of the FP64 bit pattern u at the window exponent E >= its own: byte
-// 7 - i of the result is d_i + 128 (byte 0 is the dropped fraction; the added
-// 0x80 in it rounds to nearest).  Negative values are complemented, not
-// negated: off by 2^-8 of the last digit's unit.
-GKBA_OZ_HD uint64_t oz_digits(uint64_t u, int E) {
-    const uint32_t hi = (uint32_t)(u >> 32);
-    const uint32_t ef = (hi >> 20) & 0x7FFu;
-    const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | (ef ? 0x100000u : 0u)) << 32) | (uint32_t)u;
-    const int s = E - (int)(ef > 1u ? ef : 1u);
-    uint64_t t = s < 64 ? (m << 9) >> s : 0ull;
-    const uint64_t neg = (uint64_t)((int64_t)u >> 63);
-    t ^= neg;
-    return t + 0x8080808080808080ull;
+// Window exponent E from the largest exponent field (high word, masked) of a row.
+GKBA_OZ_HD int oz_exponent(uint32_t emax) { return emax == kOzExpMask ? kOzNonFinite : (int)(emax >> 20); }
+
+// Digits of the FP64 value (hi, lo) for a row whose largest exponent field is
+// emax >= kOzExpMin: byte 7 - i of the result is d_i + 128 (byte 0 is the
+// dropped fraction; the 0x80 added to it rounds to nearest).  Negative values
+// are complemented, not negated: off by 2^-8 of the last digit's unit.
+GKBA_OZ_HD uint64_t oz_digits(uint32_t hi, uint32_t lo, uint32_t emax) {
+    const uint32_t s = (emax >> 20) - ((hi << 1) >> 21);
+    const uint32_t m = (hi & 0xFFFFFu) | 0x100000u;
+    uint64_t t = ((uint64_t)((m << 9) | (lo >> 23)) << 32) | (uint32_t)(lo << 9);
+#if defined(__CUDA_ARCH__)
+    asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(t), "r"(s));  // 0 for s >= 64
+#else
+    t = s < 64 ? t >> s : 0ull;
+#endif
+    const uint64_t neg = (uint64_t)((int64_t)((uint64_t)hi << 32) >> 63);
+    return (t ^ neg) + 0x8080808080808080ull;
 }
 
 // Digit i (0 = leading) of an oz_digits word.
 GKBA_OZ_HD int oz_digit(uint64_t t, int i) { return (int)((t >> (8 * (7 - i))) & 0xFF) - 128; }
 
-// Round-to-nearest FP64 bit pattern of sum_l a_l 2^(96 - 8 l) 2^(Ea + Eb - 2152)
-// for level sums a_0 .. a_7 of a window of at most 96 K.  Integer arithmetic
-// only (the GPU's FP64 rate is 1/64 of its FP32 rate): the sum is formed as a
-// 64-bit integer in units of 2^-44 of level 0, |W| < 2^62.6, and normalised.
-// Ea or Eb = 0x7FF (a non-finite operand) gives NaN; results below the normal
-// range give zero.
-GKBA_OZ_HD int oz_clz64(uint64_t w) {
+// Powers of two as run-time values.  The multiply-adds by them then stay on the
+// FMA pipe; as constants they become shifts and adds on the integer pipe, which
+// has half the rate and bounds the kernels that use this header.
+struct OzMul {
+    int m4, m8, m12, m20, m28, one;
+};
+constexpr OzMul kOzMul = {1 << 4, 1 << 8, 1 << 12, 1 << 20, 1 << 28, 1};
+
 #if defined(__CUDA_ARCH__)
-    return __clzll((long long)w);
-#else
-    return w ? __builtin_clzll(w) : 64;
-#endif
+__device__ __forceinline__ uint32_t oz_mad(uint32_t a, int b, uint32_t c) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
 }
-GKBA_OZ_HD uint64_t oz_combine(const int (&a)[kOzLevels], int Ea, int Eb) {
-    const int c = a[5] * 16 + ((a[6] + (a[7] >> 8)) >> 4);
-    const int b3 = a[3] * 256 + a[4];
-    const int b1 = a[1] * 256 + a[2];
-    int64_t W = (int64_t)c + (int64_t)b3 * 4096 + (int64_t)b1 * (1 << 28);
-    W = (int64_t)((uint64_t)W + ((uint64_t)(uint32_t)(a[0] * 4096) << 32));
-    const uint64_t neg = (uint64_t)(W >> 63);
-    uint64_t w = (uint64_t)W ^ neg;
-    const int z = oz_clz64(w);
-    w <<= z & 63;
-    const int Er = Ea + Eb - z - 1014;
-    uint64_t r = (w >> 11) + ((w >> 10) & 1u) + ((uint64_t)(uint32_t)(Er - 1) << 52);
-    if (Er < 1 || z == 64) r = 0;
-    if (Er > 2046 && z != 64) r = 0x7FF0000000000000ull;
-    r |= neg & 0x8000000000000000ull;
-    if (Ea == 0x7FF || Eb == 0x7FF) r = 0x7FF8000000000000ull;
-    return r;
+__device__ __forceinline__ int64_t oz_mad_wide(int a, int b, int64_t c) {
+    int64_t d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+GKBA_OZ_HD uint32_t oz_bits(float x) { return __float_as_uint(x); }
+GKBA_OZ_HD int oz_int(float x) { return __float2int_rn(x); }
+GKBA_OZ_HD int oz_clz(uint32_t x) { return __clz((int)x); }
+GKBA_OZ_HD float oz_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+#else
+inline uint32_t oz_mad(uint32_t a, int b, uint32_t c) { return a * (uint32_t)b + c; }
+inline int64_t oz_mad_wide(int a, int b, int64_t c) { return (int64_t)a * b + c; }
+inline uint32_t oz_bits(float x) {
+    uint32_t u;
+    std::memcpy(&u, &x, 4);
+    return u;
+}
+inline int oz_int(float x) { return (int)std::lrintf(x); }
+inline int oz_clz(uint32_t x) { return x ? __builtin_clz(x) : 32; }
+inline float oz_fma(float a, float b, float c) { return std::fmaf(a, b, c); }
+#endif
+
+// FP64 bit pattern (round to nearest) of sum_l a_l 2^(96 - 8 l) 2^(Ea + Eb - 2152)
+// for the level sums a_0 .. a_7 of a window of at most 96 K; Es = Ea + Eb - 1014.
+// Integer and FP32 arithmetic only (the FP64 rate is 1/64 of the FP32 rate).
+//
+// oz_sum: the sum as a 64-bit integer W = (hi, lo) in units of 2^-44 of level 0
+// (|W| < 2^62.6).  The sums of levels 0 - 2 are below 2^22 and become integers
+// by adding 1.5 2^23 (the conversion instruction runs at an eighth of the FP32
+// rate; the constant's bits 0x4B400000 vanish modulo 2^32 when shifted by 12);
+// levels 6 and 7 are rounded to W's unit together.
+GKBA_OZ_HD void oz_sum(const float (&a)[kOzLevels], const OzMul& k, uint32_t& hi, uint32_t& lo) {
+    const float kMagic = 12582912.0f;
+    const uint32_t m0 = oz_bits(a[0] + kMagic), m1 = oz_bits(a[1] + kMagic), m2 = oz_bits(a[2] + kMagic);
+    const int c = (int)oz_mad((uint32_t)oz_int(a[5]), k.m4,
+                              (uint32_t)oz_int(oz_fma(a[7], 1.0f / 4096.0f, a[6] * 0.0625f)));
+    const int b3 = (int)oz_mad((uint32_t)oz_int(a[3]), k.m8, (uint32_t)oz_int(a[4]));
+    const int b1 = (int)oz_mad(m1, k.m8, m2 - 257u * 0x4B400000u);
+    const int64_t W = oz_mad_wide(b1, k.m28, oz_mad_wide(b3, k.m12, (int64_t)c));
+    hi = oz_mad(m0, k.m12, (uint32_t)((uint64_t)W >> 32));
+    lo = (uint32_t)W;
+}
+// W as FP64 when its absolute value's high word ha is not zero and the biased
+// exponent e1 + 1 is in 1 .. 2046 (the caller checks both).
+GKBA_OZ_HD uint64_t oz_pack(uint32_t hi, uint32_t lo, int Es, const OzMul& k, uint32_t& ha, uint32_t& e1) {
+    const uint32_t neg = (uint32_t)((int32_t)hi >> 31);
+    ha = hi ^ neg;
+    // leading bit to bit 62, half a unit of the last place added, exponent in place
+    const int z = oz_clz(ha);
+    uint64_t w = ((uint64_t)ha << 32) | (lo ^ neg);
+    w = (uint64_t)oz_mad_wide(0x200, k.one, (int64_t)(w << (z - 1))) >> 10;
+    e1 = (uint32_t)(Es - 1 - z);
+    const uint32_t rh = oz_mad(e1, k.m20, (uint32_t)(w >> 32)) | (neg & 0x80000000u);
+    return ((uint64_t)rh << 32) | (uint32_t)w;
+}
+GKBA_OZ_HD bool oz_packed(uint32_t ha, uint32_t e1) { return ha != 0u && e1 <= 2045u; }
+// W as FP64 in every case: Es >= kOzNonFinite / 2 (a non-finite operand) gives
+// NaN, results below the normal range zero.
+GKBA_OZ_HD uint64_t oz_pack_any(uint32_t hi, uint32_t lo, int Es) {
+    const uint32_t neg = (uint32_t)((int32_t)hi >> 31);
+    hi ^= neg;
+    lo ^= neg;
+    int z = oz_clz(hi);
+    if (hi == 0) z = 32 + oz_clz(lo);
+    uint64_t w = ((uint64_t)hi << 32) | lo;
+    w = ((w << ((z - 1) & 63)) + 0x200u) >> 10;
+    const int Er = (hi | lo) == 0 ? Es - 4096 : Es - z;
+    uint32_t rh = (uint32_t)(w >> 32) + ((uint32_t)(Er - 1) << 20), rl = (uint32_t)w;
+    if ((uint32_t)(Er - 1) > 2045u) {
+        rh = Es >= kOzNonFinite / 2 ? 0x7FF80000u : Er > 2046 ? 0x7FF00000u : 0u;
+        rl = 0u;
+    }
+    return ((uint64_t)(rh | (neg & 0x80000000u)) << 32) | rl;
 }
 
 }  // namespace gkba

@@ -11,9 +11,13 @@
 // together with integer instructions only.  The result is closer to the exact
 // sum than the FMA chain's (tests/test_oz_digits.py; whole Heun steps and
 // self-energies: 1.1-2.0e-15 from 64-bit references where the FMA chain had
-// 1.8-3.3e-15).  Whole calls, FMA chain -> here: Heun step at N = 24, 301 points
-// 309 -> 36 ms; 40 self-energies at N = 33 78 -> 5.8 ms; Heun step at N = 10, 501
-// points 23.8 -> 3.6 ms; three time-linear steps at N = 48 137 -> 20 ms.
+// 1.2-2.8e-15).  Whole calls, FMA chain -> here: Heun step at N = 24, 301 points
+// 309 -> 17.1 ms; 40 self-energies at N = 33 78 -> 2.7 ms; Heun step at N = 10,
+// 501 points 23.8 -> 1.7 ms; three time-linear steps at N = 48 137 -> 14.1 ms.
+//
+// What bounds it: the integer instructions of the epilogue and the converter
+// (about 64 a result and 47 an element; at N = 24 the integer pipe is 52 % busy,
+// the tensor pipe 27 %, DRAM 25 %).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -27,13 +31,19 @@ namespace gkba {
 namespace {
 
 constexpr int kOzBM = 128;       // rows per tile (tensor-memory lanes)
+constexpr int kOzLbo = kOzBM * 16 + 32;  // bytes between the 8-wide K chunks of a digit plane of A
 constexpr int kOzMaxNB = 32;     // columns per accumulator: 8 levels x 32 = 256 TMEM columns
 constexpr int kOzSub = 6;        // 8-wide K chunks of one B pipeline stage (48 K)
-constexpr int kOzRing = 8;       // row-exponent ring (windows in flight)
-constexpr int kOzEpiWarps = 8, kOzConvWarps = 8;
-constexpr int kOzThreads = 32 * (kOzEpiWarps + kOzConvWarps + 2);
+constexpr int kOzRing = 8;       // exponent rings: more than the windows and accumulators in flight
+// Warps of the kernel: epilogue, converter, then producer, MMA issuer and two
+// that fill the warpgroup.
+constexpr int kOzConvWarps = 8;
+constexpr int oz_epi_warps(bool multi) { return multi ? 8 : 16; }
+constexpr int oz_threads(bool multi) { return 32 * (oz_epi_warps(multi) + kOzConvWarps + (multi ? 2 : 4)); }
 constexpr size_t kOzSmemMax = 227 * 1024;
-constexpr int kOzMisc = kOzRing * kOzBM * 4 + 256;  // row exponents, barriers
+constexpr int kOzMaxCols = 256;  // 2 N, N <= 128
+// column offsets, row and column exponent rings, barriers
+constexpr int kOzMisc = kOzMaxCols * 4 + kOzRing * (kOzBM + kOzMaxNB) * 4 + 256;
 
 // Shape of one GEMM: column blocks of NB (a multiple of 8, at most 32) and K
 // windows of kw (a multiple of 16, at most 96).
@@ -68,12 +78,13 @@ struct OzParams {
     double* out;
     long long sOz;
     StageMap map;
-    int Nc, NB, nblk, kw, nwin;
+    int Nc, NB, nblk, nwin;
     long long K;
     int mtiles;          // ceil(M / 128)
     int nitem, wper;     // split K: items per row tile, windows per item
     long long sOitem;
     long long tiles;     // z x item x row tile
+    OzMul mul;
     int na, nbs;         // A and B pipeline stages
     int* err;
 };
@@ -83,8 +94,9 @@ struct OzParams {
 // K-major core-matrix layout the MMA reads (8 rows x 16 bytes, no swizzle):
 // row j NB + c holds digit j of column c of the block, rows 7 NB .. 8 NB - 1
 // are zero (they clear the accumulator's last level).  A window's K is
-// permuted, chunk p holding k = p + no q (q = 0..7, no the window's chunks), as
-// the converter of A does.
+// permuted as the converter of A reads it: of the no chunks of the window,
+// chunk p holds k = p + no q, q = 0..7 (K odd), or the pairs 2 (p + no q) + {0, 1},
+// q = 0..3 (K even, 16-byte loads).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, long long ldb, long long sBz,
                                                   int Nc, long long K, int NB, int nblk, int kw, int nwin,
@@ -103,25 +115,27 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
     const int Kw = (int)(K - k0 < kw ? K - k0 : kw);
     const int no = 2 * ((Kw + 15) / 16);
     const double* b = B + z * sBz + (long long)col * ldb + k0;
-    uint64_t x[2][2];
-    int E = 1;
+    uint2 x[2][2];  // (lo, hi)
+    uint32_t emax = kOzExpMin;
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int p = (lane >> 2) + 8 * u, k = p + no * (2 * (lane & 3) + h);
-            x[u][h] = (col < Nc && p < no && k < Kw) ? (uint64_t)__double_as_longlong(b[k]) : 0ull;
-            E = max(E, oz_exponent((uint32_t)(x[u][h] >> 32)));
+            const int p = (lane >> 2) + 8 * u, q = lane & 3;
+            const int k = (K & 1) ? p + no * (2 * q + h) : 2 * (p + no * q) + h;
+            x[u][h] = make_uint2(0u, 0u);
+            if (col < Nc && p < no && k < Kw) x[u][h] = *reinterpret_cast<const uint2*>(b + k);
+            emax = max(emax, x[u][h].y & kOzExpMask);
         }
-    E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
-    if (lane == 0) ecol[z * ecol_z + (long long)w * ncp + col] = E;
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    if (lane == 0) ecol[z * ecol_z + (long long)w * ncp + col] = oz_exponent(emax);
     const int blk = col / NB, c = col % NB;
     uint8_t* o = img + z * img_z + ((long long)w * nblk + blk) * (kw / 8) * (8 * NB * 16);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
         const int p = (lane >> 2) + 8 * u;
         if (p >= no) continue;
-        const uint64_t t0 = oz_digits(x[u][0], E), t1 = oz_digits(x[u][1], E);
+        const uint64_t t0 = oz_digits(x[u][0].y, x[u][0].x, emax), t1 = oz_digits(x[u][1].y, x[u][1].x, emax);
         uint8_t* op = o + (long long)p * (8 * NB * 16) + c * 16 + (lane & 3) * 4;
 #pragma unroll
         for (int j = 0; j < kOzSlices; ++j) {
@@ -135,13 +149,18 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
 // ---------------------------------------------------------------------------
 // The GEMM kernel: one CTA per SM, persistent over 128-row tiles.
 //
-// Warps 0-7 epilogue (two per tensor-memory lane quarter, half of a block's
-// columns each), 8-15 converter (16 rows each), 16 TMA producer of B's digit
-// images, 17 MMA issuer.
+// Warps: the epilogue (two warps per tensor-memory lane quarter, half of a
+// block's columns each; with one K window two such groups drain alternate
+// accumulators), 8 converter warps (16 rows each), one producer of B's digit
+// images and one MMA issuer.  Epilogue and converter are long chains of integer
+// instructions that bound the kernel together; a second epilogue group overlaps
+// more of them (N = 33: 78 -> 68 us a self-energy).
 //
 // A: the converter reads a window's rows (FP64, through L1), takes the row's
 // largest exponent, and writes the seven digit planes [chunk][128 rows][16 B]
-// to shared memory (na stages).  B: bulk copies of pre-split images, one stage
+// to shared memory (na stages).  The four lanes of a row read 64 contiguous
+// bytes; chunks are kOzLbo apart, 32 bytes off a multiple of 128, so that eight
+// lanes (two rows, four chunks) store to different banks.  B: bulk copies of pre-split images, one stage
 // per 48 K of a 32-column block (nbs stages).  Digit i of A times the stacked
 // digits 0 .. of B is one MMA of N = (digits) x NB columns at column offset
 // i NB of the accumulator: level l = i + j lands in columns [l NB, (l+1) NB),
@@ -154,14 +173,21 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
 // once and multiplied with every column block.  Longer K: per block and
 // window, the window results are added in FP64 registers.
 // ---------------------------------------------------------------------------
-__device__ bool oz_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+// Bounded wait.  The tries sleep in between (polls without it were a seventh of
+// the issued instructions, of a kernel bound by them); the timer is read once in
+// 64 tries.
+__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int code,
+                                        unsigned sleep_ns = 40) {
     if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = gtimer();
+    unsigned long long t0 = 0;
     for (uint32_t it = 1;; ++it) {
+        __nanosleep(sleep_ns);
         if (mbar_try(bar, parity)) return true;
         if ((it & 63u) == 0) {
             if (*abort_flag) return false;
-            if (gtimer() - t0 > kWaitLimitNs) {
+            const unsigned long long now = gtimer();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitLimitNs) {
                 *abort_flag = 1;
                 atomicCAS(err, 0, code);
                 return false;
@@ -213,32 +239,69 @@ __device__ __forceinline__ unsigned long long desc_plain(uint32_t saddr, uint32_
            (unsigned long long)(128 >> 4) << 32 | 1ull << 46;
 }
 
-// The position of a tile: unit z, split-K item and row tile.
-struct OzTile {
+// Position of a tile in a CTA's range (row tiles fastest, then split-K items,
+// then units), advanced without divisions.
+struct OzPos {
     long long z;
     int item, mt, w0, nw;
-    __device__ OzTile(const OzParams& p, long long t) {
+    __device__ __forceinline__ OzPos(const OzParams& p, long long t) {
         mt = (int)(t % p.mtiles);
         const long long r = t / p.mtiles;
         item = (int)(r % p.nitem);
         z = r / p.nitem;
+        windows(p);
+    }
+    __device__ __forceinline__ void windows(const OzParams& p) {
         w0 = item * p.wper;
         nw = min(p.wper, p.nwin - w0);
     }
+    __device__ __forceinline__ void next(const OzParams& p) {
+        if (++mt < p.mtiles) return;
+        mt = 0;
+        if (++item == p.nitem) {
+            item = 0;
+            ++z;
+        }
+        windows(p);
+    }
 };
 
-template <bool MULTI>
-__global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant__ OzParams p) {
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    const uint32_t plane = (uint32_t)(kOzBM * p.kw * 2);          // one digit plane of A
+// 8-wide K chunks of window w (an even number, NO but for a short last window).
+template <int NO, bool MULTI>
+__device__ __forceinline__ int oz_chunks(const OzParams& p, int w) {
+    if (!MULTI) return NO;
+    const long long left = p.K - (long long)w * (8 * NO);
+    return left >= 8 * NO ? NO : 2 * (((int)left + 15) >> 4);
+}
+
+// Register split of the one-window kernel (28 warps, 72 registers a thread at
+// launch): 16 x 64 + 8 x 104 + 4 x 40 = 28 x 72.
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+template <int NO, bool MULTI, bool VEC>
+__global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_constant__ OzParams p) {
+    // used as declared, without integer casts: those would lose the address space
+    // and turn every access into a generic one (four times the latency)
+    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int kEpi = oz_epi_warps(MULTI), kWorkers = kEpi + kOzConvWarps;
+    constexpr int KW = 8 * NO;                                    // K of a window
+    constexpr uint32_t kPlane = (uint32_t)(NO * kOzLbo);          // one digit plane of A
+    constexpr uint32_t kAStage = kOzSlices * kPlane;
     const uint32_t brow = (uint32_t)(8 * p.NB * 16);              // one 8-wide K chunk of a block's image
-    const int no_full = p.kw / 8;
-    const uint32_t bstage = (uint32_t)min(kOzSub, no_full) * brow;
+    const uint32_t bstage = (uint32_t)(NO < kOzSub ? NO : kOzSub) * brow;
     uint8_t* sA = smem;
-    uint8_t* sB = sA + (size_t)p.na * kOzSlices * plane;
-    int* sExp = (int*)(sB + (size_t)p.nbs * bstage);
-    uint64_t* bars = (uint64_t*)(sExp + kOzRing * kOzBM);
+    uint8_t* sB = sA + (size_t)p.na * kAStage;
+    uint32_t* sCol = (uint32_t*)(sB + (size_t)p.nbs * bstage);  // output offset of each column
+    int* sExp = (int*)(sCol + kOzMaxCols);
+    int* sEcol = sExp + kOzRing * kOzBM;  // column exponents of an accumulator
+    uint64_t* bars = (uint64_t*)(sEcol + kOzRing * kOzMaxNB);
     constexpr int AFULL = 0, AEMPTY = 2, BFULL = 4, BEMPTY = 8, ACCF = 12, ACCE = 14, DRAIN = 16, NBARS = 17;
     uint32_t* tmem_slot = (uint32_t*)(bars + NBARS);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
@@ -249,7 +312,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
             mbar_init(bar(AFULL + s), kOzConvWarps);
             mbar_init(bar(AEMPTY + s), 1);
             mbar_init(bar(ACCF + s), 1);
-            mbar_init(bar(ACCE + s), kOzEpiWarps);
+            mbar_init(bar(ACCE + s), 8);
         }
         for (int s = 0; s < 4; ++s) {
             mbar_init(bar(BFULL + s), 1);
@@ -259,7 +322,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
         *abort_flag = 0;
         fence_barrier_init();
     }
-    if (warp == 17) {
+    for (int col = threadIdx.x; col < p.Nc; col += oz_threads(MULTI))
+        sCol[col] = (uint32_t)((long long)(col / p.map.Dy) * p.map.SC + (long long)(col % p.map.Dy) * p.map.SY);
+    if (warp == kWorkers + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -268,58 +333,101 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const long long t0 = p.tiles * blockIdx.x / gridDim.x, t1 = p.tiles * (blockIdx.x + 1) / gridDim.x;
+    const long long t0 = p.tiles * blockIdx.x / gridDim.x;
+    const int ntile = (int)(p.tiles * (blockIdx.x + 1) / gridDim.x - t0);
+    OzPos T(p, t0);
 
-    if (warp < kOzEpiWarps) {
+    if (warp < kEpi) {
         // ---------------- epilogue ----------------
-        const int q = warp & 3, h = warp >> 2;
+        if (!MULTI) regs_dec<64>();
+        const int q = warp & 3, h = (warp >> 2) & 1, grp = warp >> 3;
         const int half = p.NB / 2, cb = h * half;  // this warp's columns of a block (a multiple of 4)
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
+        const OzMul mul = p.mul;
         uint32_t aseq = 0, accseq = 0;
         bool ok = true;
-        for (long long t = t0; t < t1 && ok; ++t) {
-            const OzTile T(p, t);
-            const uint32_t row = (uint32_t)T.mt * kOzBM + q * 32 + lane;
-            const bool rok = row < (uint32_t)p.M;
-            const uint32_t x = row % (uint32_t)p.map.Dx, rb = row / (uint32_t)p.map.Dx;
-            double* o = p.out + T.z * p.sOz + T.item * p.sOitem + (long long)(rb / (uint32_t)p.map.Db) * p.map.SA +
-                        (long long)(rb % (uint32_t)p.map.Db) * p.map.SB + (long long)x * p.map.SX;
+        // row = (ra Db + rb) Dx + rx of the output map; a tile further is 128 rows
+        // = (ia, ib, ix) further, with carries (a division is 20 instructions)
+        const int Dx = p.map.Dx, Db = p.map.Db;
+        const int ix = kOzBM % Dx, ib = (kOzBM / Dx) % Db, ia = kOzBM / Dx / Db;
+        int rx = 0, rb = 0, ra = 0;
+        for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
+            const int row = T.mt * kOzBM + q * 32 + lane;
+            const bool rok = row < p.M;
+            if (t == 0 || T.mt == 0) {
+                rx = row % Dx;
+                rb = (row / Dx) % Db;
+                ra = row / Dx / Db;
+            } else {
+                rx += ix;
+                rb += ib;
+                ra += ia;
+                if (rx >= Dx) {
+                    rx -= Dx;
+                    ++rb;
+                }
+                if (rb >= Db) {
+                    rb -= Db;
+                    ++ra;
+                }
+            }
+            double* o = p.out + T.z * p.sOz + T.item * p.sOitem + ra * p.map.SA + rb * p.map.SB + rx * p.map.SX;
             const int nouter = MULTI ? p.nblk * T.nw : 1, ninner = MULTI ? 1 : p.nblk;
             double sum[kOzMaxNB / 2];
+            int blk = 0, wi = 0;
             for (int ao = 0; ao < nouter && ok; ++ao, ++aseq) {
-                const int wi = MULTI ? ao % T.nw : 0;
                 for (int bi = 0; bi < ninner; ++bi, ++accseq) {
-                    const int blk = MULTI ? ao / T.nw : bi;
                     const int ab = (int)(accseq & 1);
-                    const int* ec = p.ecol + T.z * p.ecol_z + (long long)(T.w0 + wi) * p.nblk * p.NB + blk * p.NB + cb;
+                    const int col0 = blk * p.NB + cb;
+                    if (!MULTI) ++blk;
+                    if (!MULTI && ab != grp) continue;
+                    const int* ec = sEcol + (accseq % kOzRing) * kOzMaxNB + cb;
                     if (!oz_warp_wait(bar(ACCF + ab), (accseq >> 1) & 1, abort_flag, p.err, 41)) { ok = false; break; }
                     tc_fence_after();
-                    const int Ea = sExp[(aseq % kOzRing) * kOzBM + q * 32 + lane];
-                    const uint32_t col0 = lane_base + (uint32_t)(ab * 256 + cb);
+                    const int Ea = sExp[(aseq % kOzRing) * kOzBM + q * 32 + lane] - 1014;
+                    uint32_t tc[kOzLevels];
 #pragma unroll
-                    for (int c4 = 0; c4 < kOzMaxNB / 8; ++c4) {
-                        if (4 * c4 < half) {
-                            uint32_t v[kOzLevels][4];
+                    for (int l = 0; l < kOzLevels; ++l) tc[l] = lane_base + (uint32_t)(ab * 256 + cb + l * p.NB);
+#pragma unroll(MULTI ? kOzMaxNB / 8 : 1)
+                    for (int j = 0; j < (MULTI ? kOzMaxNB / 2 : half); j += 4) {  // four columns at a time
+                        if (MULTI && j >= half) continue;
+                        uint32_t v[kOzLevels][4];
 #pragma unroll
-                            for (int l = 0; l < kOzLevels; ++l) tmem_ld4(col0 + (uint32_t)(l * p.NB + 4 * c4), v[l]);
-                            const int4 e4 = *reinterpret_cast<const int4*>(ec + 4 * c4);
-                            const int Eb[4] = {e4.x, e4.y, e4.z, e4.w};
-                            tmem_wait_ld();
+                        for (int l = 0; l < kOzLevels; ++l) tmem_ld4(tc[l] + (uint32_t)j, v[l]);
+                        const int4 e4 = *reinterpret_cast<const int4*>(ec + j);
+                        const int Es[4] = {Ea + e4.x, Ea + e4.y, Ea + e4.z, Ea + e4.w};
+                        tmem_wait_ld();
+                        // four independent chains; the rare cases in a second pass
+                        uint32_t hi[4], lo[4], hmin = 0xffffffffu, emax = 0u;
+                        uint64_t r[4];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                int a[kOzLevels];
+                        for (int k = 0; k < 4; ++k) {
+                            float a[kOzLevels];
 #pragma unroll
-                                for (int l = 0; l < kOzLevels; ++l) a[l] = __float2int_rn(__uint_as_float(v[l][j]));
-                                const double r = __longlong_as_double((long long)oz_combine(a, Ea, Eb[j]));
-                                if (MULTI) {
-                                    sum[4 * c4 + j] = wi == 0 ? r : sum[4 * c4 + j] + r;
-                                } else {
-                                    const int col = blk * p.NB + cb + 4 * c4 + j;
-                                    const int cc = col >= p.map.Dy ? 1 : 0;
-                                    if (rok && col < p.Nc)
-                                        o[cc * p.map.SC + (long long)(col - cc * p.map.Dy) * p.map.SY] = r;
-                                }
+                            for (int l = 0; l < kOzLevels; ++l) a[l] = __uint_as_float(v[l][k]);
+                            uint32_t ha, e1;
+                            oz_sum(a, mul, hi[k], lo[k]);
+                            r[k] = oz_pack(hi[k], lo[k], Es[k], mul, ha, e1);
+                            hmin = min(hmin, ha);
+                            emax = max(emax, e1);
+                        }
+                        if (!oz_packed(hmin, emax)) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) r[k] = oz_pack_any(hi[k], lo[k], Es[k]);
+                        }
+                        if (MULTI) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const double d = __longlong_as_double((long long)r[k]);
+                                sum[j + k] = wi == 0 ? d : sum[j + k] + d;
                             }
+                        } else {
+                            const uint4 off = *reinterpret_cast<const uint4*>(sCol + col0 + j);
+                            const int ncol = rok ? p.Nc - (col0 + j) : 0;
+                            if (ncol > 0) o[off.x] = __longlong_as_double((long long)r[0]);
+                            if (ncol > 1) o[off.y] = __longlong_as_double((long long)r[1]);
+                            if (ncol > 2) o[off.z] = __longlong_as_double((long long)r[2]);
+                            if (ncol > 3) o[off.w] = __longlong_as_double((long long)r[3]);
                         }
                     }
                     tc_fence_before();
@@ -327,162 +435,211 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
                     if (lane == 0) mbar_arrive(bar(ACCE + ab));
                     if (MULTI && wi == T.nw - 1) {
 #pragma unroll
-                        for (int j = 0; j < kOzMaxNB / 2; ++j) {
-                            const int col = blk * p.NB + cb + j;
-                            const int cc = col >= p.map.Dy ? 1 : 0;
-                            if (j < half && rok && col < p.Nc)
-                                o[cc * p.map.SC + (long long)(col - cc * p.map.Dy) * p.map.SY] = sum[j];
-                        }
+                        for (int j = 0; j < kOzMaxNB / 2; ++j)
+                            if (j < half && rok && col0 + j < p.Nc) o[sCol[col0 + j]] = sum[j];
                     }
+                }
+                if (MULTI && ++wi == T.nw) {
+                    wi = 0;
+                    ++blk;
                 }
             }
         }
-    } else if (warp < kOzEpiWarps + kOzConvWarps) {
+    } else if (warp < kWorkers) {
         // ---------------- converter: FP64 rows of A -> digit planes ----------------
-        // A warp owns 16 rows as two groups of 8 (lane & 7).  The 2 no (group,
-        // chunk) tasks of a pass are dealt over the four lane groups s; windows
-        // of more than 8 chunks take one pass per row group.  The loads of the
-        // next pass are in flight while the warp waits for its stage.
-        const int cw = warp - kOzEpiWarps, r8 = lane & 7, s = lane >> 3;
-        uint64_t x[4][8];
-        // pass position
-        long long t = t0;
-        int ao = 0, pass = 0;
+        // A warp owns 16 rows as two groups of 8 (lane / 4).  Up to 6 chunks a
+        // window, the 2 no (group, chunk) tasks of both groups are dealt over
+        // the four lanes s of a row in one pass; longer windows take one pass per
+        // row group (at most three tasks a lane either way).  The loads of the
+        // next pass are in flight while the warp waits for its stage, and the
+        // lines of the tile (or windows) after it are on their way to L2.
+        constexpr bool kBoth = NO <= 6;
+        constexpr int NT = kBoth ? NO / 2 : (NO + 3) / 4, NPASS = kBoth ? 1 : 2;
+        if (!MULTI) regs_inc<104>();
+        const int cw = warp - kEpi, r8 = lane >> 2, s = lane & 3;
+        uint2 x[NT][8];  // (lo, hi), then digits
+        int t = 0, blk = 0, wi = 0, pass = 0;
         uint32_t aseq = 0;
+        OzPos P2 = T;  // the tile after the one being loaded
+        P2.next(p);
         auto load = [&]() {
-            const OzTile T(p, t);
-            const int w = T.w0 + (MULTI ? ao % T.nw : 0);
-            const long long k0 = (long long)w * p.kw;
-            const int Kw = (int)(p.K - k0 < p.kw ? p.K - k0 : p.kw);
-            const int no = 2 * ((Kw + 15) >> 4);
-            const int ntask = no <= 8 ? 2 * no : no;
-            const int row0 = T.mt * kOzBM + 16 * cw + r8;
+            const int w = T.w0 + wi;
+            const long long k0 = (long long)w * KW;
+            const int no = oz_chunks<NO, MULTI>(p, w);
+            const int Kw = MULTI ? (int)min((long long)KW, p.K - k0) : (int)p.K;
+            const int ntask = kBoth ? 2 * no : no;
+            const int row0 = T.mt * kOzBM + 16 * cw, rmax = p.M - 1 - row0;  // rmax < 0: past the end
             const double* a = p.A + T.z * p.sAz + (long long)row0 * p.lda + k0;
+            // rows, chunks and K past the end are clamped: their products meet
+            // zero digits of B or are not stored
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int c = s + 4 * i;
-                const int rg = no <= 8 ? (c >= no ? 1 : 0) : pass;
-                const int pc = no <= 8 ? c - rg * no : c;
-                const bool ok = c < ntask && row0 + 8 * rg < p.M;
-                const double* ar = a + (long long)(8 * rg) * p.lda;
+            for (int i = 0; i < NT; ++i) {
+                const int c = min(s + 4 * i, ntask - 1);
+                const int rg = kBoth ? (c >= no ? 1 : 0) : pass;
+                const int pc = kBoth ? c - rg * no : c;
+                const double* ar = a + (long long)min(8 * rg + r8, rmax) * p.lda;
+                if (VEC) {
+                    const int kp = Kw >> 1;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int k = pc + no * q;
-                    x[i][q] = ok && k < Kw ? (uint64_t)__double_as_longlong(__ldg(ar + k)) : 0ull;
+                    for (int q = 0; q < 4; ++q) {
+                        const int k = !MULTI && NO * q + NO - 1 <= 4 * NO - 8 ? pc + NO * q : min(pc + no * q, kp - 1);
+                        const uint4 u = __ldg(reinterpret_cast<const uint4*>(ar) + k);
+                        x[i][2 * q] = make_uint2(u.x, u.y);
+                        x[i][2 * q + 1] = make_uint2(u.z, u.w);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int k = !MULTI && NO * q + NO - 1 <= 8 * NO - 16 ? pc + NO * q : min(pc + no * q, Kw - 1);
+                        x[i][q] = __ldg(reinterpret_cast<const uint2*>(ar) + k);
+                    }
                 }
             }
+            if (MULTI) {
+                // this warp's rows of the window after the next
+                if (pass == 0 && wi + 2 < T.nw) {
+                    const int rr = T.mt * kOzBM + 16 * cw + (lane & 15);
+                    const char* b = (const char*)(p.A + T.z * p.sAz + (long long)rr * p.lda + k0 + 2 * KW);
+                    if (rr < p.M && k0 + 3 * KW <= p.K)
+                        for (int o = (lane >> 4) * 128; o < KW * 8; o += 256)
+                            asm volatile("prefetch.global.L2 [%0];" ::"l"(b + o));
+                }
+            } else if (pass == 0 && t + 1 < ntile && P2.mt * kOzBM + 16 * cw + 16 <= p.M) {
+                // this warp's rows of the next tile (contiguous up to the row stride)
+                const char* b = (const char*)(p.A + P2.z * p.sAz + (long long)(P2.mt * kOzBM + 16 * cw) * p.lda);
+                const int bytes = 16 * (int)p.lda * 8;
+                for (int o = lane * 128; o < bytes; o += 32 * 128)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(b + o));
+            }
         };
-        bool ok = true;
-        if (t < t1) load();
-        while (t < t1 && ok) {
-            const OzTile T(p, t);
-            const int w = T.w0 + (MULTI ? ao % T.nw : 0);
-            const long long k0 = (long long)w * p.kw;
-            const int Kw = (int)(p.K - k0 < p.kw ? p.K - k0 : p.kw);
-            const int no = 2 * ((Kw + 15) >> 4);
-            const bool two = no <= 8;  // both row groups in one pass
-            const int ntask = two ? 2 * no : no;
-            const int npass = two ? 1 : 2;
+        if (ntile > 0) load();
+        while (t < ntile) {
+            const int no = oz_chunks<NO, MULTI>(p, T.w0 + wi);
+            const int ntask = kBoth ? 2 * no : no;
             // row exponents
-            int E0 = 1, E1 = 1;
+            uint32_t E0 = kOzExpMin, E1 = kOzExpMin;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int e = 1;
+            for (int i = 0; i < NT; ++i) {
+                uint32_t e = kOzExpMin;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) e = max(e, oz_exponent((uint32_t)(x[i][q] >> 32)));
-                const bool g1 = two ? s + 4 * i >= no : pass != 0;
-                if (g1) E1 = max(E1, e);
+                for (int q = 0; q < 8; ++q) e = max(e, x[i][q].y & kOzExpMask);
+                if (kBoth && s + 4 * i >= no) E1 = max(E1, e);
                 else E0 = max(E0, e);
             }
 #pragma unroll
-            for (int d = 8; d < 32; d <<= 1) {
+            for (int d = 1; d < 4; d <<= 1) {
                 E0 = max(E0, __shfl_xor_sync(0xffffffffu, E0, d));
-                E1 = max(E1, __shfl_xor_sync(0xffffffffu, E1, d));
+                if (kBoth) E1 = max(E1, __shfl_xor_sync(0xffffffffu, E1, d));
             }
-            int* se = sExp + (aseq % kOzRing) * kOzBM + 16 * cw + r8;
             if (s == 0) {
-                if (two || pass == 0) se[0] = E0;
-                if (two || pass == 1) se[8] = E1;
+                int* se = sExp + (aseq % kOzRing) * kOzBM + 16 * cw + r8;
+                se[kBoth ? 0 : 8 * pass] = oz_exponent(E0);
+                if (kBoth) se[8] = oz_exponent(E1);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const bool g1 = two ? s + 4 * i >= no : pass != 0;
-                const int E = g1 ? E1 : E0;
+            for (int i = 0; i < NT; ++i) {
+                const uint32_t E = kBoth && s + 4 * i >= no ? E1 : E0;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) x[i][q] = oz_digits(x[i][q], E);
+                for (int q = 0; q < 8; ++q) {
+                    const uint64_t d = oz_digits(x[i][q].y, x[i][q].x, E);
+                    x[i][q] = make_uint2((uint32_t)d, (uint32_t)(d >> 32));
+                }
             }
-            const int as = (int)(aseq % (uint32_t)p.na);
-            if (pass == 0 &&
-                !oz_warp_wait(bar(AEMPTY + as), ((aseq / (uint32_t)p.na) & 1) ^ 1, abort_flag, p.err, 42)) {
-                ok = false;
-                break;
-            }
-            uint8_t* ap = sA + (size_t)as * kOzSlices * plane;
+            const int as = p.na == 2 ? (int)(aseq & 1) : 0;
+            const uint32_t aph = (p.na == 2 ? aseq >> 1 : aseq) & 1;
+            if (pass == 0 && !oz_warp_wait(bar(AEMPTY + as), aph ^ 1, abort_flag, p.err, 42)) break;
+            uint8_t* ap = sA + (size_t)as * kAStage + 2 * cw * 128 + r8 * 16;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < NT; ++i) {
                 const int c = s + 4 * i;
                 if (c < ntask) {
-                    const int rg = two ? (c >= no ? 1 : 0) : pass;
-                    const int pc = two ? c - rg * no : c;
-                    uint8_t* o = ap + pc * (kOzBM * 16) + (2 * cw + rg) * 128 + r8 * 16;
+                    const int rg = kBoth ? (c >= no ? 1 : 0) : pass;
+                    const int pc = kBoth ? c - rg * no : c;
+                    uint8_t* o = ap + pc * kOzLbo + rg * 128;
+// the same byte of two elements side by side, two digits at a
+                    // time, then each digit as FP16 1024 + byte, minus 1152
 #pragma unroll
-                    for (int d = 0; d < kOzSlices; ++d) {
-                        // byte 7 - d of each element -> 1024 + byte as FP16, minus 1152
-                        const int byte = 7 - d;
-                        const uint32_t sel = (uint32_t)((byte & 3) | ((4 + (byte & 3)) << 8));
-                        uint32_t v[4];
+                    for (int w2 = 0; w2 < 4; ++w2) {  // bytes (7,6) (5,4) (3,2) (1,-)
+                        uint32_t v[2][4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const uint32_t a0 = byte >= 4 ? (uint32_t)(x[i][2 * q] >> 32) : (uint32_t)x[i][2 * q];
-                            const uint32_t a1 =
-                                byte >= 4 ? (uint32_t)(x[i][2 * q + 1] >> 32) : (uint32_t)x[i][2 * q + 1];
-                            const uint32_t b = (__byte_perm(a0, a1, sel) & 0x00FF00FFu) | 0x64006400u;
-                            const __half2 hd = __hsub2(*reinterpret_cast<const __half2*>(&b),
-                                                       __half2half2(__ushort_as_half(0x6480)));
-                            v[q] = *reinterpret_cast<const uint32_t*>(&hd);
+                            const uint32_t a0 = w2 < 2 ? x[i][2 * q].y : x[i][2 * q].x;
+                            const uint32_t a1 = w2 < 2 ? x[i][2 * q + 1].y : x[i][2 * q + 1].x;
+                            const uint32_t pr = __byte_perm(a0, a1, (w2 & 1) ? 0x4051 : 0x6273);
+                            v[0][q] = __byte_perm(pr, 0x64646464u, 0x4140);
+                            v[1][q] = __byte_perm(pr, 0x64646464u, 0x4342);
                         }
-                        *reinterpret_cast<uint4*>(o + (size_t)d * plane) = make_uint4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            if (2 * w2 + k >= kOzSlices) continue;
+                            uint32_t d[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const __half2 hd = __hsub2(*reinterpret_cast<const __half2*>(&v[k][q]),
+                                                           __half2half2(__ushort_as_half(0x6480)));
+                                d[q] = *reinterpret_cast<const uint32_t*>(&hd);
+                            }
+                            *reinterpret_cast<uint4*>(o + (2 * w2 + k) * kPlane) = make_uint4(d[0], d[1], d[2], d[3]);
+                        }
                     }
                 }
             }
             // next pass
-            if (pass == npass - 1) {
+            if (pass == NPASS - 1) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(AFULL + as));
                 ++aseq;
                 pass = 0;
-                if (++ao == (MULTI ? p.nblk * T.nw : 1)) {
-                    ao = 0;
+                bool done = true;  // all windows and blocks of the tile
+                if (MULTI) {
+                    if (++wi == T.nw) {
+                        wi = 0;
+                        ++blk;
+                    }
+                    done = blk == p.nblk;
+                }
+                if (done) {
+                    blk = 0;
                     ++t;
+                    T.next(p);
+                    P2.next(p);
                 }
             } else {
                 ++pass;
             }
-            if (t < t1) load();
+            if (t < ntile) load();
         }
-    } else if (warp == 16) {
+    } else if (warp == kWorkers) {
+        if (!MULTI) regs_dec<40>();
         if (lane == 0) {
             // ---------------- producer of B's digit images ----------------
-            uint32_t bseq = 0;
+            uint32_t bseq = 0, accseq = 0;
             bool ok = true;
-            for (long long t = t0; t < t1 && ok; ++t) {
-                const OzTile T(p, t);
+            for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
                 const int nacc = MULTI ? p.nblk * T.nw : p.nblk;
-                for (int a = 0; a < nacc && ok; ++a) {
-                    const int blk = MULTI ? a / T.nw : a, w = T.w0 + (MULTI ? a % T.nw : 0);
-                    const long long k0 = (long long)w * p.kw;
-                    const int no = 2 * (int)(((p.K - k0 < p.kw ? p.K - k0 : p.kw) + 15) >> 4);
-                    const uint8_t* src = p.img + T.z * p.img_z + ((long long)w * p.nblk + blk) * no_full * brow;
+                int blk = 0, wi = 0;
+                for (int a = 0; a < nacc && ok; ++a, ++accseq) {
+                    const int w = T.w0 + wi;
+                    const int no = oz_chunks<NO, MULTI>(p, w);
+                    const uint8_t* src = p.img + T.z * p.img_z + ((long long)w * p.nblk + blk) * NO * brow;
                     for (int c0 = 0; c0 < no; c0 += kOzSub, ++bseq) {
                         const int st = (int)(bseq % (uint32_t)p.nbs);
-                        if (!oz_wait(bar(BEMPTY + st), ((bseq / (uint32_t)p.nbs) & 1) ^ 1, abort_flag, p.err, 43)) {
+                        if (!oz_wait(bar(BEMPTY + st), ((bseq / (uint32_t)p.nbs) & 1) ^ 1, abort_flag, p.err, 43, 300)) {
                             ok = false;
                             break;
                         }
                         const uint32_t bytes = (uint32_t)min(kOzSub, no - c0) * brow;
-                        mbar_expect_tx(bar(BFULL + st), bytes);
+                        mbar_expect_tx(bar(BFULL + st), bytes + (c0 == 0 ? p.NB * 4u : 0u));
+                        if (c0 == 0)
+                            bulk_load(smem_u32(sEcol + (accseq % kOzRing) * kOzMaxNB),
+                                      p.ecol + T.z * p.ecol_z + ((long long)w * p.nblk + blk) * p.NB, p.NB * 4u,
+                                      bar(BFULL + st));
                         bulk_load(smem_u32(sB + (size_t)st * bstage), src + (size_t)c0 * brow, bytes, bar(BFULL + st));
+                    }
+                    if (!MULTI || ++wi == T.nw) {
+                        wi = 0;
+                        ++blk;
                     }
                 }
             }
@@ -497,21 +654,23 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
                 }
             }
         }
+    } else if (!MULTI && warp > kWorkers + 1) {
+        regs_dec<40>();
     } else {
         // ---------------- MMA issuer ----------------
+        if (!MULTI) regs_dec<40>();
         uint32_t aseq = 0, bseq = 0, accseq = 0;
-        const uint32_t lboB = brow;
         bool ok = true;
-        for (long long t = t0; t < t1 && ok; ++t) {
-            const OzTile T(p, t);
+        for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
             const int nouter = MULTI ? p.nblk * T.nw : 1, ninner = MULTI ? 1 : p.nblk;
+            int wi = 0;
             for (int ao = 0; ao < nouter && ok; ++ao, ++aseq) {
-                const int w = T.w0 + (MULTI ? ao % T.nw : 0);
-                const long long k0 = (long long)w * p.kw;
-                const int no = 2 * (int)(((p.K - k0 < p.kw ? p.K - k0 : p.kw) + 15) >> 4);
-                const int as = (int)(aseq % (uint32_t)p.na);
-                if (!oz_warp_wait(bar(AFULL + as), (aseq / (uint32_t)p.na) & 1, abort_flag, p.err, 44)) { ok = false; break; }
-                const unsigned long long ad = desc_plain(smem_u32(sA + (size_t)as * kOzSlices * plane), kOzBM * 16);
+                const int no = oz_chunks<NO, MULTI>(p, T.w0 + wi);
+                if (MULTI && ++wi == T.nw) wi = 0;
+                const int as = p.na == 2 ? (int)(aseq & 1) : 0;
+                const uint32_t aph = (p.na == 2 ? aseq >> 1 : aseq) & 1;
+                if (!oz_warp_wait(bar(AFULL + as), aph, abort_flag, p.err, 44)) { ok = false; break; }
+                const unsigned long long ad = desc_plain(smem_u32(sA + (size_t)as * kAStage), kOzLbo);
                 for (int bi = 0; bi < ninner && ok; ++bi, ++accseq) {
                     const int ab = (int)(accseq & 1);
                     if (!oz_warp_wait(bar(ACCE + ab), ((accseq >> 1) & 1) ^ 1, abort_flag, p.err, 45)) { ok = false; break; }
@@ -520,7 +679,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
                         const int st = (int)(bseq % (uint32_t)p.nbs);
                         if (!oz_warp_wait(bar(BFULL + st), (bseq / (uint32_t)p.nbs) & 1, abort_flag, p.err, 46)) { ok = false; break; }
                         tc_fence_after();
-                        const unsigned long long bd = desc_plain(smem_u32(sB + (size_t)st * bstage), lboB);
+                        const unsigned long long bd = desc_plain(smem_u32(sB + (size_t)st * bstage), brow);
                         const int ns = min(kOzSub, no - c0) / 2;
 #pragma unroll
                         for (int i = 0; i < kOzSlices; ++i) {
@@ -531,7 +690,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
                             const uint32_t id = (1u << 4) | ((n >> 3) << 17) | ((uint32_t)(kOzBM >> 4) << 24);
                             for (int ks = 0; ks < ns; ++ks)
                                 oz_mma(acc + (uint32_t)(i * p.NB),
-                                       ad + (((unsigned long long)i * plane + (unsigned long long)(c0 + 2 * ks) * (kOzBM * 16)) >> 4),
+                                       ad + (((unsigned long long)i * kPlane + (unsigned long long)(c0 + 2 * ks) * kOzLbo) >> 4),
                                        bd + (((unsigned long long)(2 * ks) * brow) >> 4), id, (c0 | i | ks) ? 1u : 0u);
                         }
                         oz_commit(bar(BEMPTY + st));
@@ -550,15 +709,33 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const __grid_constant
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 17) {
+    if (warp == kWorkers + 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
 }
 
+using OzKernel = void (*)(const OzParams);
+// The kernel of a window of kw K (16 .. 96).
+template <bool MULTI, bool VEC>
+OzKernel oz_kernel(int kw) {
+    switch (kw / 16) {
+        case 1: return k_oz_gemm<2, MULTI, VEC>;
+        case 2: return k_oz_gemm<4, MULTI, VEC>;
+        case 3: return k_oz_gemm<6, MULTI, VEC>;
+        case 4: return k_oz_gemm<8, MULTI, VEC>;
+        case 5: return k_oz_gemm<10, MULTI, VEC>;
+        default: return k_oz_gemm<12, MULTI, VEC>;
+    }
+}
+OzKernel oz_kernel(int kw, bool multi, bool vec) {
+    if (multi) return vec ? oz_kernel<true, true>(kw) : oz_kernel<true, false>(kw);
+    return vec ? oz_kernel<false, true>(kw) : oz_kernel<false, false>(kw);
+}
+
 // A stages (1 or 2) and B stages (2 to 4) that fit the shared memory.
 void oz_stages(const OzGeom& g, int* na, int* nbs, size_t* smem) {
-    const size_t a = (size_t)kOzSlices * kOzBM * g.kw * 2;
+    const size_t a = (size_t)kOzSlices * (g.kw / 8) * kOzLbo;
     const size_t b = (size_t)std::min(kOzSub, g.kw / 8) * 8 * g.NB * 16;
     *na = 2 * a + 2 * b + kOzMisc + 128 <= kOzSmemMax ? 2 : 1;
     int n = 2;
@@ -575,8 +752,11 @@ size_t oz_img_bytes(int Nc, long long K) {
 }
 
 gkba_status oz_prepare(gkba_ctx* c) {
-    GKBA_CUDA(c, cudaFuncSetAttribute(k_oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmemMax));
-    GKBA_CUDA(c, cudaFuncSetAttribute(k_oz_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmemMax));
+    for (int kw = 16; kw <= kOzMaxKw; kw += 16)
+        for (int m = 0; m < 4; ++m)
+            GKBA_CUDA(c, cudaFuncSetAttribute(oz_kernel(kw, (m & 1) != 0, (m & 2) != 0),
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)kOzSmemMax));
     return GKBA_OK;
 }
 
@@ -606,6 +786,13 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
                     int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
                     long long sOitem, StageMap map, double flops, double bytes) {
     const OzGeom g = oz_geom(Nc, K);
+    if (Nc > kOzMaxCols) return fail(c, GKBA_EINVAL, "oz_gemm: %d columns", Nc);
+    // 16-byte loads of A (the digit images have the matching order, by K's parity)
+    const bool vec = (K & 1) == 0;
+    if (vec && ((lda & 1) || (sAz & 1) || ((uintptr_t)A & 15)))
+        return fail(c, GKBA_EINVAL, "oz_gemm: rows of even K must be 16-byte aligned");
+    if ((unsigned long long)(Nc / map.Dy) * map.SC + (unsigned long long)map.Dy * map.SY >= 1ull << 32)
+        return fail(c, GKBA_EINVAL, "oz_gemm: column offsets past 32 bits");
     OzParams p{};
     p.A = A;
     p.lda = lda;
@@ -621,7 +808,6 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
     p.Nc = Nc;
     p.NB = g.NB;
     p.nblk = g.nblk;
-    p.kw = g.kw;
     p.nwin = g.nwin;
     p.K = K;
     p.mtiles = (M + kOzBM - 1) / kOzBM;
@@ -629,14 +815,15 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
     p.nitem = (g.nwin + p.wper - 1) / p.wper;
     if (p.nitem != nitem) return fail(c, GKBA_EINVAL, "oz_gemm: %d items for %d windows", nitem, g.nwin);
     p.sOitem = sOitem;
+    p.mul = kOzMul;
     p.tiles = (long long)nz * p.nitem * p.mtiles;
+    if (p.tiles >= 1LL << 31) return fail(c, GKBA_EINVAL, "oz_gemm: %lld tiles", p.tiles);
     p.err = c->dint + 1;
     size_t smem = 0;
     oz_stages(g, &p.na, &p.nbs, &smem);
     const unsigned grid = (unsigned)std::min<long long>(p.tiles, c->num_sms);
     auto t = launch_begin(c, cls, flops, bytes);
-    if (g.nwin == 1) k_oz_gemm<false><<<grid, kOzThreads, smem, c->stream>>>(p);
-    else k_oz_gemm<true><<<grid, kOzThreads, smem, c->stream>>>(p);
+    oz_kernel(g.kw, g.nwin > 1, vec)<<<grid, oz_threads(g.nwin > 1), smem, c->stream>>>(p);
     return launch_end(c, t);
 }
 
