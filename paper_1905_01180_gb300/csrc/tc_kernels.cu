@@ -102,6 +102,10 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
+// Bytes to the next 1024-byte boundary.  Aligning by an offset keeps the pointer
+// in the shared address space; a cast to an integer and back made every access
+// through it a generic one.
+__device__ __forceinline__ uint32_t smem_pad1024(const void* p) { return (0u - smem_u32(p)) & 1023u; }
 // Bounded wait of the CTA-pair kernel; on timeout it raises this CTA's and the
 // peer CTA's abort flags (peer_abort: shared::cluster address).
 __device__ bool mbar_wait_cl(uint32_t bar, uint32_t parity, volatile int* abort_flag,
@@ -397,7 +401,7 @@ template <bool SPLIT_ACC, bool GROUPED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
     k_tc_pair(const __grid_constant__ StageLaunch L) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = smem_raw + smem_pad1024(smem_raw);
     // the group this cluster works on: the launch's clusters are split between
     // its groups (problems of different Np or operands), each runs the
     // pipeline below with its own parameters and tensor maps
@@ -1019,7 +1023,7 @@ template <bool GROUPED, bool PACKED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFinThreads, 1)
     k_tc_final_pair(const __grid_constant__ FinalLaunch L) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = smem_raw + smem_pad1024(smem_raw);
     // the group this cluster works on (see StageLaunch)
     const int cid_all = (int)cluster_id_x();
     int grp = 0;
