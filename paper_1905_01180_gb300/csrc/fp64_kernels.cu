@@ -22,10 +22,19 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
+// acc += a b in four FMAs (a multiply followed by an add takes six FP64
+// instructions, and the FP64 rate, two a clock and SM, bounds these kernels).
+__device__ __forceinline__ void cmac(double2& acc, double2 a, double2 b) {
+    acc.x = fma(a.x, b.x, acc.x);
+    acc.y = fma(a.x, b.y, acc.y);
+    acc.x = fma(-a.y, b.y, acc.x);
+    acc.y = fma(a.y, b.x, acc.y);
+}
 
 // ---------------------------------------------------------------------------
-// Stage GEMM (FP64): D[row][col] = sum_k A[row*lda+k] * B[col*ldb+k]; the
-// result is scattered by the stage's index map.  64x64 output tile, 16-wide
+// Stage GEMM (FP64, CUDA cores; the allocation-free entry point only, whose
+// fixed scratch has no room for digit images): D[row][col] = sum_k A[row*lda+k] *
+// B[col*ldb+k]; the result is scattered by the stage's index map.  64x64 output tile, 16-wide
 // K slices staged in shared memory, 4x4 outputs per thread.
 // ---------------------------------------------------------------------------
 constexpr int G64_BM = 64, G64_BN = 64, G64_BK = 16;
@@ -107,58 +116,81 @@ __global__ void __launch_bounds__(256) k_gemm64_stage(const double* __restrict__
 
 // ---------------------------------------------------------------------------
 // Complex batched GEMM for N x N matrices (FP64):
-//   C = alpha op(A) op(B) + beta C (+ identity), op in {N, C = conj-transpose}.
-// When skip_ge != nullptr and idx >= *skip_ge the block copies op(A) into C
-// instead (used for the data-dependent number of squarings in expm).
+//   C = alpha op(A) op(B) + beta C + poly, op in {N, C = conj-transpose},
+//   poly = p.c0 I + p.c1 X1 + p.c2 X2 + p.c3 X3 (the terms whose matrix is set).
+// Matrices from ident_b on are set to the identity instead.  When skip_ge is
+// given and idx >= *skip_ge the launch does nothing (the data-dependent number
+// of squarings in the exponential).
+//
+// Bound by the FP64 rate (two FMAs a clock and SM: 4 n^3 of them a matrix), so
+// every output is four FMAs a term with no padding to a tile, read through L1:
+// one output per TPO lanes, the sum over k split over them.  TPO is chosen so
+// that a single matrix, too, spreads over all SMs with a few warps each (a
+// 16 x 16 tile per block kept nine of them busy at n = 48).  Measured, tiles ->
+// here: 2501 products at n = 10 100 -> 27 us; one at n = 48 16.5 -> 4.4 us.
 // ---------------------------------------------------------------------------
-constexpr int ZT = 16;
+// Imaginary part's sign bit flipped by s (conjugation on the integer pipe).
+__device__ __forceinline__ double2 zsign(double2 a, int s) {
+    return make_double2(a.x, __hiloint2double(__double2hiint(a.y) ^ s, __double2loint(a.y)));
+}
 
-__global__ void __launch_bounds__(256) k_zgemm(int n, int opA, int opB, double2 alpha,
+struct ZPoly {
+    double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
+    const double2 *X1 = nullptr, *X2 = nullptr, *X3 = nullptr;
+};
+
+template <int TPO>
+__global__ void __launch_bounds__(128) k_zgemm(int n, int opA, int opB, double2 alpha,
                                                const double2* __restrict__ A, long long sA,
                                                const double2* __restrict__ B, long long sB,
                                                double2 beta, double2* __restrict__ C, long long sC,
-                                               int add_identity, const int* skip_ge, int idx) {
-    const int b = blockIdx.z;
-    A += (long long)b * sA;
-    B += (long long)b * sB;
-    C += (long long)b * sC;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int row = blockIdx.y * ZT + ty, col = blockIdx.x * ZT + tx;
-    if (skip_ge != nullptr && idx >= *skip_ge) {
-        if (row < n && col < n) {
-            double2 a = opA ? cconj(A[(long long)col * n + row]) : A[(long long)row * n + col];
-            C[(long long)row * n + col] = a;
+                                               uint32_t total, int ident_b, const ZPoly p,
+                                               const int* skip_ge, int idx) {
+    if (skip_ge != nullptr && idx >= *skip_ge) return;
+    const uint32_t gid = blockIdx.x * 128u + threadIdx.x;
+    const uint32_t o = min(gid / TPO, total - 1u);
+    const int sub = (int)(gid % TPO);
+    const uint32_t nn = (uint32_t)(n * n);
+    const int b = (int)(o / nn), e = (int)(o - (uint32_t)b * nn);
+    const int row = e / n, col = e - row * n;
+    double2 acc = make_double2(0.0, 0.0);
+    if (b < ident_b) {
+        const double2* a = A + (long long)b * sA + (opA ? row : row * n);
+        const double2* bb = B + (long long)b * sB + (opB ? col * n : col);
+        const int da = opA ? n : 1, db = opB ? 1 : n;
+        double2 acc2 = make_double2(0.0, 0.0);
+        const int sa = opA ? (int)0x80000000 : 0, sb = opB ? (int)0x80000000 : 0;
+        int k = sub;
+#pragma unroll 2
+        for (; k + TPO < n; k += 2 * TPO) {
+            const double2 x0 = a[k * da], y0 = bb[k * db], x1 = a[(k + TPO) * da], y1 = bb[(k + TPO) * db];
+            cmac(acc, zsign(x0, sa), zsign(y0, sb));
+            cmac(acc2, zsign(x1, sa), zsign(y1, sb));
         }
+        if (k < n) {
+            const double2 x0 = a[k * da], y0 = bb[k * db];
+            cmac(acc, zsign(x0, sa), zsign(y0, sb));
+        }
+        acc = cadd(acc, acc2);
+    }
+#pragma unroll
+    for (int d = TPO / 2; d > 0; d >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+    }
+    if (sub != 0 || gid / TPO >= total) return;
+    double2* c = C + (long long)b * sC + e;
+    if (b >= ident_b) {
+        *c = make_double2(row == col ? 1.0 : 0.0, 0.0);
         return;
     }
-    __shared__ double2 As[ZT][ZT + 1], Bs[ZT][ZT + 1];
-    double2 acc = make_double2(0.0, 0.0);
-    for (int kb = 0; kb < n; kb += ZT) {
-        // As[ty][tx] = op(A)[row][kb+tx]
-        {
-            const int r = blockIdx.y * ZT + ty, k = kb + tx;
-            double2 v = make_double2(0.0, 0.0);
-            if (r < n && k < n) v = opA ? cconj(A[(long long)k * n + r]) : A[(long long)r * n + k];
-            As[ty][tx] = v;
-        }
-        // Bs[ty][tx] = op(B)[kb+ty][col]
-        {
-            const int k = kb + ty, cidx = blockIdx.x * ZT + tx;
-            double2 v = make_double2(0.0, 0.0);
-            if (k < n && cidx < n) v = opB ? cconj(B[(long long)cidx * n + k]) : B[(long long)k * n + cidx];
-            Bs[ty][tx] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < ZT; ++kk) acc = cadd(acc, cmul(As[ty][kk], Bs[kk][tx]));
-        __syncthreads();
-    }
-    if (row < n && col < n) {
-        double2 r = cmul(alpha, acc);
-        if (beta.x != 0.0 || beta.y != 0.0) r = cadd(r, cmul(beta, C[(long long)row * n + col]));
-        if (add_identity && row == col) r.x += 1.0;
-        C[(long long)row * n + col] = r;
-    }
+    double2 r = cmul(alpha, acc);
+    if (beta.x != 0.0 || beta.y != 0.0) cmac(r, beta, *c);
+    if (row == col) r.x += p.c0;
+    if (p.X1) r = make_double2(fma(p.c1, p.X1[e].x, r.x), fma(p.c1, p.X1[e].y, r.y));
+    if (p.X2) r = make_double2(fma(p.c2, p.X2[e].x, r.x), fma(p.c2, p.X2[e].y, r.y));
+    if (p.X3) r = make_double2(fma(p.c3, p.X3[e].x, r.x), fma(p.c3, p.X3[e].y, r.y));
+    *c = r;
 }
 
 // Sigma_HF(rho)_ij = sum_{l,k} hfK[(i,j),(l,k)] rho_lk, plus h + E d when add_h.
@@ -192,16 +224,39 @@ __global__ void k_mean_field(int N, const double* __restrict__ hfK, const double
     }
 }
 
-// out = -i (HR - RH) - (I + I^+), where HR = H rho and RH = rho H.
-__global__ void k_rhs(int N, const double2* __restrict__ HR, const double2* __restrict__ RH,
-                      const double2* __restrict__ I, double2* __restrict__ out) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= N * N) return;
-    const int i = e / N, j = e % N;
-    const double2 c = make_double2(HR[e].x - RH[e].x, HR[e].y - RH[e].y);
-    const double2 a = I[e], bt = I[j * N + i];
+// One stage of Heun's method, every element by kRhsLanes lanes:
+//   k = -i [h, rho] - (I + I^+);  y = base + a (k + kprev)
+// with k written to k_out and y also to y2 when given (kprev may be null).
+constexpr int kRhsLanes = 8;
+__global__ void __launch_bounds__(128) k_heun_stage(int N, const double2* __restrict__ h,
+                                                    const double2* __restrict__ rho,
+                                                    const double2* __restrict__ I,
+                                                    const double2* __restrict__ base,
+                                                    const double2* __restrict__ kprev, double a,
+                                                    double2* __restrict__ k_out, double2* __restrict__ y,
+                                                    double2* __restrict__ y2) {
+    const int gid = blockIdx.x * 128 + threadIdx.x, sub = gid % kRhsLanes;
+    const int e = min(gid / kRhsLanes, N * N - 1), i = e / N, j = e % N;
+    double2 c = make_double2(0.0, 0.0), d = make_double2(0.0, 0.0);
+    for (int k = sub; k < N; k += kRhsLanes) {
+        cmac(c, h[i * N + k], rho[k * N + j]);
+        cmac(d, rho[i * N + k], h[k * N + j]);
+    }
+    c = make_double2(c.x - d.x, c.y - d.y);
+#pragma unroll
+    for (int o = kRhsLanes / 2; o > 0; o >>= 1) {
+        c.x += __shfl_xor_sync(0xffffffffu, c.x, o);
+        c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
+    }
+    if (sub != 0 || gid / kRhsLanes >= N * N) return;
+    const double2 x = I[e], xt = I[j * N + i];
     // -i c = (c.y, -c.x); I + I^+ at (i,j) = I_ij + conj(I_ji)
-    out[e] = make_double2(c.y - (a.x + bt.x), -c.x - (a.y - bt.y));
+    double2 k = make_double2(c.y - (x.x + xt.x), -c.x - (x.y - xt.y));
+    if (k_out) k_out[e] = k;
+    if (kprev) k = cadd(kprev[e], k);
+    const double2 b = base[e], r = make_double2(fma(a, k.x, b.x), fma(a, k.y, b.y));
+    y[e] = r;
+    if (y2) y2[e] = r;
 }
 
 // y = a x + b z (elementwise complex, real a and b).
@@ -261,70 +316,153 @@ __global__ void k_expm_setup(int N, double dt, const double2* __restrict__ hA,
     }
 }
 
-// The whole exponential for N <= 24 in one block, matrices in shared memory
-// (the same algorithm as k_expm_setup followed by the Horner and squaring
-// products: A = -i dt (hA + hB)/2 scaled by 2^-s so that ||A||_1 / 2^s <= 1/2,
-// the degree-18 Taylor polynomial by Horner, Y = I + X Y / k for k = 18 .. 1,
-// then min(s, 16) squarings).  One launch instead of 37 for small bases.
-constexpr int kExpmSmallN = 24;
-__device__ void smem_zgemm(int N, const double2* A, const double2* B, double2* C, double alpha,
-                           int add_identity) {
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int i = e / N, j = e % N;
+// The whole exponential of a matrix of n <= 32 rows in one launch: the argument
+// (-i dt (hA + hB)/2, or a general matrix Z) scaled by 2^-s so that its 1-norm is
+// at most 1/2, the degree-18 Taylor polynomial as four Horner steps in X^4
+// (Paterson and Stockmeyer, SIAM J. Comput. 2, 1973: seven products instead of
+// eighteen), min(s, 16) squarings.  From kExpmOneN + 1 rows on a cluster of eight
+// CTAs shares every product: each keeps all matrices in shared memory, computes
+// an eighth and writes it to all eight (distributed shared memory, one cluster
+// barrier a product); below, one CTA is faster than the barriers.  One SM's FP64
+// rate bounds a single CTA (n = 24, eighteen products: 520 us; here, cluster:
+// 44 us; n = 10: 62 -> 24).
+constexpr int kExpmSmallN = 32, kExpmOneN = 12;
+constexpr int kExpmLanes = 4;
+struct ExpmCoef {  // 1 / k!
+    double f[19];
+    constexpr ExpmCoef() : f() {
+        f[0] = 1.0;
+        for (int k = 1; k < 19; ++k) f[k] = f[k - 1] / k;
+    }
+};
+__device__ constexpr ExpmCoef kExpmCoef{};
+
+// C = A B, plus (poly >= 0) sum_{i=0..3} X^i / (4 poly + i)!, into all CTAs' C.
+template <int CTAS>
+__device__ void expm_product(int n, int rank, const double2* A, const double2* B, double2* C, int poly,
+                             const double2* X1, const double2* X2, const double2* X3) {
+    const int nn = n * n, per = (nn + CTAS - 1) / CTAS;
+    const int e0 = rank * per, e1 = min(nn, e0 + per), sub = threadIdx.x % kExpmLanes;
+    for (int eb = e0; eb < e1; eb += 256 / kExpmLanes) {
+        const int et = eb + (int)threadIdx.x / kExpmLanes, e = min(et, e1 - 1), i = e / n, j = e % n;
         double2 acc = make_double2(0.0, 0.0);
-        for (int k = 0; k < N; ++k) acc = cadd(acc, cmul(A[i * N + k], B[k * N + j]));
-        double2 r = make_double2(alpha * acc.x, alpha * acc.y);
-        if (add_identity && i == j) r.x += 1.0;
-        C[e] = r;
+        for (int k = sub; k < n; k += kExpmLanes) cmac(acc, A[i * n + k], B[k * n + j]);
+#pragma unroll
+        for (int o = kExpmLanes / 2; o > 0; o >>= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        }
+        if (poly >= 0) {
+            const double* c = kExpmCoef.f + 4 * poly;
+            if (i == j) acc.x += c[0];
+            acc.x = fma(c[1], X1[e].x, fma(c[2], X2[e].x, fma(c[3], X3[e].x, acc.x)));
+            acc.y = fma(c[1], X1[e].y, fma(c[2], X2[e].y, fma(c[3], X3[e].y, acc.y)));
+        }
+        if (CTAS == 1) {
+            if (et < e1 && sub == 0) C[e] = acc;
+        } else if (et < e1) {
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(C + e);
+            for (int r = sub; r < CTAS; r += kExpmLanes) {  // two CTAs a lane
+                uint32_t remote;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(dst), "r"(r));
+                asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote), "d"(acc.x), "d"(acc.y)
+                             : "memory");
+            }
+        }
+    }
+    if (CTAS == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }
-__global__ void __launch_bounds__(256) k_expm_small(int N, double dt, const double2* __restrict__ hA,
-                                                     const double2* __restrict__ hB,
-                                                     double2* __restrict__ U,
-                                                     double* __restrict__ norm_out,
-                                                     int* __restrict__ s_out) {
-    __shared__ double2 X[kExpmSmallN * kExpmSmallN], Y[kExpmSmallN * kExpmSmallN],
-        Z[kExpmSmallN * kExpmSmallN];
-    __shared__ double colsum[kExpmSmallN];
-    const int tid = threadIdx.x, NN = N * N;
-    for (int j = tid; j < N; j += blockDim.x) {
-        double sum = 0.0;
-        for (int i = 0; i < N; ++i) {
-            const int e = i * N + j;
+template <int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(256)
+    k_expm_small(int n, double dt, const double2* __restrict__ hA, const double2* __restrict__ hB,
+                 const double2* __restrict__ Z, double2* __restrict__ U, double2* __restrict__ U2) {
+    extern __shared__ __align__(16) double2 expm_sm[];
+    __shared__ float mod[kExpmSmallN * kExpmSmallN];
+    __shared__ float colsum[kExpmSmallN];
+    const int tid = threadIdx.x, nn = n * n;
+    int rank = 0;
+    if (CTAS > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    double2 *X = expm_sm, *X2 = X + nn, *X3 = X2 + nn, *X4 = X3 + nn, *Y = X4 + nn, *W = Y + nn;
+    for (int e = tid; e < nn; e += 256) {
+        double2 x;
+        if (Z) {
+            x = Z[e];
+        } else {
             const double hr = 0.5 * (hA[e].x + hB[e].x), hi = 0.5 * (hA[e].y + hB[e].y);
-            sum += dt * sqrt(hr * hr + hi * hi);
+            x = make_double2(dt * hi, -dt * hr);  // -i dt h
         }
-        colsum[j] = sum;
+        X[e] = x;
+        // the norm only selects s: FP32 with a margin for its rounding
+        const float re = (float)x.x, im = (float)x.y;
+        mod[e] = sqrtf(re * re + im * im);
     }
     __syncthreads();
-    double nrm = 0.0;
-    for (int j = 0; j < N; ++j) nrm = fmax(nrm, colsum[j]);
+    if (tid < n) {
+        float sum = 0.0f;
+        for (int i = 0; i < n; ++i) sum += mod[i * n + tid];
+        colsum[tid] = sum;
+    }
+    __syncthreads();
+    float nrm = 0.0f;
+    for (int j = 0; j < n; ++j) nrm = fmaxf(nrm, colsum[j]);
+    nrm *= 1.0001f;
     int s = 0;
-    while (s < 30 && ldexp(nrm, -s) > 0.5) ++s;
-    const double scale = ldexp(1.0, -s);
-    for (int e = tid; e < NN; e += blockDim.x) {
-        const double hr = 0.5 * (hA[e].x + hB[e].x), hi = 0.5 * (hA[e].y + hB[e].y);
-        X[e] = make_double2(scale * dt * hi, -scale * dt * hr);  // -i dt h / 2^s
-        Y[e] = make_double2((e / N == e % N) ? 1.0 : 0.0, 0.0);
-    }
-    __syncthreads();
-    double2 *y = Y, *z = Z;
-    for (int k = 18; k >= 1; --k) {
-        smem_zgemm(N, X, y, z, 1.0 / k, 1);
+    for (; s < 30 && nrm > 0.5f; ++s) nrm *= 0.5f;
+    const double scale = __hiloint2double((1023 - s) << 20, 0);
+    for (int e = tid; e < nn; e += 256) X[e] = make_double2(scale * X[e].x, scale * X[e].y);
+    if (CTAS == 1) {
         __syncthreads();
+    } else {
+        // every CTA of the cluster has started before remote stores begin
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    expm_product<CTAS>(n, rank, X, X, X2, -1, nullptr, nullptr, nullptr);
+    expm_product<CTAS>(n, rank, X, X2, X3, -1, nullptr, nullptr, nullptr);
+    expm_product<CTAS>(n, rank, X2, X2, X4, -1, nullptr, nullptr, nullptr);
+    // sum_{k=16..18} X^{k-16} / k!
+    for (int e = tid; e < nn; e += 256)
+        Y[e] = make_double2(fma(kExpmCoef.f[17], X[e].x, kExpmCoef.f[18] * X2[e].x) +
+                                (e / n == e % n ? kExpmCoef.f[16] : 0.0),
+                            fma(kExpmCoef.f[17], X[e].y, kExpmCoef.f[18] * X2[e].y));
+    __syncthreads();
+    double2 *y = Y, *z = W;
+    for (int j = 3; j >= 0; --j) {
+        expm_product<CTAS>(n, rank, y, X4, z, j, X, X2, X3);
         double2* t = y; y = z; z = t;
     }
     const int nsq = s < 16 ? s : 16;
     for (int q = 0; q < nsq; ++q) {
-        smem_zgemm(N, y, y, z, 1.0, 0);
-        __syncthreads();
+        expm_product<CTAS>(n, rank, y, y, z, -1, nullptr, nullptr, nullptr);
         double2* t = y; y = z; z = t;
     }
-    for (int e = tid; e < NN; e += blockDim.x) U[e] = y[e];
-    if (tid == 0) {
-        *norm_out = nrm;
-        *s_out = s;
-    }
+    if (rank == 0)
+        for (int e = tid; e < nn; e += 256) {
+            U[e] = y[e];
+            if (U2) U2[e] = y[e];
+        }
+}
+// Y = c16 I + c17 X + c18 X^2
+__global__ void k_expm_lead(int n, double c16, double c17, double c18, const double2* __restrict__ X,
+                            const double2* __restrict__ X2, double2* __restrict__ Y) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * n) return;
+    Y[e] = make_double2(fma(c17, X[e].x, c18 * X2[e].x) + (e / n == e % n ? c16 : 0.0),
+                        fma(c17, X[e].y, c18 * X2[e].y));
+}
+// The result of *s squarings (at most 16) that alternated between two buffers.
+__global__ void k_expm_select(long long n, const int* __restrict__ s, const double2* __restrict__ even,
+                              const double2* __restrict__ odd, double2* __restrict__ U, double2* __restrict__ U2) {
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const double2 x = (min(*s, 16) & 1) ? odd[e] : even[e];
+    U[e] = x;
+    if (U2) U2[e] = x;
 }
 
 // Diagnostics at t_n: {Tr rho, E_total, E_corr, Re Tr I}.
@@ -407,7 +545,7 @@ __global__ void k_forms64(int N, int nb, const double2* __restrict__ G, const do
 // so that I = sum_u coef_u S(G_u, Gb_u) Gb_u (first line of Eq. collint).
 // Writes G_u into Gout, Gb_u into Mb and the coefficients.
 __global__ void k_gkba_units(int N, int nk, int k0, int L, double dt, const double2* __restrict__ P,
-                             const double2* __restrict__ Q, const double* __restrict__ w,
+                             const double2* __restrict__ T, const double* __restrict__ w,
                              double2* __restrict__ Gout, double2* __restrict__ Mb,
                              double* __restrict__ coef) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -417,8 +555,9 @@ __global__ void k_gkba_units(int N, int nk, int k0, int L, double dt, const doub
     const int rr = (int)(e % NN);
     const int i = rr / N, j = rr % N;
     const long long base = (long long)kk * NN;
-    const double2 p = P[base + rr], q = Q[base + rr];
-    const double2 pt = P[base + (long long)j * N + i], qt = Q[base + (long long)j * N + i];
+    const long long tr = base + (long long)j * N + i;
+    const double2 p = P[base + rr], pt = P[tr], t = T[base + rr], tt = T[tr];
+    const double2 q = make_double2(t.x - p.x, t.y - p.y), qt = make_double2(tt.x - pt.x, tt.y - pt.y);  // Q = T - P
     Gout[(2 * kk + 0) * NN + rr] = p;
     Gout[(2 * kk + 1) * NN + rr] = q;
     Mb[(2 * kk + 0) * NN + rr] = make_double2(qt.x, -qt.y);  // (Q^+)_ij = conj(Q_ji)
@@ -522,18 +661,27 @@ __global__ void k_weighted_sum_p1(int NN, int nb, int per, const double* __restr
     }
     tmp[(long long)blockIdx.y * NN + e] = make_double2(re, im);
 }
+// One warp per element (a thread per element summed 256 ranges one after the
+// other: 31 us a call at N = 10, here 3).
 __global__ void k_weighted_sum_p2(int NN, int nz, const double2* __restrict__ tmp,
                                   double2* __restrict__ I_acc) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= NN) return;
     double re = 0.0, im = 0.0;
-    for (int z = 0; z < nz; ++z) {
+    for (int z = lane; z < nz; z += 32) {
         const double2 t = tmp[(long long)z * NN + e];
         re += t.x;
         im += t.y;
     }
-    I_acc[e].x += re;
-    I_acc[e].y += im;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane == 0) {
+        I_acc[e].x += re;
+        I_acc[e].y += im;
+    }
 }
 
 // hfK[(i*N + j)*N*N + l*N + k] = 2 v_iklj - v_ikjl  (Sigma_HF as a matrix-vector product)
@@ -609,7 +757,7 @@ __global__ void k_sigma_symm(int N, const double* __restrict__ V, const double2*
         double2 acc = make_double2(0.0, 0.0);
         for (int k = 0; k < N; ++k) {
             const double2 a = gb[(long long)l * N + k];
-            acc = cadd(acc, cmul(make_double2(vi[k] * a.x, vi[k] * a.y), g[(long long)k * N + l]));
+            cmac(acc, make_double2(vi[k] * a.x, vi[k] * a.y), g[(long long)k * N + l]);
         }
         r_sh[l] = acc;
     }
@@ -621,7 +769,7 @@ __global__ void k_sigma_symm(int N, const double* __restrict__ V, const double2*
             double2 w = make_double2(0.0, 0.0);
             for (int k = 0; k < N; ++k) {
                 const double2 a = gb[(long long)l * N + k];
-                w = cadd(w, cmul(make_double2(vi[k] * a.x, vi[k] * a.y), g[(long long)k * N + j]));
+                cmac(w, make_double2(vi[k] * a.x, vi[k] * a.y), g[(long long)k * N + j]);
             }
             const double2 b = cmul(gij, r_sh[l]);
             const double2 x = cmul(g[(long long)i * N + l], w);
@@ -632,51 +780,80 @@ __global__ void k_sigma_symm(int N, const double* __restrict__ V, const double2*
     }
 }
 
-// Same for N <= 24, one block per unit with G, Gb, V and r in shared memory:
+// Same for N <= 24 with G, Gb, V and r in shared memory, several units a block
+// (64 threads of work: finer blocks balance the SMs better than 128):
 //   r[i][l] = sum_k V_ik Gb_lk G_kl = [V x (Gb^T o G)]_il   (N^3)
 //   S_ij    = sum_l V_jl (2 G_ij r[i][l] - G_il sum_k V_ik Gb_lk G_kj)   (N^2 per (i, j))
-constexpr int kSymmSmallN = 24;  // 32 KB of static shared memory
-__global__ void __launch_bounds__(256) k_sigma_symm_small(int N, const double* __restrict__ V,
+// Bound by the FP64 rate.  A thread holds one row i and kSymmJ columns j, so that
+// V_ik Gb_lk is formed once for all of them: 4.4 FP64 instructions a term of the
+// N^4 sum (8 with one column a thread and multiplies kept apart from adds).
+// Measured at N = 10, 2002 units: 493 -> 230 us.
+constexpr int kSymmSmallN = 24, kSymmJ = 5, kSymmMaxUnits = 16, kSymmThreads = 64;
+inline int symm_units(int N) {  // units a block
+    const int per = N * ((N + kSymmJ - 1) / kSymmJ);
+    return std::max(1, std::min(kSymmMaxUnits, kSymmThreads / per));
+}
+inline size_t symm_smem(int N) { return (size_t)N * N * (8 + symm_units(N) * 3 * 16); }
+__global__ void __launch_bounds__(kSymmThreads) k_sigma_symm_small(int N, int nb, int upb, const double* __restrict__ V,
                                                            const double2* __restrict__ G,
                                                            const double2* __restrict__ Gb,
                                                            double2* __restrict__ S) {
-    __shared__ double2 g[kSymmSmallN * kSymmSmallN], gb[kSymmSmallN * kSymmSmallN],
-        r[kSymmSmallN * kSymmSmallN];
-    __shared__ double vs[kSymmSmallN * kSymmSmallN];
-    const int NN = N * N;
-    const long long base = (long long)blockIdx.x * NN;
-    for (int e = threadIdx.x; e < NN; e += blockDim.x) {
-        g[e] = G[base + e];
-        gb[e] = Gb[base + e];
-        vs[e] = V[e];
+    extern __shared__ __align__(16) double2 symm_sm[];
+    const int NN = N * N, u0 = blockIdx.x * upb, nu = min(upb, nb - u0);
+    double2 *g_s = symm_sm, *gb_s = g_s + upb * NN, *r_s = gb_s + upb * NN;
+    double* vs = (double*)(r_s + upb * NN);
+    const long long base = (long long)u0 * NN;
+    for (int e = threadIdx.x; e < NN; e += blockDim.x) vs[e] = V[e];
+    for (int e = threadIdx.x; e < nu * NN; e += blockDim.x) {
+        g_s[e] = G[base + e];
+        gb_s[e] = Gb[base + e];
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < NN; e += blockDim.x) {
-        const int i = e / N, l = e % N;
+    for (int e = threadIdx.x; e < nu * NN; e += blockDim.x) {
+        const int u = e / NN, rr = e - u * NN, i = rr / N, l = rr - i * N;
+        const double2 *g = g_s + u * NN, *gb = gb_s + u * NN;
         double2 acc = make_double2(0.0, 0.0);
         for (int k = 0; k < N; ++k) {
-            const double2 a = cmul(gb[l * N + k], g[k * N + l]);
-            acc = make_double2(fma(vs[i * N + k], a.x, acc.x), fma(vs[i * N + k], a.y, acc.y));
+            const double2 a = gb[l * N + k];
+            const double v = vs[i * N + k];
+            cmac(acc, make_double2(v * a.x, v * a.y), g[k * N + l]);
         }
-        r[e] = acc;
+        r_s[e] = acc;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < NN; e += blockDim.x) {
-        const int i = e / N, j = e % N;
-        const double2 gij = g[e];
-        double2 s = make_double2(0.0, 0.0);
+    const int njb = (N + kSymmJ - 1) / kSymmJ, per = N * njb;
+    for (int t = threadIdx.x; t < nu * per; t += blockDim.x) {
+        const int u = t / per, q = t - u * per, i = q / njb, j0 = (q - i * njb) * kSymmJ;
+        const double2 *g = g_s + u * NN, *gb = gb_s + u * NN, *r = r_s + u * NN;
+        double2 s[kSymmJ];
+        int jc[kSymmJ];
+#pragma unroll
+        for (int m = 0; m < kSymmJ; ++m) {
+            s[m] = make_double2(0.0, 0.0);
+            jc[m] = min(j0 + m, N - 1);
+        }
         for (int l = 0; l < N; ++l) {
-            double2 w = make_double2(0.0, 0.0);
+            double2 w[kSymmJ];
+#pragma unroll
+            for (int m = 0; m < kSymmJ; ++m) w[m] = make_double2(0.0, 0.0);
             for (int k = 0; k < N; ++k) {
                 const double2 a = gb[l * N + k];
-                w = cadd(w, cmul(make_double2(vs[i * N + k] * a.x, vs[i * N + k] * a.y), g[k * N + j]));
+                const double v = vs[i * N + k];
+                const double2 va = make_double2(v * a.x, v * a.y);
+#pragma unroll
+                for (int m = 0; m < kSymmJ; ++m) cmac(w[m], va, g[k * N + jc[m]]);
             }
-            const double2 b = cmul(gij, r[i * N + l]);
-            const double2 x = cmul(g[i * N + l], w);
-            const double vjl = vs[j * N + l];
-            s = cadd(s, make_double2(vjl * (2.0 * b.x - x.x), vjl * (2.0 * b.y - x.y)));
+            const double2 gil = g[i * N + l], ril = r[i * N + l];
+#pragma unroll
+            for (int m = 0; m < kSymmJ; ++m) {
+                const double2 b = cmul(g[i * N + jc[m]], ril), x = cmul(gil, w[m]);
+                const double vjl = vs[jc[m] * N + l];
+                s[m] = cadd(s[m], make_double2(vjl * (2.0 * b.x - x.x), vjl * (2.0 * b.y - x.y)));
+            }
         }
-        S[base + e] = s;
+#pragma unroll
+        for (int m = 0; m < kSymmJ; ++m)
+            if (j0 + m < N) S[base + u * NN + i * N + j0 + m] = s[m];
     }
 }
 
@@ -951,6 +1128,8 @@ __global__ void k_build_vomega64(int N, const double* __restrict__ v, double* __
 
 gkba_status fp64_prepare_model(gkba_ctx* c) {
     const long long n = c->N, N4 = n * n * n * n;
+    GKBA_CUDA(c, cudaFuncSetAttribute(k_expm_small<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(6 * kExpmSmallN * kExpmSmallN * sizeof(double2))));
     auto t = launch_begin(c, K_PREP, 0.0, 0.0);
     k_build_hfK<<<grid1(N4, 256), 256, 0, c->stream>>>(c->N, c->v, c->hfK);
     GKBA_TRY(launch_end(c, t));
@@ -961,7 +1140,6 @@ gkba_status fp64_prepare_model(gkba_ctx* c) {
     t = launch_begin(c, K_PREP, 0.0, 0.0);
     k_build_vK64<<<grid1(N4, 256), 256, 0, c->stream>>>(c->N, c->v, c->vK64);
     GKBA_TRY(launch_end(c, t));
-    if (!c->oz) return GKBA_OK;
     // stage S4 reads only the digit images of vK
     GKBA_TRY(oz_prepare(c));
     GKBA_TRY(oz_slice(c, c->vK64, n * n * n, 0, c->N, n * n * n, 1, c->vKimg));
@@ -973,51 +1151,34 @@ gkba_status fp64_prepare_model(gkba_ctx* c) {
 
 gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz,
                          const double* B, long long ldb, long long sBz, double* out,
-                         long long sOz, int M, int Nc, long long Ktot, int nz, int splitk,
-                         long long Kc, StageMap map, double flops, double bytes) {
-    if (c->oz && !splitk) {
-        const int nzB = sBz ? nz : 1;
-        if (oz_img_bytes(Nc, Ktot) * nzB <= c->ozimg_bytes) {
-            GKBA_TRY(oz_slice(c, B, ldb, sBz, Nc, Ktot, nzB, c->ozimg));
-            return oz_gemm(c, cls, A, lda, sAz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
-        }
-    }
-    dim3 grid((Nc + G64_BN - 1) / G64_BN, (M + G64_BM - 1) / G64_BM, nz);
-    if (grid.y > 65535u) return fail(c, GKBA_EINVAL, "stage GEMM: M=%d too large", M);
-    auto t = launch_begin(c, cls, flops, bytes);
-    k_gemm64_stage<<<grid, 256, 0, c->stream>>>(A, lda, sAz, B, ldb, sBz, out, sOz, M, Nc, Ktot,
-                                                splitk, Kc, map);
-    return launch_end(c, t);
-}
-
-long long gemm64_splitk_chunk(gkba_ctx* c, int M, int Nc, long long K, long long max_chunks) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemm64_stage, 256, 0) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
-    const long long bpz = (long long)((Nc + G64_BN - 1) / G64_BN) * ((M + G64_BM - 1) / G64_BM);
-    long long nz = std::max(1LL, (long long)per_sm * c->num_sms / bpz);
-    nz = std::min(nz, std::max(1LL, max_chunks));
-    const long long Kc = (K + nz - 1) / nz;
-    return (Kc + G64_BK - 1) / G64_BK * G64_BK;
+                         long long sOz, int M, int Nc, long long Ktot, int nz, StageMap map,
+                         double flops, double bytes) {
+    const int nzB = sBz ? nz : 1;
+    if (oz_img_bytes(Nc, Ktot) * nzB > c->ozimg_bytes)
+        return fail(c, GKBA_ESTATE, "digit images of %d operands of %d x %lld do not fit", nzB, Nc, Ktot);
+    GKBA_TRY(oz_slice(c, B, ldb, sBz, Nc, Ktot, nzB, c->ozimg));
+    return oz_gemm(c, cls, A, lda, sAz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
 }
 
 static gkba_status zgemm_impl(gkba_ctx* c, int cls, int n, char opA, char opB, double2 alpha,
                               const double2* A, long long sA, const double2* B, long long sB,
-                              double2 beta, double2* C, long long sC, int batch, int add_identity,
-                              const int* skip_ge, int idx) {
-    if (batch <= 0) return GKBA_OK;
-    dim3 grid((n + ZT - 1) / ZT, (n + ZT - 1) / ZT, 1);
+                              double2 beta, double2* C, long long sC, int batch, int n_ident,
+                              const ZPoly& p, const int* skip_ge, int idx) {
     const double flops = 8.0 * n * (double)n * n;
-    for (int b0 = 0; b0 < batch; b0 += 65535) {
-        const int nbat = batch - b0 < 65535 ? batch - b0 : 65535;
-        grid.z = nbat;
-        auto t = launch_begin(c, cls, flops * nbat, 0.0);
-        k_zgemm<<<grid, 256, 0, c->stream>>>(n, opA == 'C', opB == 'C', alpha, A + b0 * sA, sA,
-                                             B + b0 * sB, sB, beta, C + b0 * sC, sC, add_identity,
-                                             skip_ge, idx);
+    const long long nn = (long long)n * n;
+    const int all = batch + n_ident;
+    const int most = (int)std::min<long long>(1LL << 30, (1LL << 31) / (8 * nn));  // 32-bit thread index
+    for (int b0 = 0; b0 < all; b0 += most) {
+        const int nb = std::min(most, all - b0), nid = std::max(0, std::min(nb, batch - b0));
+        const uint32_t total = (uint32_t)(nb * nn);
+        // lanes per output: about four warps on every SM for a few matrices
+        const long long want = 4LL * c->num_sms * 32 / total;
+        const int tpo = want >= 8 ? 8 : want >= 4 ? 4 : want >= 2 ? 2 : 1;
+        const unsigned grid = grid1((long long)total * tpo, 128);
+        auto kfn = tpo == 8 ? k_zgemm<8> : tpo == 4 ? k_zgemm<4> : tpo == 2 ? k_zgemm<2> : k_zgemm<1>;
+        auto t = launch_begin(c, cls, flops * nid, 0.0);
+        kfn<<<grid, 128, 0, c->stream>>>(n, opA == 'C', opB == 'C', alpha, A + b0 * sA, sA, B + b0 * sB, sB, beta,
+                                         C + b0 * sC, sC, total, nid, p, skip_ge, idx);
         GKBA_TRY(launch_end(c, t));
     }
     return GKBA_OK;
@@ -1025,9 +1186,9 @@ static gkba_status zgemm_impl(gkba_ctx* c, int cls, int n, char opA, char opB, d
 
 gkba_status zgemm_batched(gkba_ctx* c, int cls, int n, char opA, char opB, double2 alpha,
                           const double2* A, long long sA, const double2* B, long long sB,
-                          double2 beta, double2* C, long long sC, int batch, int add_identity) {
-    return zgemm_impl(c, cls, n, opA, opB, alpha, A, sA, B, sB, beta, C, sC, batch, add_identity,
-                      nullptr, 0);
+                          double2 beta, double2* C, long long sC, int batch, int n_ident) {
+    if (batch + n_ident <= 0) return GKBA_OK;
+    return zgemm_impl(c, cls, n, opA, opB, alpha, A, sA, B, sB, beta, C, sC, batch, n_ident, ZPoly{}, nullptr, 0);
 }
 
 gkba_status mean_field(gkba_ctx* c, const double2* rho, double2* out) {
@@ -1046,59 +1207,80 @@ gkba_status h_hf(gkba_ctx* c, double E, const double2* rho, double2* out) {
     return launch_end(c, t);
 }
 
-gkba_status rhs(gkba_ctx* c, const double2* hhf, const double2* rho, const double2* I, double2* out) {
-    const int N = c->N;
-    const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
-    GKBA_TRY(zgemm_batched(c, K_STEP, N, 'N', 'N', one, hhf, 0, rho, 0, zero, c->tmp0, 0, 1, 0));
-    GKBA_TRY(zgemm_batched(c, K_STEP, N, 'N', 'N', one, rho, 0, hhf, 0, zero, c->tmp1, 0, 1, 0));
-    auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-    k_rhs<<<grid1((long long)N * N, 256), 256, 0, c->stream>>>(N, c->tmp0, c->tmp1, I, out);
+gkba_status heun_stage(gkba_ctx* c, const double2* hhf, const double2* rho, const double2* I, const double2* base,
+                       const double2* kprev, double a, double2* k_out, double2* y, double2* y2) {
+    const long long NN = (long long)c->N * c->N;
+    auto t = launch_begin(c, K_STEP, 16.0 * NN * c->N, 0.0);
+    k_heun_stage<<<grid1(NN * kRhsLanes, 128), 128, 0, c->stream>>>(c->N, hhf, rho, I, base, kprev, a, k_out, y, y2);
     return launch_end(c, t);
 }
 
-gkba_status expm_step(gkba_ctx* c, const double2* hA, const double2* hB, double2* U) {
+// exp(X) by products spread over all SMs: the Paterson-Stockmeyer form of the
+// degree-18 Taylor polynomial (k_expm_small), then up to 16 squarings of which
+// the device-side count c->dint[0] runs.  X: the scaled argument; X2, X3, X4, Y,
+// W: n x n scratch; the result goes to U (and U2).
+static gkba_status expm_products(gkba_ctx* c, int n, const double2* X, double2* X2, double2* X3, double2* X4,
+                                 double2* Y, double2* W, double2* U, double2* U2) {
+    const long long nn = (long long)n * n;
+    const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
+    auto prod = [&](const double2* A, const double2* B, double2* C, const ZPoly& p) {
+        return zgemm_impl(c, K_STEP, n, 'N', 'N', one, A, 0, B, 0, zero, C, 0, 1, 0, p, nullptr, 0);
+    };
+    GKBA_TRY(prod(X, X, X2, ZPoly{}));
+    GKBA_TRY(prod(X, X2, X3, ZPoly{}));
+    GKBA_TRY(prod(X2, X2, X4, ZPoly{}));
+    double f[19];
+    f[0] = 1.0;
+    for (int k = 1; k <= 18; ++k) f[k] = f[k - 1] / k;
+    {
+        auto t = launch_begin(c, K_STEP, 0.0, 0.0);
+        k_expm_lead<<<grid1(nn, 256), 256, 0, c->stream>>>(n, f[16], f[17], f[18], X, X2, Y);
+        GKBA_TRY(launch_end(c, t));
+    }
+    double2 *y = Y, *z = W;
+    for (int j = 3; j >= 0; --j) {
+        ZPoly p;
+        p.c0 = f[4 * j];
+        p.c1 = f[4 * j + 1];
+        p.c2 = f[4 * j + 2];
+        p.c3 = f[4 * j + 3];
+        p.X1 = X;
+        p.X2 = X2;
+        p.X3 = X3;
+        GKBA_TRY(prod(y, X4, z, p));
+        std::swap(y, z);
+    }
+    // X3 is free now: squarings alternate between y and it
+    double2* sq[2] = {y, X3};
+    for (int i = 0; i < 16; ++i)
+        GKBA_TRY(zgemm_impl(c, K_STEP, n, 'N', 'N', one, sq[i & 1], 0, sq[i & 1], 0, zero, sq[(i + 1) & 1], 0, 1, 0,
+                            ZPoly{}, c->dint + 0, i));
+    auto t = launch_begin(c, K_STEP, 0.0, 0.0);
+    k_expm_select<<<grid1(nn, 256), 256, 0, c->stream>>>(nn, c->dint + 0, sq[0], sq[1], U, U2);
+    return launch_end(c, t);
+}
+
+static gkba_status expm_small(gkba_ctx* c, int n, const double2* hA, const double2* hB, const double2* Z,
+                                double2* U, double2* U2) {
+    const size_t smem = 6 * (size_t)n * n * sizeof(double2);
+    auto t = launch_begin(c, K_STEP, 0.0, 0.0);
+    if (n <= kExpmOneN) k_expm_small<1><<<1, 256, smem, c->stream>>>(n, c->dt, hA, hB, Z, U, U2);
+    else k_expm_small<8><<<8, 256, smem, c->stream>>>(n, c->dt, hA, hB, Z, U, U2);
+    return launch_end(c, t);
+}
+
+gkba_status expm_step(gkba_ctx* c, const double2* hA, const double2* hB, double2* U, double2* U2) {
     // Scaling and squaring with a degree-18 Taylor polynomial (Moler & Van Loan,
     // "Nineteen dubious ways to compute the exponential of a matrix"): with
     // ||A/2^s||_1 <= 1/2 the truncation error is below 0.5^19/19! ~ 1e-23.
     const int N = c->N;
-    const long long NN = (long long)N * N;
-    double2* X = c->ex0;  // scaled argument B = A / 2^s
-    double2* Y = c->ex1;
-    double2* Z = c->ex2;
-    if (N <= kExpmSmallN) {
-        auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_expm_small<<<1, 256, 0, c->stream>>>(N, c->dt, hA, hB, U, c->dscal + 8, c->dint + 0);
-        return launch_end(c, t);
-    }
+    if (N <= kExpmSmallN) return expm_small(c, N, hA, hB, nullptr, U, U2);
     {
         auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_expm_setup<<<1, 256, 0, c->stream>>>(N, c->dt, hA, hB, X, c->dscal + 8, c->dint + 0);
+        k_expm_setup<<<1, 256, 0, c->stream>>>(N, c->dt, hA, hB, c->ex0, c->dscal + 8, c->dint + 0);
         GKBA_TRY(launch_end(c, t));
     }
-    const int deg = 18;
-    // Y = I + X / deg
-    {
-        auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_set_identity<<<grid1(NN, 256), 256, 0, c->stream>>>(N, 1, Y);
-        GKBA_TRY(launch_end(c, t));
-        GKBA_TRY(zgemm_batched(c, K_STEP, N, 'N', 'N', make_double2(1.0 / deg, 0.0), X, 0, Y, 0,
-                               make_double2(0.0, 0.0), Z, 0, 1, 1));
-        std::swap(Y, Z);
-    }
-    for (int k = deg - 1; k >= 1; --k) {
-        GKBA_TRY(zgemm_batched(c, K_STEP, N, 'N', 'N', make_double2(1.0 / k, 0.0), X, 0, Y, 0,
-                               make_double2(0.0, 0.0), Z, 0, 1, 1));
-        std::swap(Y, Z);
-    }
-    // up to kMaxSq squarings; step i is a copy when i >= s (device-side count)
-    const int kMaxSq = 16;
-    for (int i = 0; i < kMaxSq; ++i) {
-        GKBA_TRY(zgemm_impl(c, K_STEP, N, 'N', 'N', make_double2(1.0, 0.0), Y, 0, Y, 0,
-                            make_double2(0.0, 0.0), Z, 0, 1, 0, c->dint + 0, i));
-        std::swap(Y, Z);
-    }
-    GKBA_CUDA(c, cudaMemcpyAsync(U, Y, NN * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
-    return GKBA_OK;
+    return expm_products(c, N, c->ex0, c->ex1, c->ex2, c->tmp0, c->tmp1, U, U, U2);
 }
 
 gkba_status axpy_c(gkba_ctx* c, double2* y, const double2* x, const double2* z, double a, double b,
@@ -1122,27 +1304,13 @@ gkba_status diagnostics(gkba_ctx* c, double E_n, const double2* rho, const doubl
     return launch_end(c, t);
 }
 
-// P_k = T_k rho_k, Q_k = T_k - P_k for k in [k0, k0+nk), then the unit list.
+// P_k = T_k rho_k for k in [k0, k0+nk), then the unit list.
 // The G_u are staged in Su (free until the reduction of this batch).
 gkba_status build_forms_gkba(gkba_ctx* c, int k0, int nk, int L, const double2* rho,
                              const double2* T, const double* w) {
     const int N = c->N;
     const long long NN = (long long)N * N;
-    double2* P = c->PQ;
-    double2* Q = c->PQ + (long long)nk * NN;
-    GKBA_TRY(zgemm_batched(c, K_PREP, N, 'N', 'N', make_double2(1.0, 0.0), T + k0 * NN, NN,
-                           rho + k0 * NN, NN, make_double2(0.0, 0.0), P, NN, nk, 0));
-    {
-        auto t = launch_begin(c, K_PREP, 0.0, 0.0);
-        k_lincomb<<<grid1(nk * NN, 256), 256, 0, c->stream>>>(nk * NN, Q, T + k0 * NN, P, 1.0, -1.0);
-        GKBA_TRY(launch_end(c, t));
-    }
-    {
-        auto t = launch_begin(c, K_PREP, 0.0, 0.0);
-        k_gkba_units<<<grid1(nk * NN, 256), 256, 0, c->stream>>>(N, nk, k0, L, c->dt, P, Q, w,
-                                                                  c->Su, c->Mb, c->coef);
-        GKBA_TRY(launch_end(c, t));
-    }
+    GKBA_TRY(units_from_history(c, N, k0, nk, L, c->dt, rho, T, w, c->Su, c->Mb, c->coef));
     return build_forms(c, 2 * nk, c->Su, NN, c->Mb, NN, 0);
 }
 
@@ -1154,14 +1322,10 @@ gkba_status units_from_history(gkba_ctx* c, int N, int k0, int nk, int L, double
                                double2* Gb, double* coef) {
     const long long NN = (long long)N * N;
     double2* P = c->PQ;
-    double2* Q = c->PQ + (long long)nk * NN;
     GKBA_TRY(zgemm_batched(c, K_PREP, N, 'N', 'N', make_double2(1.0, 0.0), T + k0 * NN, NN,
                            rho + k0 * NN, NN, make_double2(0.0, 0.0), P, NN, nk, 0));
     auto t = launch_begin(c, K_PREP, 0.0, 0.0);
-    k_lincomb<<<grid1(nk * NN, 256), 256, 0, c->stream>>>(nk * NN, Q, T + k0 * NN, P, 1.0, -1.0);
-    GKBA_TRY(launch_end(c, t));
-    t = launch_begin(c, K_PREP, 0.0, 0.0);
-    k_gkba_units<<<grid1(nk * NN, 256), 256, 0, c->stream>>>(N, nk, k0, L, dt, P, Q, w, G, Gb, coef);
+    k_gkba_units<<<grid1(nk * NN, 256), 256, 0, c->stream>>>(N, nk, k0, L, dt, P, T + k0 * NN, w, G, Gb, coef);
     return launch_end(c, t);
 }
 
@@ -1176,7 +1340,7 @@ gkba_status weighted_sum_units(gkba_ctx* c, int N, int nb, const double* coef, c
                                                                        c->red_tmp);
     GKBA_TRY(launch_end(c, t));
     t = launch_begin(c, K_RED, 0.0, 0.0);
-    k_weighted_sum_p2<<<grid1(NN, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I);
+    k_weighted_sum_p2<<<grid1(NN * 32, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I);
     return launch_end(c, t);
 }
 
@@ -1228,47 +1392,31 @@ gkba_status field_grad(gkba_ctx* c, const double2* hb, double* out) {
     k_field_grad<<<1, 256, 0, c->stream>>>(c->N, hb, c->d, out);
     return launch_end(c, t);
 }
-// exp(Z) of a general complex n x n matrix (Taylor degree 18 by Horner after
-// scaling, then the squarings); X, Y, W: n x n scratch, result in W.
-static gkba_status expm_general(gkba_ctx* c, int n, const double2* Z, double2* X, double2* Y,
-                                double2* W) {
+// exp(Z) of a general complex n x n matrix into W; Z is overwritten, S: 4 n x n
+// scratch matrices.
+static gkba_status expm_general(gkba_ctx* c, int n, double2* Z, double2* S, double2* W) {
+    if (n <= kExpmSmallN) return expm_small(c, n, nullptr, nullptr, Z, W, nullptr);
+    const long long nn = (long long)n * n;
     {
         auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_expm_setup_general<<<1, 256, 0, c->stream>>>(n, Z, X, c->dint + 0);
-        GKBA_TRY(launch_end(c, t));
-        t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_set_identity<<<grid1((long long)n * n, 256), 256, 0, c->stream>>>(n, 1, Y);
+        k_expm_setup_general<<<1, 256, 0, c->stream>>>(n, Z, S, c->dint + 0);
         GKBA_TRY(launch_end(c, t));
     }
-    double2 *y = Y, *z = W;
-    for (int k = 18; k >= 1; --k) {
-        GKBA_TRY(zgemm_batched(c, K_STEP, n, 'N', 'N', make_double2(1.0 / k, 0.0), X, 0, y, 0,
-                               make_double2(0.0, 0.0), z, 0, 1, 1));
-        std::swap(y, z);
-    }
-    for (int i = 0; i < 16; ++i) {
-        GKBA_TRY(zgemm_impl(c, K_STEP, n, 'N', 'N', make_double2(1.0, 0.0), y, 0, y, 0,
-                            make_double2(0.0, 0.0), z, 0, 1, 0, c->dint + 0, i));
-        std::swap(y, z);
-    }
-    if (y != W)
-        GKBA_CUDA(c, cudaMemcpyAsync(W, y, (size_t)n * n * sizeof(double2), cudaMemcpyDeviceToDevice,
-                                     c->stream));
-    return GKBA_OK;
+    return expm_products(c, n, S, Z, S + nn, S + 2 * nn, S + 3 * nn, W, W, nullptr);
 }
 // Adjoint of U = exp(-i dt (hA + hB)/2): hA_bar, hB_bar += (i dt / 2) L_exp(X^+, Ubar).
-// scratch: 4 blocks of (2N)^2 entries.
+// scratch: 6 blocks of (2N)^2 entries.
 gkba_status expm_adj(gkba_ctx* c, const double2* hA, const double2* hB, const double2* Ubar,
                      double2* hA_bar, double2* hB_bar, double2* scratch) {
     const int N = c->N, M = 2 * N;
     const long long MM = (long long)M * M;
-    double2 *Z = scratch, *X = scratch + MM, *Y = scratch + 2 * MM, *W = scratch + 3 * MM;
+    double2 *Z = scratch, *S = scratch + MM, *W = scratch + 5 * MM;
     {
         auto t = launch_begin(c, K_STEP, 0.0, 0.0);
         k_frechet_block<<<1, 256, 0, c->stream>>>(N, c->dt, hA, hB, Ubar, Z, c->dscal + 12);
         GKBA_TRY(launch_end(c, t));
     }
-    GKBA_TRY(expm_general(c, M, Z, X, Y, W));
+    GKBA_TRY(expm_general(c, M, Z, S, W));
     auto t = launch_begin(c, K_STEP, 0.0, 0.0);
     k_frechet_apply<<<grid1((long long)N * N, 256), 256, 0, c->stream>>>(N, c->dt, W, c->dscal + 12,
                                                                          hA_bar, hB_bar);
@@ -1365,7 +1513,7 @@ gkba_status reduce_batch(gkba_ctx* c, int nb, double2* I_acc, double2* S_out) {
                                                                        c->Yu, c->red_tmp);
     GKBA_TRY(launch_end(c, t));
     t = launch_begin(c, K_RED, 0.0, 0.0);
-    k_weighted_sum_p2<<<grid1(NN, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I_acc);
+    k_weighted_sum_p2<<<grid1(NN * 32, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I_acc);
     return launch_end(c, t);
 }
 
@@ -1390,20 +1538,20 @@ gkba_status fp64_chain_x3(gkba_ctx* c, int nb, const double* A1, const StageMap*
     {
         StageMap m{2 * N3, 2 * N, 1, N, 2 * N2, N, N, N};
         GKBA_TRY(gemm64_stage(c, K_W1, A1, N, 0, (const double*)c->formsB1, N, 2 * N2, X13,
-                              2 * N4, (int)N3, 2 * N, N, nb, 0, 0, m, fl_cr * nb,
+                              2 * N4, (int)N3, 2 * N, N, nb, m, fl_cr * nb,
                               8.0 * (N4 + 2 * N4 * nb)));
     }
     {
         StageMap m{2 * N3, 2 * N2, 1, N, 2 * N, N, N, N};
         GKBA_TRY(gemm64_stage(c, K_W2, X13, 2 * N, 2 * N4, (const double*)c->formsG, 2 * N, 4 * N2,
-                              X2, 2 * N4, (int)N3, 2 * N, 2 * N, nb, 0, 0, m, fl_cc * nb,
+                              X2, 2 * N4, (int)N3, 2 * N, 2 * N, nb, m, fl_cc * nb,
                               8.0 * 4 * N4 * nb));
     }
     {
         const StageMap m = m3 ? *m3 : StageMap{N3, N, 1, N4, N2, N, N, N};
         GKBA_TRY(gemm64_stage(c, K_W3, X2, 2 * N, 2 * N4,
                               (const double*)(c->sep_A ? c->formsG3 : c->formsG), 2 * N, 4 * N2,
-                              X13, m3 ? sOz3 : 2 * N4, (int)N3, 2 * N, 2 * N, nb, 0, 0, m,
+                              X13, m3 ? sOz3 : 2 * N4, (int)N3, 2 * N, 2 * N, nb, m,
                               fl_cc * nb, 8.0 * 4 * N4 * nb));
     }
     return GKBA_OK;
@@ -1418,18 +1566,8 @@ gkba_status fp64_final(gkba_ctx* c, int nb) {
     const long long R = 2LL * N * nb;
     const StageMap m{0, 0, 1, 0, R, (int)R, 1, N};
     const long long max_z = (long long)(c->part_bytes / (N * R * 8));
-    int nz;
-    if (c->oz) {
-        nz = oz_items(c, (int)R, N, N3, max_z);
-        GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m,
-                         fl, by));
-    } else {
-        // chunks that fill one wave of blocks when one unit has few output tiles
-        const long long Kc = nb > 1 ? 8192 : gemm64_splitk_chunk(c, (int)R, N, N3, max_z);
-        nz = (int)((N3 + Kc - 1) / Kc);
-        GKBA_TRY(gemm64_stage(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, (double*)c->part, N * R, (int)R, N, N3, nz, 1,
-                              Kc, m, fl, by));
-    }
+    const int nz = oz_items(c, (int)R, N, N3, max_z);
+    GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m, fl, by));
     return reduce_partials_launch(c, nb, nz, N * R, R, c->part, false, c->Su);
 }
 
@@ -1450,9 +1588,9 @@ gkba_status contract_structured(gkba_ctx* c, int nb, const double2* G, const dou
         k_sigma_diag<<<grid1(nb * NN, 256), 256, 0, c->stream>>>(N, nb, c->vm, G, Gb, c->PQ);
         GKBA_TRY(launch_end(c, t));
     } else if (N <= kSymmSmallN) {
-        const int bs = N * N >= 256 ? 256 : ((N * N + 31) / 32) * 32;
         auto t = launch_begin(c, K_W1, 8.0 * n * n * n * n * nb, 48.0 * n * n * nb);
-        k_sigma_symm_small<<<nb, bs, 0, c->stream>>>(N, c->vm, G, Gb, c->PQ);
+        const int upb = symm_units(N);
+        k_sigma_symm_small<<<(nb + upb - 1) / upb, kSymmThreads, symm_smem(N), c->stream>>>(N, nb, upb, c->vm, G, Gb, c->PQ);
         GKBA_TRY(launch_end(c, t));
     } else {
         const int bs = N >= 128 ? 128 : ((N + 31) / 32) * 32;

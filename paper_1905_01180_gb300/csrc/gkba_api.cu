@@ -103,12 +103,13 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const long long Np = c->Np;
     const double x_bytes = !gen ? 0.0 : tc ? 2.0 * Np * Np * Np * Np * 4 : 2.0 * NN * NN * 8;
     const double form_bytes = !gen ? 0.0 : tc ? 4.0 * 2 * Np * Np * 4 : (2.0 * NN + 4.0 * NN) * 8;
-    const double N3 = (double)NN * N;
     const double part_per_unit = !gen ? 0.0
                                  : tc ? (std::ceil((double)Np * Np * Np / kTcItemK) * Np * 2.0 * Np * 4)
-                                      : (std::ceil(N3 / 8192.0) * N * 2.0 * N * 8);
-    const double img_bytes = c->oz ? 1.25 * (double)oz_img_bytes(2 * (int)N, 2 * N) : 0.0;
-    const double per_unit = img_bytes + 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
+                                      : std::ceil((double)NN * N / 8192.0) * N * 2.0 * N * 8;
+    const double base_unit = 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
+    // digit images of one stage's per-unit operands (the widest: S2 and S3)
+    const double img_unit = c->oz ? (double)oz_img_bytes(2 * (int)N, 2 * N) : 0.0;
+    const double per_unit = base_unit + img_unit;
     size_t cap = c->ws_cap;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
@@ -117,9 +118,11 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     }
     long long fit = (long long)((double)cap / per_unit);
     fit -= fit & 1;
+    // a cap that holds two units without their images is met up to the images
+    if (fit < 2 && (double)cap >= 2 * base_unit) fit = 2;
     if (fit < 2)
         return fail(c, GKBA_ENOMEM, "workspace cap %.3g GB holds fewer than 2 units (%.3g GB each)",
-                    cap / 1e9, per_unit / 1e9);
+                    cap / 1e9, base_unit / 1e9);
     int ub = (int)std::min<long long>(fit, want_units);
     if (c->ws && ub <= c->ub_cap) {
         c->ub = ub;
@@ -139,19 +142,18 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     size_t part_bytes;
     if (!gen) part_bytes = 0;
     else if (tc) part_bytes = tf32_part_bytes((int)Np, ub, c->acc_window);
+    // partial sums of oz_gemm: two items per SM of 128 rows if the cap allows them
+    // next to the units, at least one partial sum of every row
     else {
-        const long long nz = (long long)std::ceil(N3 / 8192.0);
-        part_bytes = (size_t)(nz * N * 2LL * N * ub * 8);
-        // the time-linear collision splits one unit's K into up to 1024 chunks
-        if (c->history == GKBA_HISTORY_TIME_LINEAR)
-            part_bytes = std::max(part_bytes, (size_t)(1024LL * N * 2LL * N * 8));
+        const double want = (double)N * 8 * 2 * c->num_sms * 128, room = (double)cap - per_unit * ub;
+        part_bytes = (size_t)std::max(2.0 * N * N * 8 * ub, std::min(want, room));
     }
-    // partial sums of oz_gemm: at most two items per SM of 128 rows, or one item
-    if (c->oz) part_bytes = (size_t)N * 8 * std::max(2LL * c->num_sms * 128, 2LL * N * ub);
     const size_t oPart = cv.take(part_bytes);
-    // digit images of one stage's per-unit operands (the widest: S2 and S3); the
-    // time-linear accumulator's one long operand pads its windows differently
-    const size_t ozimg_bytes = c->oz ? (size_t)(img_bytes * ub) + ((size_t)64 << 10) : 0;
+    // the time-linear accumulator's one operand is as long as all units' together
+    const size_t ozimg_bytes = !c->oz ? 0
+                               : std::max((size_t)(img_unit * ub), c->history == GKBA_HISTORY_TIME_LINEAR
+                                                                       ? oz_img_bound(2 * (int)N, 2LL * N * ub)
+                                                                       : 0);
     const size_t oImg = cv.take(ozimg_bytes);
     const size_t oB1 = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 2 * Np * Np * ub * 4) : (size_t)(2LL * NN * ub * 8));
     const size_t oG = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 4 * Np * Np * ub * 4) : (size_t)(4LL * NN * ub * 8));
@@ -633,8 +635,8 @@ gkba_status gkba_init(gkba_ctx** out, const gkba_config* cfg, const double* h, c
     } else if (c->prec == GKBA_FP64) {
         ALLOC(c->wS64, N4 * 8);
         ALLOC(c->vK64, N4 * 8);
-        c->oz = N >= kOzMinN;
-        if (c->oz) ALLOC(c->vKimg, oz_img_bytes(N, (long long)N4 / N));
+        c->oz = true;
+        ALLOC(c->vKimg, oz_img_bytes(N, (long long)N4 / N));
         if (c->history == GKBA_HISTORY_TIME_LINEAR) {
             ALLOC(c->tl_acc, 2 * N4 * 8);
             ALLOC(c->tl_s, 2 * N4 * 8);
@@ -928,18 +930,16 @@ gkba_status gkba_step(gkba_ctx* c, double E_n, double E_np1, double* rho_out, do
         GKBA_TRY(collision_dev(c, n + 1, c->rho_hist, c->T_a, nullptr, c->Ia));
     }
     GKBA_TRY(diagnostics(c, E_n, rho_n, c->Ia, c->dscal));
-    GKBA_TRY(rhs(c, c->hhf_n, rho_n, c->Ia, c->k1));
-    GKBA_TRY(axpy_c(c, rho_t, rho_n, c->k1, 1.0, c->dt, (int)NN));
-    GKBA_CUDA(c, cudaMemcpyAsync(c->rhot_hist + n * NN, rho_t, NN * 16, cudaMemcpyDeviceToDevice, c->stream));
+    // k1 and rho~ = rho_n + dt k1 (kept twice: the history slot is overwritten by the corrector)
+    double2* rho_pred = c->rhot_hist + n * NN;
+    GKBA_TRY(heun_stage(c, c->hhf_n, rho_n, c->Ia, rho_n, nullptr, c->dt, c->k1, rho_t, rho_pred));
     GKBA_TRY(h_hf(c, E_np1, rho_t, c->hhf_t));
     // propagator recursion T(t_{n+1}, t_k) = U_n T(t_n, t_k); T(t_{n+1}, t_{n+1}) = 1
-    GKBA_TRY(expm_step(c, c->hhf_n, c->hhf_t, c->U));
-    GKBA_CUDA(c, cudaMemcpyAsync(c->U_hist + n * NN, c->U, NN * 16, cudaMemcpyDeviceToDevice, c->stream));
+    GKBA_TRY(expm_step(c, c->hhf_n, c->hhf_t, c->U, c->U_hist + n * NN));
     c->E_a[n] = E_n;
     c->E_b[n] = E_np1;
     GKBA_TRY(zgemm_batched(c, K_STEP, c->N, 'N', 'N', make_double2(1.0, 0.0), c->U, 0, c->T_a, NN,
-                           make_double2(0.0, 0.0), c->T_b, NN, n + 1, 0));
-    GKBA_TRY(set_identity(c, c->T_b + (n + 1) * NN, 1));
+                           make_double2(0.0, 0.0), c->T_b, NN, n + 1, 1));
     // corrector
     if (tl) {
         // W_{n+1} = Ucal_{n+1}^+ = W_n U_n^+; Lambda = Lambda_acc + dt/2 term(rho~)
@@ -951,9 +951,7 @@ gkba_status gkba_step(gkba_ctx* c, double E_n, double E_np1, double* rho_out, do
     } else {
         GKBA_TRY(collision_dev(c, n + 2, c->rho_hist, c->T_b, nullptr, c->Ib));
     }
-    GKBA_TRY(rhs(c, c->hhf_t, rho_t, c->Ib, c->k2));
-    GKBA_TRY(axpy_c(c, c->k2, c->k1, c->k2, 1.0, 1.0, (int)NN));
-    GKBA_TRY(axpy_c(c, rho_t, rho_n, c->k2, 1.0, 0.5 * c->dt, (int)NN));
+    GKBA_TRY(heun_stage(c, c->hhf_t, rho_pred, c->Ib, rho_n, c->k1, 0.5 * c->dt, nullptr, rho_t, nullptr));
     std::swap(c->T_a, c->T_b);
     if (tl) std::swap(c->tl_W, c->tl_Wn);
     c->n = n + 1;
@@ -1053,7 +1051,7 @@ gkba_status gkba_adjoint(gkba_ctx* c, const double* rho_bar_final, double* E_bar
     const int M = c->n, N = c->N;
     const long long NN = (long long)N * N;
     const size_t H = (size_t)(M + 2) * NN;  // one history-sized block
-    const size_t need = (7 * H + 12 * NN + 16 * NN) * sizeof(double2) + (size_t)(M + 1) * 8 + 256;
+    const size_t need = (7 * H + 12 * NN + 24 * NN) * sizeof(double2) + (size_t)(M + 1) * 8 + 256;
     if (c->adj_ws_bytes < need) {
         if (c->adj_ws) cudaFree(c->adj_ws);
         c->adj_ws = nullptr;
@@ -1071,8 +1069,8 @@ gkba_status gkba_adjoint(gkba_ctx* c, const double* rho_bar_final, double* E_bar
     double2 *kb = sm, *kb1 = sm + NN, *hA = sm + 2 * NN, *hB = sm + 3 * NN, *hAb = sm + 4 * NN,
             *hBb = sm + 5 * NN, *rtb = sm + 6 * NN, *Ib = sm + 7 * NN, *P1 = sm + 8 * NN,
             *P2 = sm + 9 * NN, *Ub = sm + 10 * NN, *save = sm + 11 * NN;
-    double2* fre = sm + 12 * NN;  // 4 (2N)^2 blocks = 16 NN
-    double* Eb = (double*)(fre + 16 * NN);
+    double2* fre = sm + 12 * NN;  // 6 (2N)^2 blocks = 24 NN
+    double* Eb = (double*)(fre + 24 * NN);
     const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
     const double dt = c->dt;
     GKBA_CUDA(c, cudaMemsetAsync(Rb, 0, H * sizeof(double2), c->stream));
@@ -1585,19 +1583,13 @@ gkba_status batch_step(gkba_batch* b, const double* E_n, const double* E_np1,
         double2* rho_n = c->rho_hist + n * NN;
         double2* rho_t = c->rho_hist + (n + 1) * NN;
         GKBA_TRY(diagnostics(c, E_n[i], rho_n, c->Ia, c->dscal));
-        GKBA_TRY(rhs(c, c->hhf_n, rho_n, c->Ia, c->k1));
-        GKBA_TRY(axpy_c(c, rho_t, rho_n, c->k1, 1.0, c->dt, (int)NN));
-        GKBA_CUDA(c, cudaMemcpyAsync(c->rhot_hist + n * NN, rho_t, NN * 16, cudaMemcpyDeviceToDevice,
-                                     c->stream));
+        GKBA_TRY(heun_stage(c, c->hhf_n, rho_n, c->Ia, rho_n, nullptr, c->dt, c->k1, rho_t, c->rhot_hist + n * NN));
         GKBA_TRY(h_hf(c, E_np1[i], rho_t, c->hhf_t));
-        GKBA_TRY(expm_step(c, c->hhf_n, c->hhf_t, c->U));
-        GKBA_CUDA(c, cudaMemcpyAsync(c->U_hist + n * NN, c->U, NN * 16, cudaMemcpyDeviceToDevice,
-                                     c->stream));
+        GKBA_TRY(expm_step(c, c->hhf_n, c->hhf_t, c->U, c->U_hist + n * NN));
         c->E_a[n] = E_n[i];
         c->E_b[n] = E_np1[i];
         GKBA_TRY(zgemm_batched(c, K_STEP, c->N, 'N', 'N', make_double2(1.0, 0.0), c->U, 0, c->T_a,
-                               NN, make_double2(0.0, 0.0), c->T_b, NN, n + 1, 0));
-        GKBA_TRY(set_identity(c, c->T_b + (n + 1) * NN, 1));
+                               NN, make_double2(0.0, 0.0), c->T_b, NN, n + 1, 1));
     }
     GKBA_TRY(batch_collision(b, 1));
     for (size_t i = 0; i < b->ctx.size(); ++i) {
@@ -1606,9 +1598,8 @@ gkba_status batch_step(gkba_batch* b, const double* E_n, const double* E_np1,
         const long long NN = (long long)c->N * c->N;
         double2* rho_n = c->rho_hist + n * NN;
         double2* rho_t = c->rho_hist + (n + 1) * NN;
-        GKBA_TRY(rhs(c, c->hhf_t, rho_t, c->Ib, c->k2));
-        GKBA_TRY(axpy_c(c, c->k2, c->k1, c->k2, 1.0, 1.0, (int)NN));
-        GKBA_TRY(axpy_c(c, rho_t, rho_n, c->k2, 1.0, 0.5 * c->dt, (int)NN));
+        GKBA_TRY(heun_stage(c, c->hhf_t, c->rhot_hist + n * NN, c->Ib, rho_n, c->k1, 0.5 * c->dt, nullptr, rho_t,
+                            nullptr));
         std::swap(c->T_a, c->T_b);
         c->n = n + 1;
         if (rho_out && rho_out[i])

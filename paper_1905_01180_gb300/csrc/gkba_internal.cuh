@@ -81,8 +81,8 @@ struct gkba_ctx {
 
     // FP64 contraction operands (natural N)
     double* wS64 = nullptr;  // [j][m][q][s] = w_mqsj
-    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn (null when vKimg holds its digits)
-    bool oz = false;         // stage GEMMs on the FP16 tensor cores (oz_gemm.cu)
+    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn, until vKimg holds its digits
+    bool oz = false;         // FP64 with a general v: digit images are needed (oz_gemm.cu)
     void* vKimg = nullptr;   // digit images of vK (oz)
 
     // split-TF32 contraction operands (padded Np, zero padding)
@@ -222,19 +222,18 @@ struct StageMap {
     long long XB = 0;  // nonzero: x enters as (x / 32) * XB + x % 32 (K-blocked layout)
 };
 
-// D[z][row][col] = sum_k A[z][row*lda + k] * B[z][col*ldb + k] (FP64, K-major).
-// Mode 0: z indexes units (per-z strides sAz, sBz, sOz; K = Ktot).
-// Mode 1: z indexes K-chunks of length Kc (split-K; out += z*sOz).
+// D[z][row][col] = sum_k A[z][row*lda + k] * B[z][col*ldb + k] (FP64, K-major),
+// z < nz units with per-z strides sAz, sBz, sOz (sBz = 0: one B for all), on the
+// FP16 tensor cores.
 gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz,
                          const double* B, long long ldb, long long sBz, double* out,
-                         long long sOz, int M, int Nc, long long Ktot, int nz, int splitk,
-                         long long Kc, StageMap map, double flops, double bytes);
-
-// The same GEMM on the FP16 tensor cores, FP64 in and out (oz_gemm.cu).  B is
-// given as digit images: oz_img_bytes(Nc, K) bytes per z, written by oz_slice.
+                         long long sOz, int M, int Nc, long long Ktot, int nz, StageMap map,
+                         double flops, double bytes);
+// Its parts (oz_gemm.cu).  B is given as digit images: oz_img_bytes(Nc, K) bytes per z, written by oz_slice.
 // K is split into nitem ranges of whole windows (out += item * sOitem);
 // oz_items proposes a number of them for M x Nc outputs, at most max_items.
 size_t oz_img_bytes(int Nc, long long K);
+size_t oz_img_bound(int Nc, long long K);  // of any K up to this one
 gkba_status oz_prepare(gkba_ctx* c);
 gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz, int Nc, long long K, int nz,
                      void* img);
@@ -242,28 +241,25 @@ int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items);
 gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const void* img,
                     int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
                     long long sOitem, StageMap map, double flops, double bytes);
-// Bases from which the FP64 stage GEMMs run there (a row tile holds 128 of N^3 rows).
-constexpr int kOzMinN = 6;
 // Stage S4 of the FP64 chain on the X3 of nb units in X13, with its reduction: S_u -> c->Su.
 gkba_status fp64_final(gkba_ctx* c, int nb);
 
-// Complex batched GEMM: C[b] = alpha * op(A[b]) * op(B[b]) + beta * C[b] (+ I if add_identity),
-// op = 'N' or 'C' (conjugate transpose); square n x n matrices, per-batch strides in elements.
-// K chunk (a multiple of the stage GEMM's K slice) of a split-K stage GEMM of
-// M x Nc outputs so that its launch fills about one wave of resident blocks,
-// with at most max_chunks chunks.
-long long gemm64_splitk_chunk(gkba_ctx* c, int M, int Nc, long long K, long long max_chunks);
+// Complex batched GEMM: C[b] = alpha op(A[b]) op(B[b]) + beta C[b], op = 'N' or 'C' (conjugate
+// transpose); square n x n matrices, per-batch strides in elements.  The n_ident matrices after
+// the batch in C are set to the identity.
 gkba_status zgemm_batched(gkba_ctx* c, int cls, int n, char opA, char opB, double2 alpha,
                           const double2* A, long long sA, const double2* B, long long sB,
-                          double2 beta, double2* C, long long sC, int batch, int add_identity);
+                          double2 beta, double2* C, long long sC, int batch, int n_ident);
 
 // Stepper helpers.
 gkba_status mean_field(gkba_ctx* c, const double2* rho, double2* out);
 gkba_status h_hf(gkba_ctx* c, double E, const double2* rho, double2* out);  // h + E d + Sigma_HF
-gkba_status rhs(gkba_ctx* c, const double2* hhf, const double2* rho, const double2* I,
-                double2* out);  // -i[hhf, rho] - (I + I^+)
-gkba_status expm_step(gkba_ctx* c, const double2* hA, const double2* hB,
-                      double2* U);  // U = exp(-i dt (hA + hB)/2)
+// One Heun stage: k = -i[hhf, rho] - (I + I^+) (to k_out unless null), y = base + a (k + kprev)
+// (kprev may be null), y also to y2 unless null.  y must not alias rho.
+gkba_status heun_stage(gkba_ctx* c, const double2* hhf, const double2* rho, const double2* I, const double2* base,
+                       const double2* kprev, double a, double2* k_out, double2* y, double2* y2);
+// U = exp(-i dt (hA + hB)/2), also to U2 unless null.
+gkba_status expm_step(gkba_ctx* c, const double2* hA, const double2* hB, double2* U, double2* U2);
 gkba_status axpy_c(gkba_ctx* c, double2* y, const double2* x, const double2* z, double a,
                    double b, int n);  // y = a*x + b*z (elementwise, n complex)
 gkba_status set_identity(gkba_ctx* c, double2* A, int count);  // count N*N identities

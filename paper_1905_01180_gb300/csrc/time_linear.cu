@@ -142,7 +142,7 @@ gkba_status tl_terms(gkba_ctx* c, int nk, const double2* rho, const double2* W, 
     // stored as [j2][n][r][c2][p]
     const StageMap md{2 * N2, 2 * N, 1, N, 2 * N3, N, N, N};
     return gemm64_stage(c, K_TL, (const double*)c->X13, K, 0, M, K, 0, (double*)c->X2, 0,
-                        (int)N3, 2 * N, K, 1, 0, 0, md, 2.0 * N3 * 2 * N * K,
+                        (int)N3, 2 * N, K, 1, md, 2.0 * N3 * 2 * N * K,
                         8.0 * (N3 * K + 2 * N4));
 }
 
@@ -177,13 +177,13 @@ gkba_status tl_apply(gkba_ctx* c, const double2* W, double2* I_out) {
     // x_n with Ucal: rows (j, r, p) of X2 -> tl_s [j][p][n][(c, r)] (same scatter)
     const StageMap mrot{2 * N3, 1, 2 * N2, N, 2 * N, N, N, N};
     GKBA_TRY(gemm64_stage(c, K_TL, c->tl_s, 2 * N, 0, Ur, 2 * N, 0, X2, 0, (int)N3, 2 * N, 2 * N,
-                          1, 0, 0, mrot, fl, by));
+                          1, mrot, fl, by));
     GKBA_TRY(gemm64_stage(c, K_TL, X2, 2 * N, 0, Ur, 2 * N, 0, c->tl_s, 0, (int)N3, 2 * N, 2 * N,
-                          1, 0, 0, mrot, fl, by));
+                          1, mrot, fl, by));
     // x_r with conj(Ucal): rows (j, p, n) of tl_s -> X13 as X3 [c][j][n][r][p]
     const StageMap mx3{N3, 1, N2, N4, N, N, N, N};
     GKBA_TRY(gemm64_stage(c, K_TL, c->tl_s, 2 * N, 0, Urc, 2 * N, 0, X13, 0, (int)N3, 2 * N, 2 * N,
-                          1, 0, 0, mx3, fl, by));
+                          1, mx3, fl, by));
     GKBA_TRY(fp64_final(c, 1));  // stage S4 on one unit
     // I = S Ucal^+ = S W
     return zgemm_batched(c, K_RED, N, 'N', 'N', make_double2(1.0, 0.0), c->Su, 0, W, 0,

@@ -36,7 +36,7 @@ def setup(P, N, U, seed=3):
     return s, ctx, np.stack([p[0] for p in pairs]), np.stack([p[1] for p in pairs])
 
 
-@pytest.mark.parametrize("N,U", [(5, 3), (6, 1), (6, 5), (8, 3), (9, 2), (16, 3), (17, 2), (24, 5), (32, 2),
+@pytest.mark.parametrize("N,U", [(1, 3), (2, 2), (4, 40), (5, 3), (6, 1), (6, 5), (8, 3), (9, 2), (16, 3), (17, 2), (24, 5), (32, 2),
                                  (33, 1), (40, 2), (48, 1), (49, 2), (64, 1)])
 def test_sigma_edges(P, N, U):
     s, ctx, G, Gb = setup(P, N, U)
