@@ -287,7 +287,13 @@ gkba_status collision_vjp_dev(gkba_ctx* c, int L, const double2* rho, const doub
                               double2* T_bar, double* vslot, double* wslot) {
     const int N = c->N;
     const long long NN = (long long)N * N;
-    GKBA_TRY(ensure_workspace(c, 2 * L));
+    // A short history leaves the SMs idle in each of the four chains of a chunk: the
+    // three slot derivatives then run as one batch of three times the units (N = 13,
+    // 18 units: 16 + 4 launches instead of 32 + 8).  Long ones gain nothing from it.
+    const long long rows = 2LL * L * NN * N;
+    const bool merge = rows < 16LL * 128 * c->num_sms;
+    GKBA_TRY(ensure_workspace(c, (merge ? 6 : 2) * L));
+    const bool one_batch = merge && c->ub >= 6 * L;
     if (c->vjp_units < c->ub) {
         if (c->vjp) cudaFree(c->vjp);
         c->vjp = nullptr;
@@ -332,17 +338,36 @@ gkba_status collision_vjp_dev(gkba_ctx* c, int L, const double2* rho, const doub
             GKBA_TRY(fp64_chain_x3(c, nb, c->vomega));
             GKBA_TRY(vbar_slot(c, nb, Sbv, 1, (const double*)c->X13, wslot));
         }
-        GKBA_TRY(unit_xform(c, nb, Gv, tA, 1, 0));   // G*
-        GKBA_TRY(unit_xform(c, nb, Sbv, tB, 0, 1));  // Sbar^T
-        GKBA_TRY(contract3(c, nb, tA, tB, tA));
-        GKBA_TRY(unit_acc(c, nb, Gbb, c->Su, 1));
-        GKBA_TRY(unit_xform(c, nb, Gv, tB, 1, 1));   // G*^T
-        GKBA_TRY(unit_xform(c, nb, Gbv, tC, 1, 1));  // Gb*^T
-        GKBA_TRY(contract3(c, nb, Sbv, tB, tC));
-        GKBA_CUDA(c, cudaMemcpyAsync(Gbr, c->Su, nb * NN * sizeof(double2), cudaMemcpyDeviceToDevice,
-                                     c->stream));
-        GKBA_TRY(contract3(c, nb, tC, tB, Sbv));
-        GKBA_TRY(unit_acc(c, nb, Gbr, c->Su, 0));
+        if (one_batch) {
+            // blocks tA, tB, tC hold three units' worth each (3 nb <= ub)
+            const long long n1 = nb * NN;
+            GKBA_TRY(unit_xform(c, nb, Gv, tA, 1, 0));             // A: G*, Sbar, Gb*^T
+            GKBA_TRY(unit_xform(c, nb, Sbv, tA + n1, 0, 0));
+            GKBA_TRY(unit_xform(c, nb, Gbv, tA + 2 * n1, 1, 1));
+            GKBA_TRY(unit_xform(c, nb, Sbv, tB, 0, 1));            // B: Sbar^T, G*^T, G*^T
+            GKBA_TRY(unit_xform(c, nb, Gv, tB + n1, 1, 1));
+            GKBA_TRY(unit_xform(c, nb, Gv, tB + 2 * n1, 1, 1));
+            GKBA_TRY(unit_xform(c, nb, Gv, tC, 1, 0));             // C: G*, Gb*^T, Sbar
+            GKBA_TRY(unit_xform(c, nb, Gbv, tC + n1, 1, 1));
+            GKBA_TRY(unit_xform(c, nb, Sbv, tC + 2 * n1, 0, 0));
+            GKBA_TRY(contract3(c, 3 * nb, tA, tB, tC));
+            GKBA_TRY(unit_acc(c, nb, Gbb, c->Su, 1));
+            GKBA_TRY(unit_acc(c, nb, c->Su + n1, c->Su + 2 * n1, 0));
+            GKBA_CUDA(c, cudaMemcpyAsync(Gbr, c->Su + n1, n1 * sizeof(double2), cudaMemcpyDeviceToDevice,
+                                         c->stream));
+        } else {
+            GKBA_TRY(unit_xform(c, nb, Gv, tA, 1, 0));   // G*
+            GKBA_TRY(unit_xform(c, nb, Sbv, tB, 0, 1));  // Sbar^T
+            GKBA_TRY(contract3(c, nb, tA, tB, tA));
+            GKBA_TRY(unit_acc(c, nb, Gbb, c->Su, 1));
+            GKBA_TRY(unit_xform(c, nb, Gv, tB, 1, 1));   // G*^T
+            GKBA_TRY(unit_xform(c, nb, Gbv, tC, 1, 1));  // Gb*^T
+            GKBA_TRY(contract3(c, nb, Sbv, tB, tC));
+            GKBA_CUDA(c, cudaMemcpyAsync(Gbr, c->Su, nb * NN * sizeof(double2), cudaMemcpyDeviceToDevice,
+                                         c->stream));
+            GKBA_TRY(contract3(c, nb, tC, tB, Sbv));
+            GKBA_TRY(unit_acc(c, nb, Gbr, c->Su, 0));
+        }
         GKBA_TRY(vjp_points(c, nk, Gbr, Gbb, tA, tB));  // Pbar, Qbar
         GKBA_TRY(axpy_c(c, D, tA, tB, 1.0, -1.0, (int)(nk * NN)));
         GKBA_TRY(zgemm_batched(c, K_RED, N, 'C', 'N', one, T + k0 * NN, NN, D, NN, zero,
