@@ -84,6 +84,7 @@ struct OzParams {
     int nitem, wper;     // split K: items per row tile, windows per item
     long long sOitem;
     long long tiles;     // z x item x row tile
+    uint32_t mma_id[kOzSlices], mma_col[kOzSlices];  // per digit of A: instruction descriptor, accumulator column
     OzMul mul;
     int na, nbs;         // A and B pipeline stages
     int* err;
@@ -202,15 +203,17 @@ __device__ __forceinline__ bool oz_warp_wait(uint32_t bar, uint32_t parity, vola
 }
 
 // D[tmem] (+)= A[smem] B[smem], M = 128, K = 16, FP16 in, FP32 out; issued by
-// one elected lane of a converged warp.
-__device__ __forceinline__ void oz_mma(uint32_t d, unsigned long long ad, unsigned long long bd, uint32_t idesc,
-                                       uint32_t accumulate) {
+// one elected lane of a converged warp.  ad and bd are the low words of the
+// operand descriptors, the only ones that differ.
+__device__ __forceinline__ void oz_mma(uint32_t d, uint32_t ad, uint32_t bd, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %5};\n\t"
+        "mov.b64 b, {%2, %5};\n\t"
         "elect.sync _|e, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}" ::"r"(d),
+        "r"(ad), "r"(bd), "r"(idesc), "r"(accumulate), "n"((128 >> 4) | (1 << 14))
         : "memory");
 }
 __device__ __forceinline__ void oz_commit(uint32_t bar) {
@@ -233,10 +236,10 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
                  : "memory");
 }
 // K-major operand without swizzle: core matrices of 8 rows x 16 bytes, lbo
-// bytes apart along K, 128 bytes apart along the rows.
-__device__ __forceinline__ unsigned long long desc_plain(uint32_t saddr, uint32_t lbo) {
-    return (unsigned long long)((saddr & 0x3FFFFu) >> 4) | (unsigned long long)(lbo >> 4) << 16 |
-           (unsigned long long)(128 >> 4) << 32 | 1ull << 46;
+// bytes apart along K, 128 bytes apart along the rows.  The low word of the
+// descriptor (the high one is the row distance and the version).
+__device__ __forceinline__ uint32_t desc_plain(uint32_t saddr, uint32_t lbo) {
+    return ((saddr & 0x3FFFFu) >> 4) | (lbo >> 4) << 16;
 }
 
 // Position of a tile in a CTA's range (row tiles fastest, then split-K items,
@@ -275,7 +278,12 @@ __device__ __forceinline__ int oz_chunks(const OzParams& p, int w) {
 }
 
 // Register split of the one-window kernel (28 warps, 72 registers a thread at
-// launch): 16 x 64 + 8 x 104 + 4 x 40 = 28 x 72.
+// launch): 16 x 64 + 8 x 104 + 4 x 40 = 28 x 72, each by the whole of a warpgroup.
+// Other splits of the same kernel are slower (us per self-energy at N = 32 and
+// 33; this one 37.9 and 70.1): 56 / 104 / 72 41.9 and 77.2, 8 epilogue warps 42.1
+// and 78.5, 8 + 16 warps of 88 / 72 40.9 and 75.7.  The auxiliary warps live with
+// 40 because the MMA role keeps its per-digit operands among the parameters, its
+// descriptors in one word each and its stages as counters.
 template <int N>
 __device__ __forceinline__ void regs_dec() {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
@@ -610,102 +618,106 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
             }
             if (t < ntile) load();
         }
-    } else if (warp == kWorkers) {
+    } else {
         if (!MULTI) regs_dec<40>();
-        if (lane == 0) {
-            // ---------------- producer of B's digit images ----------------
-            uint32_t bseq = 0, accseq = 0;
+        if (warp == kWorkers) {
+            if (lane == 0) {
+                // ---------------- producer of B's digit images ----------------
+                uint32_t bseq = 0, accseq = 0;
+                bool ok = true;
+                for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
+                    const int nacc = MULTI ? p.nblk * T.nw : p.nblk;
+                    int blk = 0, wi = 0;
+                    for (int a = 0; a < nacc && ok; ++a, ++accseq) {
+                        const int w = T.w0 + wi;
+                        const int no = oz_chunks<NO, MULTI>(p, w);
+                        const uint8_t* src = p.img + T.z * p.img_z + ((long long)w * p.nblk + blk) * NO * brow;
+                        for (int c0 = 0; c0 < no; c0 += kOzSub, ++bseq) {
+                            const int st = (int)(bseq % (uint32_t)p.nbs);
+                            if (!oz_wait(bar(BEMPTY + st), ((bseq / (uint32_t)p.nbs) & 1) ^ 1, abort_flag, p.err, 43, 300)) {
+                                ok = false;
+                                break;
+                            }
+                            const uint32_t bytes = (uint32_t)min(kOzSub, no - c0) * brow;
+                            mbar_expect_tx(bar(BFULL + st), bytes + (c0 == 0 ? p.NB * 4u : 0u));
+                            if (c0 == 0)
+                                bulk_load(smem_u32(sEcol + (accseq % kOzRing) * kOzMaxNB),
+                                          p.ecol + T.z * p.ecol_z + ((long long)w * p.nblk + blk) * p.NB, p.NB * 4u,
+                                          bar(BFULL + st));
+                            bulk_load(smem_u32(sB + (size_t)st * bstage), src + (size_t)c0 * brow, bytes, bar(BFULL + st));
+                        }
+                        if (!MULTI || ++wi == T.nw) {
+                            wi = 0;
+                            ++blk;
+                        }
+                    }
+                }
+                if (*abort_flag) {
+                    // copies in flight must land before the CTA leaves
+                    for (uint32_t st = 0; st < (uint32_t)p.nbs; ++st) {
+                        if (bseq > st) {
+                            const uint32_t last = bseq - 1 - ((bseq - 1 - st) % (uint32_t)p.nbs);
+                            const unsigned long long g0 = gtimer();
+                            while (!mbar_try(bar(BFULL + st), (last / (uint32_t)p.nbs) & 1) && gtimer() - g0 < kWaitLimitNs) {}
+                        }
+                    }
+                }
+            }
+        } else if (warp == kWorkers + 1) {
+            // ---------------- MMA issuer ----------------
+            // stage counters with their phases: few registers, no divisions
+            uint32_t as = 0, aph = 0, st = 0, bph = 0, accseq = 0;
+            const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
             bool ok = true;
             for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
-                const int nacc = MULTI ? p.nblk * T.nw : p.nblk;
-                int blk = 0, wi = 0;
-                for (int a = 0; a < nacc && ok; ++a, ++accseq) {
-                    const int w = T.w0 + wi;
-                    const int no = oz_chunks<NO, MULTI>(p, w);
-                    const uint8_t* src = p.img + T.z * p.img_z + ((long long)w * p.nblk + blk) * NO * brow;
-                    for (int c0 = 0; c0 < no; c0 += kOzSub, ++bseq) {
-                        const int st = (int)(bseq % (uint32_t)p.nbs);
-                        if (!oz_wait(bar(BEMPTY + st), ((bseq / (uint32_t)p.nbs) & 1) ^ 1, abort_flag, p.err, 43, 300)) {
-                            ok = false;
-                            break;
-                        }
-                        const uint32_t bytes = (uint32_t)min(kOzSub, no - c0) * brow;
-                        mbar_expect_tx(bar(BFULL + st), bytes + (c0 == 0 ? p.NB * 4u : 0u));
-                        if (c0 == 0)
-                            bulk_load(smem_u32(sEcol + (accseq % kOzRing) * kOzMaxNB),
-                                      p.ecol + T.z * p.ecol_z + ((long long)w * p.nblk + blk) * p.NB, p.NB * 4u,
-                                      bar(BFULL + st));
-                        bulk_load(smem_u32(sB + (size_t)st * bstage), src + (size_t)c0 * brow, bytes, bar(BFULL + st));
-                    }
-                    if (!MULTI || ++wi == T.nw) {
-                        wi = 0;
-                        ++blk;
-                    }
-                }
-            }
-            if (*abort_flag) {
-                // copies in flight must land before the CTA leaves
-                for (uint32_t st = 0; st < (uint32_t)p.nbs; ++st) {
-                    if (bseq > st) {
-                        const uint32_t last = bseq - 1 - ((bseq - 1 - st) % (uint32_t)p.nbs);
-                        const unsigned long long g0 = gtimer();
-                        while (!mbar_try(bar(BFULL + st), (last / (uint32_t)p.nbs) & 1) && gtimer() - g0 < kWaitLimitNs) {}
-                    }
-                }
-            }
-        }
-    } else if (!MULTI && warp > kWorkers + 1) {
-        regs_dec<40>();
-    } else {
-        // ---------------- MMA issuer ----------------
-        if (!MULTI) regs_dec<40>();
-        uint32_t aseq = 0, bseq = 0, accseq = 0;
-        bool ok = true;
-        for (int t = 0; t < ntile && ok; ++t, T.next(p)) {
-            const int nouter = MULTI ? p.nblk * T.nw : 1, ninner = MULTI ? 1 : p.nblk;
-            int wi = 0;
-            for (int ao = 0; ao < nouter && ok; ++ao, ++aseq) {
-                const int no = oz_chunks<NO, MULTI>(p, T.w0 + wi);
-                if (MULTI && ++wi == T.nw) wi = 0;
-                const int as = p.na == 2 ? (int)(aseq & 1) : 0;
-                const uint32_t aph = (p.na == 2 ? aseq >> 1 : aseq) & 1;
-                if (!oz_warp_wait(bar(AFULL + as), aph, abort_flag, p.err, 44)) { ok = false; break; }
-                const unsigned long long ad = desc_plain(smem_u32(sA + (size_t)as * kAStage), kOzLbo);
-                for (int bi = 0; bi < ninner && ok; ++bi, ++accseq) {
-                    const int ab = (int)(accseq & 1);
-                    if (!oz_warp_wait(bar(ACCE + ab), ((accseq >> 1) & 1) ^ 1, abort_flag, p.err, 45)) { ok = false; break; }
-                    const uint32_t acc = tmem + (uint32_t)(ab * 256);
-                    for (int c0 = 0; c0 < no; c0 += kOzSub, ++bseq) {
-                        const int st = (int)(bseq % (uint32_t)p.nbs);
-                        if (!oz_warp_wait(bar(BFULL + st), (bseq / (uint32_t)p.nbs) & 1, abort_flag, p.err, 46)) { ok = false; break; }
-                        tc_fence_after();
-                        const unsigned long long bd = desc_plain(smem_u32(sB + (size_t)st * bstage), brow);
-                        const int ns = min(kOzSub, no - c0) / 2;
+                const int nouter = MULTI ? p.nblk * T.nw : 1, ninner = MULTI ? 1 : p.nblk;
+                int wi = 0;
+                for (int ao = 0; ao < nouter && ok; ++ao) {
+                    const int no = oz_chunks<NO, MULTI>(p, T.w0 + wi);
+                    if (MULTI && ++wi == T.nw) wi = 0;
+                    if (!oz_warp_wait(bar(AFULL + as), aph, abort_flag, p.err, 44)) { ok = false; break; }
+                    for (int bi = 0; bi < ninner && ok; ++bi, ++accseq) {
+                        const int ab = (int)(accseq & 1);
+                        if (!oz_warp_wait(bar(ACCE + ab), ((accseq >> 1) & 1) ^ 1, abort_flag, p.err, 45)) { ok = false; break; }
+#pragma unroll 1
+                        for (int c0 = 0; c0 < no; c0 += kOzSub) {
+                            if (!oz_warp_wait(bar(BFULL + st), bph, abort_flag, p.err, 46)) { ok = false; break; }
+                            tc_fence_after();
+                            const uint32_t ad = desc_plain(sA0 + as * kAStage + (uint32_t)c0 * kOzLbo, kOzLbo);
+                            const uint32_t bd = desc_plain(sB0 + st * bstage, brow);
+                            const uint32_t acc = tmem + (uint32_t)(ab * 256);
+                            const int ns = min(kOzSub, no - c0) / 2;
 #pragma unroll
-                        for (int i = 0; i < kOzSlices; ++i) {
-                            // digits of B this digit of A meets (digit 0's first step also
-                            // meets the zero rows, clearing level 7)
-                            const int cnt = i == 0 ? 8 : min(kOzSlices, kOzLevels - i);
-                            const uint32_t n = (uint32_t)((cnt * p.NB + 15) & ~15);
-                            const uint32_t id = (1u << 4) | ((n >> 3) << 17) | ((uint32_t)(kOzBM >> 4) << 24);
-                            for (int ks = 0; ks < ns; ++ks)
-                                oz_mma(acc + (uint32_t)(i * p.NB),
-                                       ad + (((unsigned long long)i * kPlane + (unsigned long long)(c0 + 2 * ks) * kOzLbo) >> 4),
-                                       bd + (((unsigned long long)(2 * ks) * brow) >> 4), id, (c0 | i | ks) ? 1u : 0u);
+                            for (int i = 0; i < kOzSlices; ++i) {
+                                // digits of B this digit of A meets (digit 0's first step also
+                                // meets the zero rows, clearing level 7)
+#pragma unroll 1
+                                for (int ks = 0; ks < ns; ++ks)
+                                    oz_mma(acc + p.mma_col[i], ad + (i * kPlane >> 4) + (uint32_t)ks * (2 * kOzLbo >> 4),
+                                           bd + (uint32_t)ks * (brow >> 3), p.mma_id[i], (c0 | i | ks) ? 1u : 0u);
+                            }
+                            oz_commit(bar(BEMPTY + st));
+                            if (++st == (uint32_t)p.nbs) {
+                                st = 0;
+                                bph ^= 1;
+                            }
                         }
-                        oz_commit(bar(BEMPTY + st));
+                        if (!ok) break;
+                        oz_commit(bar(ACCF + ab));
                     }
                     if (!ok) break;
-                    oz_commit(bar(ACCF + ab));
+                    oz_commit(bar(AEMPTY + as));
+                    if (++as == (uint32_t)p.na) {
+                        as = 0;
+                        aph ^= 1;
+                    }
                 }
-                if (!ok) break;
-                oz_commit(bar(AEMPTY + as));
             }
+            // closing commit: no MMA reads this CTA's memory after it
+            oz_commit(bar(DRAIN));
+            const unsigned long long g0 = gtimer();
+            while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
         }
-        // closing commit: no MMA reads this CTA's memory after it
-        oz_commit(bar(DRAIN));
-        const unsigned long long g0 = gtimer();
-        while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
     }
     tc_fence_before();
     __syncthreads();
@@ -823,6 +835,12 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
     if (p.nitem != nitem) return fail(c, GKBA_EINVAL, "oz_gemm: %d items for %d windows", nitem, g.nwin);
     p.sOitem = sOitem;
     p.mul = kOzMul;
+    for (int i = 0; i < kOzSlices; ++i) {
+        const int cnt = i == 0 ? 8 : std::min(kOzSlices, kOzLevels - i);
+        const uint32_t n = (uint32_t)((cnt * p.NB + 15) & ~15);
+        p.mma_id[i] = (1u << 4) | ((n >> 3) << 17) | ((uint32_t)(kOzBM >> 4) << 24);
+        p.mma_col[i] = (uint32_t)(i * p.NB);
+    }
     p.tiles = (long long)nz * p.nitem * p.mtiles;
     if (p.tiles >= 1LL << 31) return fail(c, GKBA_EINVAL, "oz_gemm: %lld tiles", p.tiles);
     p.err = c->dint + 1;
