@@ -108,9 +108,9 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v
 __device__ __forceinline__ uint32_t smem_pad1024(const void* p) { return (0u - smem_u32(p)) & 1023u; }
 // Bounded wait of the CTA-pair kernel; on timeout it raises this CTA's and the
 // peer CTA's abort flags (peer_abort: shared::cluster address).
-__device__ bool mbar_wait_cl(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                             uint32_t peer_abort, int* err, int code,
-                             unsigned long long limit_ns = kWaitLimitNs) {
+__device__ __forceinline__ bool mbar_wait_cl(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                             uint32_t peer_abort, int* err, int code,
+                                             unsigned long long limit_ns = kWaitLimitNs) {
     if (mbar_try(bar, parity)) return true;
     const unsigned long long t0 = gtimer();
     for (uint32_t it = 1;; ++it) {
@@ -331,7 +331,7 @@ struct StageParams {
     StageMap map;
     int* err;
     int wsteps;        // 0: one accumulator per tile; 1 or 2: windows of that many K steps
-    int nring;         // windowed: accumulators in the ring (<= kStageRing)
+    int nring;         // windowed: accumulators of both rings (even, <= kStageRing)
     int as2;           // windowed: ring stride in columns (2 Np rounded up to 32)
     int astages;       // A pipeline stages (4 .. kStageAStagesMax, set with the shared memory)
 };
@@ -368,7 +368,20 @@ constexpr int kStageAStagesMax = 8;
 // dynamic shared memory of one CTA
 constexpr size_t kStageSmemMax = 227 * 1024;
 constexpr int kStageRing = 8;
-constexpr int kStageThreads = 384;  // warp 0 TMA, warp 1 MMA, 4-7 converter, 8-11 epilogue
+// warp 0 TMA, warp 1 MMA, 2 B relay, 4-7 converter, 8-11 and 12-15 epilogue
+constexpr int kStageThreads = 512;
+// Register split of the warpgroups (128 a thread at launch, 4 x 128 in all): the
+// windowed epilogue keeps 96 sums.
+constexpr int kStageRegsIssue = 64, kStageRegsConv = 104, kStageRegsEpi = 168;
+static_assert(kStageRegsIssue + kStageRegsConv + 2 * kStageRegsEpi <= 4 * 128, "register split");
+template <int N>
+__device__ __forceinline__ void stage_regs_dec() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void stage_regs_inc() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
 
 // ---------------------------------------------------------------------------
 // Stages S1-S3 on CTA pairs (cta_group::2).  A cluster of two CTAs on two SMs
@@ -496,224 +509,234 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
     const long long t0 = total * cid / ncl;
     const long long t1 = total * (cid + 1) / ncl;
 
-    if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer (both CTAs) ----------------
-            int cur_u = -1;
-            uint32_t bph = 0;
-            long long it = 0;
-            Ring ar(nas);  // A stage and its phase
-            bool ok = true, loaded_b = false;
-            for (long long t = t0; t < t1 && ok; ++t) {
-                const int u = (int)((uint32_t)t / ipu32);
-                const long long row0 = (long long)((uint32_t)t % ipu32) * (2 * kBM) + (long long)rank * kBM;
-                if (u != cur_u) {
-                    if (cur_u >= 0) {
-                        if (!mbar_wait_cl(bar(BEMPTY), bph, abort_flag, peer_abort, p.err, 1)) { ok = false; break; }
-                        bph ^= 1;
+    // each warpgroup sets its register share before its roles branch
+    if (warp < 4) {
+        stage_regs_dec<kStageRegsIssue>();
+        if (warp == 0) {
+            if (lane == 0) {
+                // ---------------- TMA producer (both CTAs) ----------------
+                int cur_u = -1;
+                uint32_t bph = 0;
+                long long it = 0;
+                Ring ar(nas);  // A stage and its phase
+                bool ok = true, loaded_b = false;
+                for (long long t = t0; t < t1 && ok; ++t) {
+                    const int u = (int)((uint32_t)t / ipu32);
+                    const long long row0 = (long long)((uint32_t)t % ipu32) * (2 * kBM) + (long long)rank * kBM;
+                    if (u != cur_u) {
+                        if (cur_u >= 0) {
+                            if (!mbar_wait_cl(bar(BEMPTY), bph, abort_flag, peer_abort, p.err, 1)) { ok = false; break; }
+                            bph ^= 1;
+                        }
+                        mbar_expect_tx(bar(BFULL), 2u * nchunk * chunkB);
+                        for (int c = 0; c < nchunk; ++c) {
+                            const int pl = c / p.kch, kc = c % p.kch;
+                            const int y = (pl * 2 + (int)rank) * Np;
+                            tma_3d(smem_u32(sBhi + c * chunkB), tmBhi, bar(BFULL), kc * kKC, y, u);
+                            tma_3d(smem_u32(sBlo + c * chunkB), tmBlo, bar(BFULL), kc * kKC, y, u);
+                        }
+                        loaded_b = true;
+                        cur_u = u;
                     }
-                    mbar_expect_tx(bar(BFULL), 2u * nchunk * chunkB);
-                    for (int c = 0; c < nchunk; ++c) {
-                        const int pl = c / p.kch, kc = c % p.kch;
-                        const int y = (pl * 2 + (int)rank) * Np;
-                        tma_3d(smem_u32(sBhi + c * chunkB), tmBhi, bar(BFULL), kc * kKC, y, u);
-                        tma_3d(smem_u32(sBlo + c * chunkB), tmBlo, bar(BFULL), kc * kKC, y, u);
-                    }
-                    loaded_b = true;
-                    cur_u = u;
-                }
-                for (int c = 0; c < nchunk && ok; ++c, ++it) {
-                    const int pl = c / p.kch, kc = c % p.kch;
-                    const int s = ar.i;
-                    const uint32_t ph = ar.ph;
-                    ar.next();
-                    if (!mbar_wait_cl(bar(AEMPTY + s), ph ^ 1, abort_flag, peer_abort, p.err, 2)) { ok = false; break; }
-                    mbar_expect_tx(bar(AFULL + s), kTileBytes);
-                    const uint32_t dst = smem_u32(sA + s * kTileBytes);
-                    if (p.a_unit) tma_4d(dst, tmA, bar(AFULL + s), kc * kKC, pl, (int)row0, u);
-                    else if (p.unit_sys) tma_3d(dst, tmA, bar(AFULL + s), kc * kKC, (int)row0, p.unit_sys[u]);
-                    else tma_2d(dst, tmA, bar(AFULL + s), kc * kKC, (int)row0);
-                }
-            }
-            if (*abort_flag) {
-                for (int s = 0; s < nas; ++s) {
-                    if (it > s) {
-                        const long long last = it - 1 - ((it - 1 - s) % nas);
-                        const uint32_t ph = (uint32_t)((last / nas) & 1);
-                        const unsigned long long g0 = gtimer();
-                        while (!mbar_try(bar(AFULL + s), ph) && gtimer() - g0 < kWaitLimitNs) {}
-                    }
-                }
-                if (loaded_b) {
-                    const unsigned long long g0 = gtimer();
-                    while (!mbar_try(bar(BFULL), bph) && gtimer() - g0 < kWaitLimitNs) {}
-                }
-            }
-        }
-    } else if (warp == 1) {
-        if (rank == 0) {
-            // ---------------- MMA issuer (even CTA, for the pair) ----------------
-            const uint32_t id = idesc_tf32_pair(2 * Np);
-            const unsigned long long dBhi0 = desc_sw128(smem_u32(sBhi));
-            const unsigned long long dBlo0 = desc_sw128(smem_u32(sBlo));
-            int cur_u = -1;
-            uint32_t bfph = 0;
-            long long it = 0, tile_i = 0;
-            Ring wr(p.nring > 0 ? p.nring : 1);
-            bool ok = true, issued = false;
-            for (long long t = t0; t < t1 && ok; ++t, ++tile_i) {
-                const int u = (int)((uint32_t)t / ipu32);
-                if (u != cur_u) {
-                    if (!warp_wait_cl(bar(BFULL), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
-                    if (!warp_wait_cl(bar(BPEER), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
-                    bfph ^= 1;
-                    cur_u = u;
-                    tc_fence_after();
-                }
-                if (win) {
-                    // Windowed accumulation: every wsteps K steps go to the next
-                    // accumulator of a ring that the epilogue drains into FP32
-                    // register sums; inside a window the correction products come
-                    // first, while the accumulator is still small, then hi*hi.
-                    int kc = 0;
                     for (int c = 0; c < nchunk && ok; ++c, ++it) {
+                        const int pl = c / p.kch, kc = c % p.kch;
+                        const int s = ar.i;
+                        const uint32_t ph = ar.ph;
+                        ar.next();
+                        if (!mbar_wait_cl(bar(AEMPTY + s), ph ^ 1, abort_flag, peer_abort, p.err, 2)) { ok = false; break; }
+                        mbar_expect_tx(bar(AFULL + s), kTileBytes);
+                        const uint32_t dst = smem_u32(sA + s * kTileBytes);
+                        if (p.a_unit) tma_4d(dst, tmA, bar(AFULL + s), kc * kKC, pl, (int)row0, u);
+                        else if (p.unit_sys) tma_3d(dst, tmA, bar(AFULL + s), kc * kKC, (int)row0, p.unit_sys[u]);
+                        else tma_2d(dst, tmA, bar(AFULL + s), kc * kKC, (int)row0);
+                    }
+                }
+                if (*abort_flag) {
+                    for (int s = 0; s < nas; ++s) {
+                        if (it > s) {
+                            const long long last = it - 1 - ((it - 1 - s) % nas);
+                            const uint32_t ph = (uint32_t)((last / nas) & 1);
+                            const unsigned long long g0 = gtimer();
+                            while (!mbar_try(bar(AFULL + s), ph) && gtimer() - g0 < kWaitLimitNs) {}
+                        }
+                    }
+                    if (loaded_b) {
+                        const unsigned long long g0 = gtimer();
+                        while (!mbar_try(bar(BFULL), bph) && gtimer() - g0 < kWaitLimitNs) {}
+                    }
+                }
+            }
+        } else if (warp == 1) {
+            if (rank == 0) {
+                // ---------------- MMA issuer (even CTA, for the pair) ----------------
+                const uint32_t id = idesc_tf32_pair(2 * Np);
+                const unsigned long long dBhi0 = desc_sw128(smem_u32(sBhi));
+                const unsigned long long dBlo0 = desc_sw128(smem_u32(sBlo));
+                int cur_u = -1;
+                uint32_t bfph = 0;
+                long long it = 0, tile_i = 0;
+                // the epilogue groups' rings: tiles alternate between them
+                Ring wr0(p.nring > 1 ? p.nring / 2 : 1), wr1 = wr0;
+                bool ok = true, issued = false;
+                for (long long t = t0; t < t1 && ok; ++t, ++tile_i) {
+                    const int u = (int)((uint32_t)t / ipu32);
+                    if (u != cur_u) {
+                        if (!warp_wait_cl(bar(BFULL), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
+                        if (!warp_wait_cl(bar(BPEER), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
+                        bfph ^= 1;
+                        cur_u = u;
+                        tc_fence_after();
+                    }
+                    if (win) {
+                        // Windowed accumulation: every wsteps K steps go to the next
+                        // accumulator of a ring that the epilogue drains into FP32
+                        // register sums; inside a window the correction products come
+                        // first, while the accumulator is still small, then hi*hi.
+                        int kc = 0;
+                        for (int c = 0; c < nchunk && ok; ++c, ++it) {
+                            const int slot = (int)(it & 1);
+                            const uint32_t sph = (uint32_t)((it >> 1) & 1);
+                            if (!warp_wait_cl(bar(TFULL + slot), sph, abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
+                            tc_fence_after();
+                            const uint32_t ahi = tmem + (slot ? slot_col1 : slot_col0);
+                            const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
+                            const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
+                            const int ksteps = kc == p.kch - 1 ? ktail : 4;
+                            if (++kc == p.kch) kc = 0;
+                            for (int kw = 0; kw < ksteps; kw += p.wsteps) {
+                                const bool g1 = (tile_i & 1) != 0;
+                                const int b = g1 ? wr1.i + wr1.n : wr0.i;
+                                const uint32_t wph = g1 ? wr1.ph : wr0.ph;
+                                if (g1) wr1.next();
+                                else wr0.next();
+                                if (!warp_wait_cl(bar(WE + b), wph ^ 1u, abort_flag, peer_abort, p.err, 19)) { ok = false; break; }
+                                tc_fence_after();
+                                const uint32_t dw = tmem + 128u + (uint32_t)(b * p.as2);
+#pragma unroll 1
+                                for (int kk = kw; kk < kw + p.wsteps; ++kk) {
+                                    mma_tf32_pair(dw, ahi + kk * 8, dl + 2ull * kk, id, kk == kw ? 0u : 1u);
+                                    mma_tf32_pair(dw, ahi + kk * 8 + 32, dh + 2ull * kk, id, 1u);
+                                }
+#pragma unroll 1
+                                for (int kk = kw; kk < kw + p.wsteps; ++kk)
+                                    mma_tf32_pair(dw, ahi + kk * 8, dh + 2ull * kk, id, 1u);
+                                mma_commit_pair(bar(WF + b), (uint16_t)3);
+                            }
+                            if (!ok) break;
+                            issued = true;
+                            mma_commit_pair(bar(TEMPTY + slot), (uint16_t)3);
+                        }
+                        if (!ok) break;
+                        if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                        continue;
+                    }
+                    const int ab = SPLIT_ACC ? 0 : (int)(tile_i & 1);
+                    const uint32_t abph = SPLIT_ACC ? (uint32_t)(tile_i & 1) : (uint32_t)((tile_i >> 1) & 1);
+                    if (!warp_wait_cl(bar(ACCE + ab), abph ^ 1, abort_flag, peer_abort, p.err, 4)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t dacc = tmem + (uint32_t)(ab * 256);
+                    const uint32_t dcor = SPLIT_ACC ? tmem + 256u : dacc;
+                    // the last chunk of a plane holds Np % 32 = 16 valid K when Np is an odd
+                    // multiple of 16 (the rest is the TMA's zero fill): its zero K steps are
+                    // skipped.  kc counts chunks within the plane (no division in this loop:
+                    // this thread's issue rate bounds the kernel).
+                    if (!SPLIT_ACC && nchunk <= 2) {
+                        // The tile's whole K fits the two A slots: issue every correction
+                        // product first, while the accumulator is still small, then hi*hi,
+                        // so the only truncating additions at the scale of the result are
+                        // those of the hi*hi MMAs (as with separate accumulators, but
+                        // keeping the double-buffered accumulator).
+                        int ksteps[2];
+                        for (int c = 0; c < nchunk; ++c) {
+                            const long long ic = it + c;
+                            if (!warp_wait_cl(bar(TFULL + (int)(ic & 1)), (uint32_t)((ic >> 1) & 1), abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
+                            ksteps[c] = (c % p.kch) == p.kch - 1 ? ktail : 4;
+                        }
+                        if (!ok) break;
+                        tc_fence_after();
+                        bool first = true;
+                        for (int c = 0; c < nchunk; ++c) {
+                            const uint32_t ahi = tmem + (((it + c) & 1) ? slot_col1 : slot_col0);
+                            const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
+                            const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
+#pragma unroll 1
+                            for (int kk = 0; kk < ksteps[c]; ++kk) {
+                                mma_tf32_pair(dacc, ahi + kk * 8, dl + 2ull * kk, id, first ? 0u : 1u);
+                                mma_tf32_pair(dacc, ahi + kk * 8 + 32, dh + 2ull * kk, id, 1u);
+                                first = false;
+                            }
+                        }
+                        for (int c = 0; c < nchunk; ++c) {
+                            const uint32_t ahi = tmem + (((it + c) & 1) ? slot_col1 : slot_col0);
+                            const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
+#pragma unroll 1
+                            for (int kk = 0; kk < ksteps[c]; ++kk)
+                                mma_tf32_pair(dacc, ahi + kk * 8, dh + 2ull * kk, id, 1u);
+                            mma_commit_pair(bar(TEMPTY + (int)((it + c) & 1)), (uint16_t)3);
+                        }
+                        it += nchunk;
+                        issued = true;
+                        mma_commit_pair(bar(ACCF + ab), (uint16_t)3);
+                        if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                        continue;
+                    }
+                    int kc = 0;
+                    for (int c = 0; c < nchunk; ++c, ++it) {
                         const int slot = (int)(it & 1);
                         const uint32_t sph = (uint32_t)((it >> 1) & 1);
                         if (!warp_wait_cl(bar(TFULL + slot), sph, abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
                         tc_fence_after();
+                        // descriptor start field = address >> 4: a 32-byte K step adds 2
                         const uint32_t ahi = tmem + (slot ? slot_col1 : slot_col0);
                         const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
                         const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
                         const int ksteps = kc == p.kch - 1 ? ktail : 4;
                         if (++kc == p.kch) kc = 0;
-                        for (int kw = 0; kw < ksteps; kw += p.wsteps, wr.next()) {
-                            const int b = wr.i;
-                            if (!warp_wait_cl(bar(WE + b), wr.ph ^ 1u, abort_flag, peer_abort, p.err, 19)) { ok = false; break; }
-                            tc_fence_after();
-                            const uint32_t dw = tmem + 128u + (uint32_t)(b * p.as2);
 #pragma unroll 1
-                            for (int kk = kw; kk < kw + p.wsteps; ++kk) {
-                                mma_tf32_pair(dw, ahi + kk * 8, dl + 2ull * kk, id, kk == kw ? 0u : 1u);
-                                mma_tf32_pair(dw, ahi + kk * 8 + 32, dh + 2ull * kk, id, 1u);
-                            }
-#pragma unroll 1
-                            for (int kk = kw; kk < kw + p.wsteps; ++kk)
-                                mma_tf32_pair(dw, ahi + kk * 8, dh + 2ull * kk, id, 1u);
-                            mma_commit_pair(bar(WF + b), (uint16_t)3);
+                        for (int kk = 0; kk < ksteps; ++kk) {
+                            const uint32_t ah = ahi + kk * 8, al = ah + 32;
+                            const unsigned long long o = 2ull * kk;
+                            mma_tf32_pair(dacc, ah, dh + o, id, (c | kk) ? 1u : 0u);
+                            mma_tf32_pair(dcor, ah, dl + o, id, (SPLIT_ACC && !(c | kk)) ? 0u : 1u);
+                            mma_tf32_pair(dcor, al, dh + o, id, 1u);
                         }
-                        if (!ok) break;
                         issued = true;
                         mma_commit_pair(bar(TEMPTY + slot), (uint16_t)3);
                     }
                     if (!ok) break;
-                    if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
-                    continue;
-                }
-                const int ab = SPLIT_ACC ? 0 : (int)(tile_i & 1);
-                const uint32_t abph = SPLIT_ACC ? (uint32_t)(tile_i & 1) : (uint32_t)((tile_i >> 1) & 1);
-                if (!warp_wait_cl(bar(ACCE + ab), abph ^ 1, abort_flag, peer_abort, p.err, 4)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t dacc = tmem + (uint32_t)(ab * 256);
-                const uint32_t dcor = SPLIT_ACC ? tmem + 256u : dacc;
-                // the last chunk of a plane holds Np % 32 = 16 valid K when Np is an odd
-                // multiple of 16 (the rest is the TMA's zero fill): its zero K steps are
-                // skipped.  kc counts chunks within the plane (no division in this loop:
-                // this thread's issue rate bounds the kernel).
-                if (!SPLIT_ACC && nchunk <= 2) {
-                    // The tile's whole K fits the two A slots: issue every correction
-                    // product first, while the accumulator is still small, then hi*hi,
-                    // so the only truncating additions at the scale of the result are
-                    // those of the hi*hi MMAs (as with separate accumulators, but
-                    // keeping the double-buffered accumulator).
-                    int ksteps[2];
-                    for (int c = 0; c < nchunk; ++c) {
-                        const long long ic = it + c;
-                        if (!warp_wait_cl(bar(TFULL + (int)(ic & 1)), (uint32_t)((ic >> 1) & 1), abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
-                        ksteps[c] = (c % p.kch) == p.kch - 1 ? ktail : 4;
-                    }
-                    if (!ok) break;
-                    tc_fence_after();
-                    bool first = true;
-                    for (int c = 0; c < nchunk; ++c) {
-                        const uint32_t ahi = tmem + (((it + c) & 1) ? slot_col1 : slot_col0);
-                        const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
-                        const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
-#pragma unroll 1
-                        for (int kk = 0; kk < ksteps[c]; ++kk) {
-                            mma_tf32_pair(dacc, ahi + kk * 8, dl + 2ull * kk, id, first ? 0u : 1u);
-                            mma_tf32_pair(dacc, ahi + kk * 8 + 32, dh + 2ull * kk, id, 1u);
-                            first = false;
-                        }
-                    }
-                    for (int c = 0; c < nchunk; ++c) {
-                        const uint32_t ahi = tmem + (((it + c) & 1) ? slot_col1 : slot_col0);
-                        const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
-#pragma unroll 1
-                        for (int kk = 0; kk < ksteps[c]; ++kk)
-                            mma_tf32_pair(dacc, ahi + kk * 8, dh + 2ull * kk, id, 1u);
-                        mma_commit_pair(bar(TEMPTY + (int)((it + c) & 1)), (uint16_t)3);
-                    }
-                    it += nchunk;
-                    issued = true;
                     mma_commit_pair(bar(ACCF + ab), (uint16_t)3);
                     if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
-                    continue;
                 }
-                int kc = 0;
-                for (int c = 0; c < nchunk; ++c, ++it) {
-                    const int slot = (int)(it & 1);
-                    const uint32_t sph = (uint32_t)((it >> 1) & 1);
-                    if (!warp_wait_cl(bar(TFULL + slot), sph, abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
-                    tc_fence_after();
-                    // descriptor start field = address >> 4: a 32-byte K step adds 2
-                    const uint32_t ahi = tmem + (slot ? slot_col1 : slot_col0);
-                    const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
-                    const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
-                    const int ksteps = kc == p.kch - 1 ? ktail : 4;
-                    if (++kc == p.kch) kc = 0;
-#pragma unroll 1
-                    for (int kk = 0; kk < ksteps; ++kk) {
-                        const uint32_t ah = ahi + kk * 8, al = ah + 32;
-                        const unsigned long long o = 2ull * kk;
-                        mma_tf32_pair(dacc, ah, dh + o, id, (c | kk) ? 1u : 0u);
-                        mma_tf32_pair(dcor, ah, dl + o, id, (SPLIT_ACC && !(c | kk)) ? 0u : 1u);
-                        mma_tf32_pair(dcor, al, dh + o, id, 1u);
-                    }
-                    issued = true;
-                    mma_commit_pair(bar(TEMPTY + slot), (uint16_t)3);
-                }
-                if (!ok) break;
-                mma_commit_pair(bar(ACCF + ab), (uint16_t)3);
-                if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                (void)issued;
+                // Closing commit to both CTAs: it completes once every MMA this
+                // thread issued is done, so neither CTA leaves (or frees its TMEM)
+                // while an MMA still reads its shared memory or tensor memory,
+                // also when a wait gave up.
+                mma_commit_pair(bar(DRAIN), (uint16_t)3);
+                const unsigned long long g0 = gtimer();
+                while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
+            } else if (lane == 0) {
+                const unsigned long long g0 = gtimer();
+                while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
             }
-            (void)issued;
-            // Closing commit to both CTAs: it completes once every MMA this
-            // thread issued is done, so neither CTA leaves (or frees its TMEM)
-            // while an MMA still reads its shared memory or tensor memory,
-            // also when a wait gave up.
-            mma_commit_pair(bar(DRAIN), (uint16_t)3);
-            const unsigned long long g0 = gtimer();
-            while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
-        } else if (lane == 0) {
-            const unsigned long long g0 = gtimer();
-            while (!mbar_try(bar(DRAIN), 0) && gtimer() - g0 < kWaitLimitNs) {}
-        }
-    } else if (warp == 2) {
-        if (lane == 0 && rank == 1) {
-            // ---------------- B relay (odd CTA): its B half landed -> even CTA ----------------
-            int cur_u = -1;
-            uint32_t bph = 0;
-            for (long long t = t0; t < t1; ++t) {
-                const int u = (int)((uint32_t)t / ipu32);
-                if (u == cur_u) continue;
-                cur_u = u;
-                if (!mbar_wait_cl(bar(BFULL), bph, abort_flag, peer_abort, p.err, 9)) break;
-                bph ^= 1;
-                mbar_arrive_cluster(bar0(BPEER));
+        } else if (warp == 2) {
+            if (lane == 0 && rank == 1) {
+                // ---------------- B relay (odd CTA): its B half landed -> even CTA ----------------
+                int cur_u = -1;
+                uint32_t bph = 0;
+                for (long long t = t0; t < t1; ++t) {
+                    const int u = (int)((uint32_t)t / ipu32);
+                    if (u == cur_u) continue;
+                    cur_u = u;
+                    if (!mbar_wait_cl(bar(BFULL), bph, abort_flag, peer_abort, p.err, 9)) break;
+                    bph ^= 1;
+                    mbar_arrive_cluster(bar0(BPEER));
+                }
             }
         }
-    } else if (warp >= 4 && warp < 8) {
+    } else if (warp < 8) {
         // ---------------- converter: FP32 A tile -> TF32 hi/lo in this CTA's TMEM ----------------
+        stage_regs_dec<kStageRegsConv>();
         const int wq = warp & 3;
         const int r = wq * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
@@ -743,14 +766,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 if (lane == 0) mbar_arrive_cluster(bar0(TFULL + slot));
             }
         }
-    } else if (warp >= 8) {
+    } else {
         // ---------------- epilogue: this CTA's 128 rows, TMEM -> HBM ----------------
-        const int wq = warp & 3;
+        stage_regs_inc<kStageRegsEpi>();
+        // Windowed tiles (2 Np <= 96) alternate between two groups of four warps, each
+        // with half of the accumulator ring: one adds a tile's windows while the other
+        // stores the tile before.  With one group its chain of waits, tensor-memory
+        // loads and adds was the longest role (N = 32: 8.9 k cycles a tile, half of
+        // them waits).  Larger bases read a tile's sums once and take one group.
+        // us per unit of the TF32 self-energy, one group / two: N = 16 1.26 / 1.21,
+        // N = 24 14.2 / 13.4, N = 32 14.6 / 13.8, N = 48 77.7 / 73.1.
+        const int wq = warp & 3, grp = (warp >> 2) & 1;
         const int rloc = wq * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
         const int ncc = (2 * Np) / 32;
         long long tile_i = 0;
-        Ring wr(p.nring > 0 ? p.nring : 1);
+        Ring wr(p.nring > 1 ? p.nring / 2 : 1);
         bool ok = true;
         // 16-byte stores need rows that run contiguously in memory, 16-byte
         // aligned column offsets and a 16-byte aligned output
@@ -758,14 +789,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                              (p.map.SA % 4) == 0 && (p.map.SB % 4) == 0 && (p.map.SC % 4) == 0 &&
                              (p.map.SY % 4) == 0 && (p.out_unit % 4) == 0 && (p.map.Dx % 4) == 0 &&
                              (((uintptr_t)p.out) & 15) == 0;
-        for (long long t = t0; t < t1 && ok && win; ++t) {
+        for (long long t = t0 + grp; t < t1 && ok && win; t += 2) {
             // windowed mode (2 Np <= 96): add the tile's windows in FP32 registers
             const int u = (int)((uint32_t)t / ipu32);
             float acc[96];
 #pragma unroll
             for (int j = 0; j < 96; ++j) acc[j] = 0.0f;
             for (int i = 0; i < win_per_tile; ++i, wr.next()) {
-                const int b = wr.i;
+                const int b = grp * wr.n + wr.i;
                 if (!warp_wait_cl(bar(WF + b), wr.ph, abort_flag, peer_abort, p.err, 20)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
@@ -790,7 +821,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 // never cross the M rows of a unit (M = Np^3 is a multiple of 256).
                 const uint32_t row = ((uint32_t)t % ipu32) * (2 * kBM) + rank * kBM + wq * 32 + 4 * (lane & 7);
                 float* o = stage_out_row(p, u, row);
-                float* stg = stage_out + wq * 1024;
+                float* stg = stage_out + (grp * 4 + wq) * 1024;
 #pragma unroll
                 for (int cc = 0; cc < 3; ++cc) {
                     if (cc < ncc) {
@@ -823,7 +854,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 }
             }
         }
-        for (long long t = t0; t < t1 && ok && !win; ++t, ++tile_i) {
+        for (long long t = t0; t < t1 && ok && !win && grp == 0; ++t, ++tile_i) {
             const int u = (int)((uint32_t)t / ipu32);
             const int ab = SPLIT_ACC ? 0 : (int)(tile_i & 1);
             const uint32_t abph = SPLIT_ACC ? (uint32_t)(tile_i & 1) : (uint32_t)((tile_i >> 1) & 1);
@@ -1787,8 +1818,9 @@ constexpr int kMaxTcNp = 96;  // largest padded basis of the tensor-core path
 // Shared memory of a stage launch with `astages` A stages.
 size_t stage_smem_bytes(int Np, int astages) {
     const int kch = (Np + kKC - 1) / kKC;
-    // plus the epilogue's 4 x 4 KB staging blocks
-    return 1024 + 2ull * kch * (2 * Np * 128) + (size_t)astages * kTileBytes + 512 + 4 * 32 * 32 * 4;
+    // plus 4 KB of staging per epilogue warp (one group where tiles are not windowed)
+    const int warps = 2 * Np <= 96 ? 8 : 4;
+    return 1024 + 2ull * kch * (2 * Np * 128) + (size_t)astages * kTileBytes + 512 + warps * 32 * 32 * 4;
 }
 // The most A stages that fit next to the B operand (at least 4).
 int stage_astages(int Np) {
@@ -1891,7 +1923,7 @@ static StageParams stage_base(gkba_ctx* c, int nb) {
     // windowed accumulation where the ring fits next to the A slots (2 Np <= 96)
     sp.as2 = ((2 * Np + 31) / 32) * 32;
     sp.wsteps = 2 * Np <= 96 ? std::max(1, std::min(2, c->acc_window / 8)) : 0;
-    sp.nring = std::min(kStageRing, (512 - 128) / sp.as2);
+    sp.nring = std::min(kStageRing, (512 - 128) / sp.as2) & ~1;  // a ring for each epilogue group
     sp.astages = stage_astages(Np);
     return sp;
 }
