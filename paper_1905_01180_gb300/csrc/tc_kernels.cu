@@ -368,7 +368,7 @@ constexpr int kStageAStagesMax = 8;
 // dynamic shared memory of one CTA
 constexpr size_t kStageSmemMax = 227 * 1024;
 constexpr int kStageRing = 8;
-// warp 0 TMA, warp 1 MMA, 2 B relay, 4-7 converter, 8-11 and 12-15 epilogue
+// warp 0 TMA, warps 1 and 3 MMA, 2 B relay, 4-7 converter, 8-11 and 12-15 epilogue
 constexpr int kStageThreads = 512;
 // Register split of the warpgroups (128 a thread at launch, 4 x 128 in all): the
 // windowed epilogue keeps 96 sums.
@@ -400,7 +400,8 @@ __device__ __forceinline__ void stage_regs_inc() {
 // converters and epilogues of both CTAs arrive on the even CTA's TFULL / ACCE
 // (count 8: four warps per CTA); MMA completion is multicast to both CTAs'
 // TEMPTY / ACCF / BEMPTY.  The odd CTA forwards its B completion to the even
-// CTA's BPEER.  Every wait is bounded and a timeout raises both CTAs' abort
+// CTA's BPEER.  With windowed tiles the even CTA has two MMA warps, and TEMPTY
+// and BEMPTY take a commit of each.  Every wait is bounded and a timeout raises both CTAs' abort
 // flags.
 //
 // Tensor memory (512 columns, same address in both CTAs): accumulators at
@@ -457,14 +458,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
     if (threadIdx.x == 0) {
         mbar_init(bar(BFULL), 1);
         mbar_init(bar(BPEER), 1);
-        mbar_init(bar(BEMPTY), 1);
+        // windowed tiles have two MMA issuers
+        const uint32_t nissue = p.wsteps > 0 ? 2u : 1u;
+        mbar_init(bar(BEMPTY), nissue);
         for (int s = 0; s < nas; ++s) {
             mbar_init(bar(AFULL + s), 1);
             mbar_init(bar(AEMPTY + s), 4);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar(TFULL + s), 8);
-            mbar_init(bar(TEMPTY + s), 1);
+            mbar_init(bar(TEMPTY + s), nissue);
             mbar_init(bar(ACCF + s), 1);
             mbar_init(bar(ACCE + s), 8);
         }
@@ -472,7 +475,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
             mbar_init(bar(WF + b), 1);
             mbar_init(bar(WE + b), 8);
         }
-        mbar_init(bar(DRAIN), 1);
+        mbar_init(bar(DRAIN), 2);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -566,19 +569,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                     }
                 }
             }
-        } else if (warp == 1) {
+        } else if (warp != 2) {
             if (rank == 0) {
-                // ---------------- MMA issuer (even CTA, for the pair) ----------------
+                // ---------------- MMA issuers (even CTA, for the pair) ----------------
+                // Issuing, not the tensor pipe (15 % active), sets the pace of windowed
+                // tiles: about 290 cycles for a window's three MMAs and commit.  Two
+                // warps issue alternate windows of a ring.  At most one window of the
+                // other issuer lies between two of this one, so that with two or more
+                // accumulators in a ring a wait on WE never meets a phase two behind.
+                // us per unit, one issuer / two: N = 16 1.21 / 1.08, N = 32 13.8 / 12.4,
+                // N = 48 73.1 / 68.9.
+                const uint32_t me = warp == 3;
                 const uint32_t id = idesc_tf32_pair(2 * Np);
                 const unsigned long long dBhi0 = desc_sw128(smem_u32(sBhi));
                 const unsigned long long dBlo0 = desc_sw128(smem_u32(sBlo));
                 int cur_u = -1;
                 uint32_t bfph = 0;
                 long long it = 0, tile_i = 0;
+                uint32_t turn = 0;  // bit g: whose window is next in ring g
                 // the epilogue groups' rings: tiles alternate between them
                 Ring wr0(p.nring > 1 ? p.nring / 2 : 1), wr1 = wr0;
                 bool ok = true, issued = false;
-                for (long long t = t0; t < t1 && ok; ++t, ++tile_i) {
+                for (long long t = t0; t < t1 && ok && (win || me == 0); ++t, ++tile_i) {
                     const int u = (int)((uint32_t)t / ipu32);
                     if (u != cur_u) {
                         if (!warp_wait_cl(bar(BFULL), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
@@ -609,6 +621,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                                 const uint32_t wph = g1 ? wr1.ph : wr0.ph;
                                 if (g1) wr1.next();
                                 else wr0.next();
+                                const uint32_t whose = (turn >> (int)g1) & 1u;
+                                turn ^= 1u << (int)g1;
+                                if (whose != me) continue;
                                 if (!warp_wait_cl(bar(WE + b), wph ^ 1u, abort_flag, peer_abort, p.err, 19)) { ok = false; break; }
                                 tc_fence_after();
                                 const uint32_t dw = tmem + 128u + (uint32_t)(b * p.as2);
