@@ -228,27 +228,15 @@ __host__ __device__ constexpr uint32_t idesc_tf32_pair(int n) {
            ((uint32_t)((2 * kBM) >> 4) << 24);
 }
 
-// TF32 split of the streamed A operand, selected at compile time:
-//   0: hi = rna(x), lo = rna(x - hi)           (|error| <= 2^-23 |x| per element,
-//      unbiased: lo is exact in TF32, so no truncation toward zero remains)
-//   1: hi = x truncated to TF32, lo = rna(x - hi)
-//   2: hi = x truncated to TF32, lo = x - hi    (the MMA keeps lo's leading
-//      11 bits: |error| <= 2^-21 |x|), two full-rate integer/FP ops per element
-#ifndef GKBA_SPLIT_MODE
-#define GKBA_SPLIT_MODE 0
-#endif
-
+// TF32 split of the streamed A operand of S1-S3: hi = rna(x), lo = rna(x - hi),
+// |error| <= 2^-23 |x| per element and unbiased: lo is exact in TF32, so no
+// truncation toward zero remains.  hi is rounded on integer instructions (see
+// below), lo by the conversion: the conversion unit takes 64 cycles a warp for
+// 8 of them and bounded the converter with both (725 -> 573 cycles a chunk).  A
+// non-finite x gives a NaN lo (inf - inf, NaN - anything).
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-#if GKBA_SPLIT_MODE == 0
-    hi = tf32_rna(x);
+    hi = tf32_rna_bits(__float_as_uint(x));
     lo = tf32_rna(x - __uint_as_float(hi));
-#elif GKBA_SPLIT_MODE == 1
-    hi = __float_as_uint(x) & 0xFFFFE000u;
-    lo = tf32_rna(x - __uint_as_float(hi));
-#else
-    hi = __float_as_uint(x) & 0xFFFFE000u;
-    lo = __float_as_uint(x - __uint_as_float(hi));
-#endif
 }
 
 // Load row r (0..127) of a 128 x 32 FP32 tile written by TMA with the 128-byte
@@ -835,8 +823,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 // lane l stores rows 4 (l % 8) .. + 3 of columns l / 8 + 4 i.  Tiles
                 // never cross the M rows of a unit (M = Np^3 is a multiple of 256).
                 const uint32_t row = ((uint32_t)t % ipu32) * (2 * kBM) + rank * kBM + wq * 32 + 4 * (lane & 7);
-                float* o = stage_out_row(p, u, row);
+                float* o = stage_out_row(p, u, row) + (long long)(lane >> 3) * p.map.SY;
                 float* stg = stage_out + (grp * 4 + wq) * 1024;
+                // Np is a multiple of 16: the four columns of a store lie in one half,
+                // and their offset is the same for all lanes (computed per lane it was
+                // most of this loop: 2.9 -> 2.2 k cycles a tile at N = 32).  Stores
+                // straight from the registers, 4 bytes a lane, take twice as long.
 #pragma unroll
                 for (int cc = 0; cc < 3; ++cc) {
                     if (cc < ncc) {
@@ -844,15 +836,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
 #pragma unroll
                         for (int j = 0; j < 32; ++j) stg[j * 32 + lane] = acc[cc * 32 + j];
                         __syncwarp();
+                        float4 v4[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            v4[i] = *reinterpret_cast<const float4*>(stg + (4 * i + (lane >> 3)) * 32 + 4 * (lane & 7));
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int cl = 4 * i + (lane >> 3);
-                            const int col = cc * 32 + cl;
-                            const int hc = col >= Np ? 1 : 0;
-                            const int y = col - hc * Np;
-                            const float4 v4 = *reinterpret_cast<const float4*>(stg + cl * 32 + 4 * (lane & 7));
-                            if (col < 2 * Np && (long long)row + 3 < p.M)
-                                *reinterpret_cast<float4*>(o + hc * p.map.SC + (long long)y * p.map.SY) = v4;
+                            const int col = cc * 32 + 4 * i;
+                            const long long off = col < Np ? col * p.map.SY : p.map.SC + (col - Np) * p.map.SY;
+                            if (col < 2 * Np) *reinterpret_cast<float4*>(o + off) = v4[i];
                         }
                     }
                 }
@@ -880,7 +872,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
             float* o = stage_out_row(p, u, row);
             // 16-byte stores through the warp's staging block (see the windowed path)
             const uint32_t row4 = ((uint32_t)t % ipu32) * (2 * kBM) + rank * kBM + wq * 32 + 4 * (lane & 7);
-            float* o4 = vec_out ? stage_out_row(p, u, row4) : nullptr;
+            float* o4 = vec_out ? stage_out_row(p, u, row4) + (long long)(lane >> 3) * p.map.SY : nullptr;
             float* stg = stage_out + wq * 1024;
             for (int cc = 0; cc < ncc; ++cc) {
                 uint32_t v[32];
@@ -900,15 +892,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
 #pragma unroll
                     for (int j = 0; j < 32; ++j) stg[j * 32 + lane] = __uint_as_float(v[j]);
                     __syncwarp();
+                    float4 v4[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        v4[i] = *reinterpret_cast<const float4*>(stg + (4 * i + (lane >> 3)) * 32 + 4 * (lane & 7));
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const int cl = 4 * i + (lane >> 3);
-                        const int col = cc * 32 + cl;
-                        const int hc = col >= Np ? 1 : 0;
-                        const int y = col - hc * Np;
-                        const float4 v4 = *reinterpret_cast<const float4*>(stg + cl * 32 + 4 * (lane & 7));
-                        if ((long long)row4 + 3 < p.M)
-                            *reinterpret_cast<float4*>(o4 + hc * p.map.SC + (long long)y * p.map.SY) = v4;
+                        const int col = cc * 32 + 4 * i;
+                        const long long off = col < Np ? col * p.map.SY : p.map.SC + (col - Np) * p.map.SY;
+                        *reinterpret_cast<float4*>(o4 + off) = v4[i];
                     }
                 } else if (valid) {
 #pragma unroll
