@@ -175,6 +175,28 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask) {
         "h"(mask)
         : "memory");
 }
+// One accumulation window of one K step, and its commit to both CTAs: lo x hi,
+// hi x lo (into a cleared accumulator), hi x hi.  a: columns of A's hi (lo 32
+// further); bl, bh: low words of B's descriptors, bdh their high word.  One
+// election for the four instructions.
+__device__ __forceinline__ void mma_window_pair(uint32_t d, uint32_t a, uint32_t bl, uint32_t bh, uint32_t bdh,
+                                                uint32_t idesc, uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 l, h;\n\t.reg .b16 m;\n\t"
+        "mov.b64 l, {%3, %5};\n\t"
+        "mov.b64 h, {%4, %5};\n\t"
+        "mov.b16 m, 3;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, 0, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], l, %6, p;\n\t"
+        "setp.eq.b32 p, 0, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], [%2], h, %6, p;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], h, %6, p;\n\t"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+        "[%7], m;\n\t}" ::"r"(d),
+        "r"(a), "r"(a + 32), "r"(bl), "r"(bh), "r"(bdh), "r"(idesc), "r"(bar)
+        : "memory");
+}
 #define R8(a, o) "r"(a[o + 0]), "r"(a[o + 1]), "r"(a[o + 2]), "r"(a[o + 3]), "r"(a[o + 4]), "r"(a[o + 5]), "r"(a[o + 6]), "r"(a[o + 7])
 #define W8(a, o) "=r"(a[o + 0]), "=r"(a[o + 1]), "=r"(a[o + 2]), "=r"(a[o + 3]), "=r"(a[o + 4]), "=r"(a[o + 5]), "=r"(a[o + 6]), "=r"(a[o + 7])
 
@@ -566,7 +588,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 // other issuer lies between two of this one, so that with two or more
                 // accumulators in a ring a wait on WE never meets a phase two behind.
                 // us per unit, one issuer / two: N = 16 1.21 / 1.08, N = 32 13.8 / 12.4,
-                // N = 48 73.1 / 68.9.
+                // N = 48 73.1 / 68.9.  Bookkeeping counts as much as the MMAs: each warp
+                // walks only its own windows, counts a unit's tiles instead of dividing
+                // and elects a lane once a window (N = 32 11.4 / 10.7, N = 48 63.5 / 62.6).
                 const uint32_t me = warp == 3;
                 const uint32_t id = idesc_tf32_pair(2 * Np);
                 const unsigned long long dBhi0 = desc_sw128(smem_u32(sBhi));
@@ -574,12 +598,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                 int cur_u = -1;
                 uint32_t bfph = 0;
                 long long it = 0, tile_i = 0;
-                uint32_t turn = 0;  // bit g: whose window is next in ring g
-                // the epilogue groups' rings: tiles alternate between them
-                Ring wr0(p.nring > 1 ? p.nring / 2 : 1), wr1 = wr0;
-                bool ok = true, issued = false;
+                // the epilogue groups' rings (tiles alternate between them): entry and
+                // phase of this issuer's next window, and whose window comes next
+                const int nr = p.nring > 1 ? p.nring / 2 : 1;
+                int wi = (int)me, wi2 = (int)me, wbase = 0;
+                uint32_t wph = 0, wph2 = 0, turn = 0, turn2 = 0;
+                const int wsteps = p.wsteps;
+                const uint32_t as2 = (uint32_t)p.as2, dbh = (uint32_t)(dBhi0 >> 32), bWE = bar(WE), bWF = bar(WF);
+                int u = (int)((uint32_t)t0 / ipu32);
+                uint32_t left = ipu32 - (uint32_t)t0 % ipu32;  // tiles of unit u
+                bool ok = true;
                 for (long long t = t0; t < t1 && ok && (win || me == 0); ++t, ++tile_i) {
-                    const int u = (int)((uint32_t)t / ipu32);
                     if (u != cur_u) {
                         if (!warp_wait_cl(bar(BFULL), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
                         if (!warp_wait_cl(bar(BPEER), bfph, abort_flag, peer_abort, p.err, 3)) { ok = false; break; }
@@ -587,50 +616,72 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                         cur_u = u;
                         tc_fence_after();
                     }
+                    const bool unit_end = --left == 0 && t + 1 < t1;  // the next tile is of the next unit
+                    if (left == 0) {
+                        left = ipu32;
+                        ++u;
+                    }
                     if (win) {
                         // Windowed accumulation: every wsteps K steps go to the next
                         // accumulator of a ring that the epilogue drains into FP32
                         // register sums; inside a window the correction products come
                         // first, while the accumulator is still small, then hi*hi.
                         int kc = 0;
-                        for (int c = 0; c < nchunk && ok; ++c, ++it) {
+                        for (int c = 0; c < nchunk; ++c, ++it) {
                             const int slot = (int)(it & 1);
                             const uint32_t sph = (uint32_t)((it >> 1) & 1);
-                            if (!warp_wait_cl(bar(TFULL + slot), sph, abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
-                            tc_fence_after();
-                            const uint32_t ahi = tmem + (slot ? slot_col1 : slot_col0);
-                            const unsigned long long dh = dBhi0 + ((unsigned long long)(c * chunkB) >> 4);
-                            const unsigned long long dl = dBlo0 + ((unsigned long long)(c * chunkB) >> 4);
                             const int ksteps = kc == p.kch - 1 ? ktail : 4;
                             if (++kc == p.kch) kc = 0;
-                            for (int kw = 0; kw < ksteps; kw += p.wsteps) {
-                                const bool g1 = (tile_i & 1) != 0;
-                                const int b = g1 ? wr1.i + wr1.n : wr0.i;
-                                const uint32_t wph = g1 ? wr1.ph : wr0.ph;
-                                if (g1) wr1.next();
-                                else wr0.next();
-                                const uint32_t whose = (turn >> (int)g1) & 1u;
-                                turn ^= 1u << (int)g1;
-                                if (whose != me) continue;
-                                if (!warp_wait_cl(bar(WE + b), wph ^ 1u, abort_flag, peer_abort, p.err, 19)) { ok = false; break; }
-                                tc_fence_after();
-                                const uint32_t dw = tmem + 128u + (uint32_t)(b * p.as2);
-#pragma unroll 1
-                                for (int kk = kw; kk < kw + p.wsteps; ++kk) {
-                                    mma_tf32_pair(dw, ahi + kk * 8, dl + 2ull * kk, id, kk == kw ? 0u : 1u);
-                                    mma_tf32_pair(dw, ahi + kk * 8 + 32, dh + 2ull * kk, id, 1u);
+                            const uint32_t ahi = tmem + (slot ? slot_col1 : slot_col0);
+                            const uint32_t dh = (uint32_t)dBhi0 + (c * chunkB >> 4);
+                            const uint32_t dl = (uint32_t)dBlo0 + (c * chunkB >> 4);
+                            if (!warp_wait_cl(bar(TFULL + slot), sph, abort_flag, peer_abort, p.err, 5)) { ok = false; break; }
+                            tc_fence_after();
+                            int kw = turn == me ? 0 : wsteps;
+                            for (; kw < ksteps; kw += 2 * wsteps) {
+                                const uint32_t b = (uint32_t)(wbase + wi);
+                                if (!warp_wait_cl(bWE + 8 * b, wph ^ 1u, abort_flag, peer_abort, p.err, 19)) {
+                                    ok = false;
+                                    break;
                                 }
+                                tc_fence_after();
+                                const uint32_t dw = tmem + 128u + b * as2;
+                                if (wsteps == 1) {
+                                    mma_window_pair(dw, ahi + kw * 8, dl + 2 * kw, dh + 2 * kw, dbh, id, bWF + 8 * b);
+                                } else {
+                                    const unsigned long long qh = dBhi0 + (c * chunkB >> 4);
+                                    const unsigned long long ql = dBlo0 + (c * chunkB >> 4);
 #pragma unroll 1
-                                for (int kk = kw; kk < kw + p.wsteps; ++kk)
-                                    mma_tf32_pair(dw, ahi + kk * 8, dh + 2ull * kk, id, 1u);
-                                mma_commit_pair(bar(WF + b), (uint16_t)3);
+                                    for (int kk = kw; kk < kw + wsteps; ++kk) {
+                                        mma_tf32_pair(dw, ahi + kk * 8, ql + 2ull * kk, id, kk == kw ? 0u : 1u);
+                                        mma_tf32_pair(dw, ahi + kk * 8 + 32, qh + 2ull * kk, id, 1u);
+                                    }
+#pragma unroll 1
+                                    for (int kk = kw; kk < kw + wsteps; ++kk)
+                                        mma_tf32_pair(dw, ahi + kk * 8, qh + 2ull * kk, id, 1u);
+                                    mma_commit_pair(bWF + 8 * b, (uint16_t)3);
+                                }
+                                if ((wi += 2) >= nr) {
+                                    wi -= nr;
+                                    wph ^= 1u;
+                                }
                             }
                             if (!ok) break;
-                            issued = true;
+                            turn ^= (uint32_t)(ksteps / wsteps) & 1u;
                             mma_commit_pair(bar(TEMPTY + slot), (uint16_t)3);
                         }
                         if (!ok) break;
-                        if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                        if (unit_end) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                        // the next tile's ring
+                        const int i3 = wi;
+                        const uint32_t p3 = wph, t3 = turn;
+                        wi = wi2;
+                        wph = wph2;
+                        turn = turn2;
+                        wi2 = i3;
+                        wph2 = p3;
+                        turn2 = t3;
+                        wbase = nr - wbase;
                         continue;
                     }
                     const int ab = SPLIT_ACC ? 0 : (int)(tile_i & 1);
@@ -678,9 +729,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                             mma_commit_pair(bar(TEMPTY + (int)((it + c) & 1)), (uint16_t)3);
                         }
                         it += nchunk;
-                        issued = true;
                         mma_commit_pair(bar(ACCF + ab), (uint16_t)3);
-                        if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                        if (unit_end) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
                         continue;
                     }
                     int kc = 0;
@@ -703,14 +753,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStageThreads, 1)
                             mma_tf32_pair(dcor, ah, dl + o, id, (SPLIT_ACC && !(c | kk)) ? 0u : 1u);
                             mma_tf32_pair(dcor, al, dh + o, id, 1u);
                         }
-                        issued = true;
                         mma_commit_pair(bar(TEMPTY + slot), (uint16_t)3);
                     }
                     if (!ok) break;
                     mma_commit_pair(bar(ACCF + ab), (uint16_t)3);
-                    if (t + 1 < t1 && (int)((uint32_t)(t + 1) / ipu32) != u) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
+                    if (unit_end) mma_commit_pair(bar(BEMPTY), (uint16_t)3);
                 }
-                (void)issued;
                 // Closing commit to both CTAs: it completes once every MMA this
                 // thread issued is done, so neither CTA leaves (or frees its TMEM)
                 // while an MMA still reads its shared memory or tensor memory,
