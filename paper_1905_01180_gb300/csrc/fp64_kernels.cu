@@ -21,7 +21,6 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 // acc += a b in four FMAs (a multiply followed by an add takes six FP64
 // instructions, and the FP64 rate, two a clock and SM, bounds these kernels).
 __device__ __forceinline__ void cmac(double2& acc, double2 a, double2 b) {
@@ -127,7 +126,8 @@ __global__ void __launch_bounds__(256) k_gemm64_stage(const double* __restrict__
 // one output per TPO lanes, the sum over k split over them.  TPO is chosen so
 // that a single matrix, too, spreads over all SMs with a few warps each (a
 // 16 x 16 tile per block kept nine of them busy at n = 48).  Measured, tiles ->
-// here: 2501 products at n = 10 100 -> 27 us; one at n = 48 16.5 -> 4.4 us.
+// here: the five products of a Heun step at n = 10 (four over 2501 points) 914 ->
+// 194 us together; one at n = 48 16.5 -> 3.0 us.
 // ---------------------------------------------------------------------------
 // Imaginary part's sign bit flipped by s (conjugation on the integer pipe).
 __device__ __forceinline__ double2 zsign(double2 a, int s) {
@@ -662,7 +662,7 @@ __global__ void k_weighted_sum_p1(int NN, int nb, int per, const double* __restr
     tmp[(long long)blockIdx.y * NN + e] = make_double2(re, im);
 }
 // One warp per element (a thread per element summed 256 ranges one after the
-// other: 31 us a call at N = 10, here 3).
+// other: 31 us a call at N = 10, here 4).
 __global__ void k_weighted_sum_p2(int NN, int nz, const double2* __restrict__ tmp,
                                   double2* __restrict__ I_acc) {
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -787,7 +787,7 @@ __global__ void k_sigma_symm(int N, const double* __restrict__ V, const double2*
 // Bound by the FP64 rate.  A thread holds one row i and kSymmJ columns j, so that
 // V_ik Gb_lk is formed once for all of them: 4.4 FP64 instructions a term of the
 // N^4 sum (8 with one column a thread and multiplies kept apart from adds).
-// Measured at N = 10, 2002 units: 493 -> 230 us.
+// Measured at N = 10, 2002 units: 493 -> 270 us.
 constexpr int kSymmSmallN = 24, kSymmJ = 5, kSymmMaxUnits = 16, kSymmThreads = 64;
 inline int symm_units(int N) {  // units a block
     const int per = N * ((N + kSymmJ - 1) / kSymmJ);

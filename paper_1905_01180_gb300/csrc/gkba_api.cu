@@ -462,7 +462,7 @@ void free_ctx(gkba_ctx* c) {
     void* ptrs[] = {c->tl_acc, c->tl_s, c->tl_W, c->tl_Wn, c->tl_uf,
                     c->h, c->d, c->v, c->vm, c->vjp, c->rhot_hist, c->U_hist, c->adj_ws, c->vomega,
                     c->vgrad, c->hfK, c->wS64, c->vK64, c->vKimg, c->wS32, c->vO32, c->xsw, c->vKhi, c->vKlo,
-                    c->rho_hist, c->T_a, c->T_b, c->hhf_n, c->hhf_t, c->k1, c->k2, c->Ia, c->Ib,
+                    c->rho_hist, c->T_a, c->T_b, c->hhf_n, c->hhf_t, c->k1, c->Ia, c->Ib,
                     c->U, c->ex0, c->ex1, c->ex2, c->tmp0, c->tmp1, c->dscal, c->dint, c->ws,
                     c->stage};
     for (void* p : ptrs)
@@ -644,7 +644,6 @@ gkba_status gkba_init(gkba_ctx** out, const gkba_config* cfg, const double* h, c
     ALLOC(c->hhf_n, NN * 16);
     ALLOC(c->hhf_t, NN * 16);
     ALLOC(c->k1, NN * 16);
-    ALLOC(c->k2, NN * 16);
     ALLOC(c->Ia, NN * 16);
     ALLOC(c->Ib, NN * 16);
     ALLOC(c->U, NN * 16);

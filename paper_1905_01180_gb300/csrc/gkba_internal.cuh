@@ -103,7 +103,6 @@ struct gkba_ctx {
     double2* hhf_n = nullptr;
     double2* hhf_t = nullptr;
     double2* k1 = nullptr;
-    double2* k2 = nullptr;
     double2* Ia = nullptr;       // I(t_n)
     double2* Ib = nullptr;       // I(t_{n+1}) of the corrector
     double2* U = nullptr;

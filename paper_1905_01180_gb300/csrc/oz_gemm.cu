@@ -12,8 +12,8 @@
 // sum than the FMA chain's (tests/test_oz_digits.py; whole Heun steps and
 // self-energies: 1.1-2.0e-15 from 64-bit references where the FMA chain had
 // 1.2-2.8e-15).  Whole calls, FMA chain -> here: Heun step at N = 24, 301 points
-// 309 -> 17.1 ms; 40 self-energies at N = 33 78 -> 2.7 ms; Heun step at N = 10,
-// 501 points 23.8 -> 1.7 ms; three time-linear steps at N = 48 137 -> 14.1 ms.
+// 309 -> 15.8 ms; 40 self-energies at N = 33 78 -> 2.8 ms; Heun step at N = 10,
+// 501 points 23.8 -> 1.4 ms; three time-linear steps at N = 48 137 -> 11.4 ms.
 //
 // What bounds it: the integer instructions of the epilogue and the converter
 // (about 64 a result and 47 an element; at N = 24 the integer pipe is 52 % busy,
