@@ -7,6 +7,7 @@
 //    U_n = exp(-i dt h) by scaling and squaring with a Taylor polynomial,
 //    the propagator recursion T(t_{n+1},t_k) = U_n T(t_n,t_k), Heun updates.
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 #include <cstdarg>
 #include <mutex>
@@ -28,6 +29,56 @@ __device__ __forceinline__ void cmac(double2& acc, double2 a, double2 b) {
     acc.y = fma(a.x, b.y, acc.y);
     acc.x = fma(-a.y, b.y, acc.x);
     acc.y = fma(a.y, b.x, acc.y);
+}
+// a b in a fixed form, rounded by itself.  The N x N products of split-TF32 contexts
+// add such terms in the order of k (dot_seq): their results become FP32 operands,
+// and one that falls on the other side of an FP32 rounding boundary moves a
+// collision integral by up to 1e-8.
+__device__ __forceinline__ double2 cmul_seq(double2 a, double2 b) {
+    return make_double2(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ double flip(double a, int s) {
+    return __hiloint2double(__double2hiint(a) ^ s, __double2loint(a));
+}
+// Re (comp 0, sgn the sign bit) or Im (comp 1, sgn 0) of a b.
+__device__ __forceinline__ double prod_seq(double2 a, double2 b, int comp, int sgn) {
+    const double u = comp ? a.y : a.x, w = comp ? a.x : a.y;
+    return __fma_rn(u, b.x, flip(__dmul_rn(w, b.y), sgn));
+}
+// The whole sum over k of a[k da] b[k db]: COMP 2 both components (of one lane), else
+// acc.x takes the component comp.  The products of eight terms are formed before they
+// are added: one chain of load, multiply, FMA and add a term has four latencies.
+template <int COMP>
+__device__ __forceinline__ void dot_seq(double2& acc, const double2* a, int da, int sa, const double2* b, int db,
+                                        int sb, int n, int comp) {
+    constexpr int U = 8;
+    const int sgn = comp ? 0 : (int)0x80000000;
+    auto chunk = [&](int k0, auto count) {
+        constexpr int C = decltype(count)::value;
+        double2 x[C], y[C];
+        double p[C], q[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            x[i] = a[(k0 + i) * da];
+            y[i] = b[(k0 + i) * db];
+        }
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            x[i].y = flip(x[i].y, sa);
+            y[i].y = flip(y[i].y, sb);
+            p[i] = prod_seq(x[i], y[i], COMP == 2 ? 0 : comp, COMP == 2 ? (int)0x80000000 : sgn);
+            if (COMP == 2) q[i] = prod_seq(x[i], y[i], 1, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            acc.x = __dadd_rn(acc.x, p[i]);
+            if (COMP == 2) acc.y = __dadd_rn(acc.y, q[i]);
+        }
+    };
+    int k = 0;
+    for (; k + U <= n; k += U) chunk(k, std::integral_constant<int, U>{});
+    for (; k + 2 <= n; k += 2) chunk(k, std::integral_constant<int, 2>{});
+    if (k < n) chunk(k, std::integral_constant<int, 1>{});
 }
 
 // ---------------------------------------------------------------------------
@@ -122,24 +173,27 @@ __global__ void __launch_bounds__(256) k_gemm64_stage(const double* __restrict__
 // of squarings in the exponential).
 //
 // Bound by the FP64 rate (two FMAs a clock and SM: 4 n^3 of them a matrix), so
-// every output is four FMAs a term with no padding to a tile, read through L1:
-// one output per TPO lanes, the sum over k split over them.  TPO is chosen so
-// that a single matrix, too, spreads over all SMs with a few warps each (a
-// 16 x 16 tile per block kept nine of them busy at n = 48).  Measured, tiles ->
-// here: the five products of a Heun step at n = 10 (four over 2501 points) 914 ->
-// 194 us together; one at n = 48 16.5 -> 3.0 us.
+// outputs are summed without padding to a tile, read through L1, in an order that
+// is fixed whatever the other matrices of the launch.  SEQ (split-TF32 contexts):
+// rounded products added in the order of k, by one lane an output or, where the
+// launch has few outputs, by two, its real and its imaginary part.  Else FMA chains:
+// eight, one a lane, from n = 32 on (single matrices, of the exponential, count
+// most there: at n = 48 3.7 us each, 7.4 by two lanes); below, of even and of odd k,
+// by one lane or by two.  Measured, 16 x 16 tiles -> here: the five
+// products of a Heun step at n = 10 (over 2501 points, two of them over 5002
+// matrices) 914 -> 204 us together; one matrix of n = 48 16.5 -> 3.7 us.  SEQ takes
+// six FP64 instructions a term where FMAs take four: the five products at n = 24,
+// 501 points, 619 us (FMAs 426).
 // ---------------------------------------------------------------------------
 // Imaginary part's sign bit flipped by s (conjugation on the integer pipe).
-__device__ __forceinline__ double2 zsign(double2 a, int s) {
-    return make_double2(a.x, __hiloint2double(__double2hiint(a.y) ^ s, __double2loint(a.y)));
-}
+__device__ __forceinline__ double2 zsign(double2 a, int s) { return make_double2(a.x, flip(a.y, s)); }
 
 struct ZPoly {
     double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
     const double2 *X1 = nullptr, *X2 = nullptr, *X3 = nullptr;
 };
 
-template <int TPO>
+template <int LANES, bool SEQ>
 __global__ void __launch_bounds__(128) k_zgemm(int n, int opA, int opB, double2 alpha,
                                                const double2* __restrict__ A, long long sA,
                                                const double2* __restrict__ B, long long sB,
@@ -147,9 +201,9 @@ __global__ void __launch_bounds__(128) k_zgemm(int n, int opA, int opB, double2 
                                                uint32_t total, int ident_b, const ZPoly p,
                                                const int* skip_ge, int idx) {
     if (skip_ge != nullptr && idx >= *skip_ge) return;
-    const uint32_t gid = blockIdx.x * 128u + threadIdx.x;
-    const uint32_t o = min(gid / TPO, total - 1u);
-    const int sub = (int)(gid % TPO);
+    const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t o = min(gid / LANES, total - 1u);
+    const int sub = (int)(gid % LANES);
     const uint32_t nn = (uint32_t)(n * n);
     const int b = (int)(o / nn), e = (int)(o - (uint32_t)b * nn);
     const int row = e / n, col = e - row * n;
@@ -158,34 +212,42 @@ __global__ void __launch_bounds__(128) k_zgemm(int n, int opA, int opB, double2 
         const double2* a = A + (long long)b * sA + (opA ? row : row * n);
         const double2* bb = B + (long long)b * sB + (opB ? col * n : col);
         const int da = opA ? n : 1, db = opB ? 1 : n;
-        double2 acc2 = make_double2(0.0, 0.0);
         const int sa = opA ? (int)0x80000000 : 0, sb = opB ? (int)0x80000000 : 0;
-        int k = sub;
+        if (SEQ) {
+            dot_seq<LANES == 1 ? 2 : 1>(acc, a, da, sa, bb, db, sb, n, sub);
+        } else {
+            // the chains of k = 0 .. CH - 1 (mod CH), in as many lanes, or both of two in one
+            constexpr int CH = LANES == 1 ? 2 : LANES;
+            double2 acc2 = make_double2(0.0, 0.0);
+            int k = sub;
 #pragma unroll 2
-        for (; k + TPO < n; k += 2 * TPO) {
-            const double2 x0 = a[k * da], y0 = bb[k * db], x1 = a[(k + TPO) * da], y1 = bb[(k + TPO) * db];
-            cmac(acc, zsign(x0, sa), zsign(y0, sb));
-            cmac(acc2, zsign(x1, sa), zsign(y1, sb));
+            for (; k + CH - LANES < n; k += CH) {
+                cmac(acc, zsign(a[k * da], sa), zsign(bb[k * db], sb));
+                if (LANES == 1) cmac(acc2, zsign(a[(k + 1) * da], sa), zsign(bb[(k + 1) * db], sb));
+            }
+            if (LANES == 1) {
+                if (k < n) cmac(acc, zsign(a[k * da], sa), zsign(bb[k * db], sb));
+                acc = cadd(acc, acc2);
+            }
         }
-        if (k < n) {
-            const double2 x0 = a[k * da], y0 = bb[k * db];
-            cmac(acc, zsign(x0, sa), zsign(y0, sb));
-        }
-        acc = cadd(acc, acc2);
     }
+    if (SEQ) {
+        if (LANES == 2) acc.y = __shfl_xor_sync(0xffffffffu, acc.x, 1);  // the other lane's part
+    } else {
 #pragma unroll
-    for (int d = TPO / 2; d > 0; d >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+        for (int d = LANES / 2; d > 0; d >>= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+        }
     }
-    if (sub != 0 || gid / TPO >= total) return;
+    if (sub != 0 || gid / LANES >= total) return;
     double2* c = C + (long long)b * sC + e;
     if (b >= ident_b) {
         *c = make_double2(row == col ? 1.0 : 0.0, 0.0);
         return;
     }
-    double2 r = cmul(alpha, acc);
-    if (beta.x != 0.0 || beta.y != 0.0) cmac(r, beta, *c);
+    double2 r = cmul_seq(alpha, acc);
+    if (beta.x != 0.0 || beta.y != 0.0) r = cadd(r, cmul_seq(beta, *c));
     if (row == col) r.x += p.c0;
     if (p.X1) r = make_double2(fma(p.c1, p.X1[e].x, r.x), fma(p.c1, p.X1[e].y, r.y));
     if (p.X2) r = make_double2(fma(p.c2, p.X2[e].x, r.x), fma(p.c2, p.X2[e].y, r.y));
@@ -224,39 +286,35 @@ __global__ void k_mean_field(int N, const double* __restrict__ hfK, const double
     }
 }
 
-// One stage of Heun's method, every element by kRhsLanes lanes:
+// One stage of Heun's method, every element by four lanes, the two components of
+// h rho and of rho h (fixed order of k, rounded products: see dot_seq):
 //   k = -i [h, rho] - (I + I^+);  y = base + a (k + kprev)
 // with k written to k_out and y also to y2 when given (kprev may be null).
-constexpr int kRhsLanes = 8;
-__global__ void __launch_bounds__(128) k_heun_stage(int N, const double2* __restrict__ h,
-                                                    const double2* __restrict__ rho,
-                                                    const double2* __restrict__ I,
-                                                    const double2* __restrict__ base,
-                                                    const double2* __restrict__ kprev, double a,
-                                                    double2* __restrict__ k_out, double2* __restrict__ y,
-                                                    double2* __restrict__ y2) {
-    const int gid = blockIdx.x * 128 + threadIdx.x, sub = gid % kRhsLanes;
-    const int e = min(gid / kRhsLanes, N * N - 1), i = e / N, j = e % N;
-    double2 c = make_double2(0.0, 0.0), d = make_double2(0.0, 0.0);
-    for (int k = sub; k < N; k += kRhsLanes) {
-        cmac(c, h[i * N + k], rho[k * N + j]);
-        cmac(d, rho[i * N + k], h[k * N + j]);
-    }
-    c = make_double2(c.x - d.x, c.y - d.y);
-#pragma unroll
-    for (int o = kRhsLanes / 2; o > 0; o >>= 1) {
-        c.x += __shfl_xor_sync(0xffffffffu, c.x, o);
-        c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
-    }
-    if (sub != 0 || gid / kRhsLanes >= N * N) return;
+__global__ void __launch_bounds__(64) k_heun_stage(int N, const double2* __restrict__ h,
+                                                   const double2* __restrict__ rho,
+                                                   const double2* __restrict__ I,
+                                                   const double2* __restrict__ base,
+                                                   const double2* __restrict__ kprev, double a,
+                                                   double2* __restrict__ k_out, double2* __restrict__ y,
+                                                   double2* __restrict__ y2) {
+    const int gid = blockIdx.x * 64 + threadIdx.x, sub = gid & 3, comp = sub & 1;
+    const int e = min(gid >> 2, N * N - 1), i = e / N, j = e % N;
+    const double2 *l = (sub & 2 ? rho : h) + i * N, *r = (sub & 2 ? h : rho) + j;
+    double2 acc = make_double2(0.0, 0.0);
+    dot_seq<1>(acc, l, 1, 0, r, N, 0, N, comp);
+    double s = acc.x;
+    s = __dadd_rn(s, -__shfl_xor_sync(0xffffffffu, s, 2));
+    const double2 c = make_double2(s, __shfl_xor_sync(0xffffffffu, s, 1));  // of lane 0
+    if (sub != 0 || (gid >> 2) >= N * N) return;
     const double2 x = I[e], xt = I[j * N + i];
     // -i c = (c.y, -c.x); I + I^+ at (i,j) = I_ij + conj(I_ji)
     double2 k = make_double2(c.y - (x.x + xt.x), -c.x - (x.y - xt.y));
     if (k_out) k_out[e] = k;
     if (kprev) k = cadd(kprev[e], k);
-    const double2 b = base[e], r = make_double2(fma(a, k.x, b.x), fma(a, k.y, b.y));
-    y[e] = r;
-    if (y2) y2[e] = r;
+    const double2 b = base[e];
+    const double2 v = make_double2(__dadd_rn(b.x, __dmul_rn(a, k.x)), __dadd_rn(b.y, __dmul_rn(a, k.y)));
+    y[e] = v;
+    if (y2) y2[e] = v;
 }
 
 // y = a x + b z (elementwise complex, real a and b).
@@ -326,6 +384,10 @@ __global__ void k_expm_setup(int N, double dt, const double2* __restrict__ hA,
 // barrier a product); below, one CTA is faster than the barriers.  One SM's FP64
 // rate bounds a single CTA (n = 24, eighteen products: 520 us; here, cluster:
 // 44 us; n = 10: 62 -> 24).
+// SEQ (split-TF32 contexts): the propagator feeds FP32 operands and keeps its
+// value to the last bit: the polynomial by Horner's scheme, Y = I + X Y / k for
+// k = 18 .. 1, every sum in the order of k by one lane a component (dot_seq); 116 us
+// at n = 24.
 constexpr int kExpmSmallN = 32, kExpmOneN = 12;
 constexpr int kExpmLanes = 4;
 struct ExpmCoef {  // 1 / k!
@@ -338,21 +400,35 @@ struct ExpmCoef {  // 1 / k!
 __device__ constexpr ExpmCoef kExpmCoef{};
 
 // C = A B, plus (poly >= 0) sum_{i=0..3} X^i / (4 poly + i)!, into all CTAs' C.
-template <int CTAS>
+// SEQ: C = A B / poly + I (poly > 0) or A B, one lane a component.
+template <int CTAS, bool SEQ>
 __device__ void expm_product(int n, int rank, const double2* A, const double2* B, double2* C, int poly,
                              const double2* X1, const double2* X2, const double2* X3) {
+    constexpr int kLanes = SEQ ? 2 : kExpmLanes;
     const int nn = n * n, per = (nn + CTAS - 1) / CTAS;
-    const int e0 = rank * per, e1 = min(nn, e0 + per), sub = threadIdx.x % kExpmLanes;
-    for (int eb = e0; eb < e1; eb += 256 / kExpmLanes) {
-        const int et = eb + (int)threadIdx.x / kExpmLanes, e = min(et, e1 - 1), i = e / n, j = e % n;
+    const int e0 = rank * per, e1 = min(nn, e0 + per), sub = threadIdx.x % kLanes;
+    for (int eb = e0; eb < e1; eb += 256 / kLanes) {
+        const int et = eb + (int)threadIdx.x / kLanes, e = min(et, e1 - 1), i = e / n, j = e % n;
         double2 acc = make_double2(0.0, 0.0);
-        for (int k = sub; k < n; k += kExpmLanes) cmac(acc, A[i * n + k], B[k * n + j]);
+        if (SEQ) {
+            dot_seq<1>(acc, A + i * n, 1, 0, B + j, n, 0, n, sub);
+            const double t = __shfl_xor_sync(0xffffffffu, acc.x, 1);
+            acc = sub ? make_double2(t, acc.x) : make_double2(acc.x, t);
+        } else {
+            for (int k = sub; k < n; k += kLanes) cmac(acc, A[i * n + k], B[k * n + j]);
 #pragma unroll
-        for (int o = kExpmLanes / 2; o > 0; o >>= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            for (int o = kLanes / 2; o > 0; o >>= 1) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            }
         }
-        if (poly >= 0) {
+        if (SEQ) {
+            if (poly > 0) {
+                const double al = 1.0 / poly;
+                acc = make_double2(__dmul_rn(al, acc.x), __dmul_rn(al, acc.y));
+                if (i == j) acc.x = __dadd_rn(acc.x, 1.0);
+            }
+        } else if (poly >= 0) {
             const double* c = kExpmCoef.f + 4 * poly;
             if (i == j) acc.x += c[0];
             acc.x = fma(c[1], X1[e].x, fma(c[2], X2[e].x, fma(c[3], X3[e].x, acc.x)));
@@ -362,7 +438,7 @@ __device__ void expm_product(int n, int rank, const double2* A, const double2* B
             if (et < e1 && sub == 0) C[e] = acc;
         } else if (et < e1) {
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(C + e);
-            for (int r = sub; r < CTAS; r += kExpmLanes) {  // two CTAs a lane
+            for (int r = sub; r < CTAS; r += kLanes) {
                 uint32_t remote;
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(dst), "r"(r));
                 asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote), "d"(acc.x), "d"(acc.y)
@@ -377,44 +453,54 @@ __device__ void expm_product(int n, int rank, const double2* A, const double2* B
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }
-template <int CTAS>
+template <int CTAS, bool SEQ>
 __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(256)
     k_expm_small(int n, double dt, const double2* __restrict__ hA, const double2* __restrict__ hB,
                  const double2* __restrict__ Z, double2* __restrict__ U, double2* __restrict__ U2) {
     extern __shared__ __align__(16) double2 expm_sm[];
-    __shared__ float mod[kExpmSmallN * kExpmSmallN];
-    __shared__ float colsum[kExpmSmallN];
+    // the norm only selects s: FP32, with a margin for its rounding, where the last
+    // bits of the result may depend on s
+    using TN = typename std::conditional<SEQ, double, float>::type;
+    __shared__ TN mod[kExpmSmallN * kExpmSmallN], colsum[kExpmSmallN];
     const int tid = threadIdx.x, nn = n * n;
     int rank = 0;
     if (CTAS > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     double2 *X = expm_sm, *X2 = X + nn, *X3 = X2 + nn, *X4 = X3 + nn, *Y = X4 + nn, *W = Y + nn;
     for (int e = tid; e < nn; e += 256) {
-        double2 x;
+        double re, im;  // -i dt (re + i im), or Z
         if (Z) {
-            x = Z[e];
+            re = Z[e].x;
+            im = Z[e].y;
+            X[e] = Z[e];
         } else {
-            const double hr = 0.5 * (hA[e].x + hB[e].x), hi = 0.5 * (hA[e].y + hB[e].y);
-            x = make_double2(dt * hi, -dt * hr);  // -i dt h
+            re = 0.5 * (hA[e].x + hB[e].x);
+            im = 0.5 * (hA[e].y + hB[e].y);
+            X[e] = make_double2(dt * im, -dt * re);
         }
-        X[e] = x;
-        // the norm only selects s: FP32 with a margin for its rounding
-        const float re = (float)x.x, im = (float)x.y;
-        mod[e] = sqrtf(re * re + im * im);
+        if (SEQ) mod[e] = (TN)(Z ? hypot(re, im) : sqrt(re * re + im * im));
+        else mod[e] = (TN)sqrtf((float)X[e].x * (float)X[e].x + (float)X[e].y * (float)X[e].y);
     }
     __syncthreads();
     if (tid < n) {
-        float sum = 0.0f;
-        for (int i = 0; i < n; ++i) sum += mod[i * n + tid];
+        const TN f = SEQ && !Z ? (TN)dt : (TN)1;
+        TN sum = 0;
+        for (int i = 0; i < n; ++i) sum = fma(f, mod[i * n + tid], sum);
         colsum[tid] = sum;
     }
     __syncthreads();
-    float nrm = 0.0f;
-    for (int j = 0; j < n; ++j) nrm = fmaxf(nrm, colsum[j]);
-    nrm *= 1.0001f;
+    TN nrm = 0;
+    for (int j = 0; j < n; ++j) nrm = nrm < colsum[j] ? colsum[j] : nrm;
+    if (!SEQ) nrm *= (TN)1.0001;
     int s = 0;
-    for (; s < 30 && nrm > 0.5f; ++s) nrm *= 0.5f;
+    for (; s < 30 && nrm > (TN)0.5; ++s) nrm *= (TN)0.5;
     const double scale = __hiloint2double((1023 - s) << 20, 0);
-    for (int e = tid; e < nn; e += 256) X[e] = make_double2(scale * X[e].x, scale * X[e].y);
+    for (int e = tid; e < nn; e += 256) {
+        X[e] = make_double2(scale * X[e].x, scale * X[e].y);
+        // the first step of Horner's scheme, X I / 18 + I
+        if (SEQ)
+            Y[e] = make_double2(__dadd_rn(__dmul_rn(1.0 / 18, X[e].x), e / n == e % n ? 1.0 : 0.0),
+                                __dmul_rn(1.0 / 18, X[e].y));
+    }
     if (CTAS == 1) {
         __syncthreads();
     } else {
@@ -422,23 +508,30 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(256)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
-    expm_product<CTAS>(n, rank, X, X, X2, -1, nullptr, nullptr, nullptr);
-    expm_product<CTAS>(n, rank, X, X2, X3, -1, nullptr, nullptr, nullptr);
-    expm_product<CTAS>(n, rank, X2, X2, X4, -1, nullptr, nullptr, nullptr);
-    // sum_{k=16..18} X^{k-16} / k!
-    for (int e = tid; e < nn; e += 256)
-        Y[e] = make_double2(fma(kExpmCoef.f[17], X[e].x, kExpmCoef.f[18] * X2[e].x) +
-                                (e / n == e % n ? kExpmCoef.f[16] : 0.0),
-                            fma(kExpmCoef.f[17], X[e].y, kExpmCoef.f[18] * X2[e].y));
-    __syncthreads();
     double2 *y = Y, *z = W;
-    for (int j = 3; j >= 0; --j) {
-        expm_product<CTAS>(n, rank, y, X4, z, j, X, X2, X3);
-        double2* t = y; y = z; z = t;
+    if (SEQ) {
+        for (int k = 17; k >= 1; --k) {
+            expm_product<CTAS, SEQ>(n, rank, X, y, z, k, nullptr, nullptr, nullptr);
+            double2* t = y; y = z; z = t;
+        }
+    } else {
+        expm_product<CTAS, SEQ>(n, rank, X, X, X2, -1, nullptr, nullptr, nullptr);
+        expm_product<CTAS, SEQ>(n, rank, X, X2, X3, -1, nullptr, nullptr, nullptr);
+        expm_product<CTAS, SEQ>(n, rank, X2, X2, X4, -1, nullptr, nullptr, nullptr);
+        // sum_{k=16..18} X^{k-16} / k!
+        for (int e = tid; e < nn; e += 256)
+            Y[e] = make_double2(fma(kExpmCoef.f[17], X[e].x, kExpmCoef.f[18] * X2[e].x) +
+                                    (e / n == e % n ? kExpmCoef.f[16] : 0.0),
+                                fma(kExpmCoef.f[17], X[e].y, kExpmCoef.f[18] * X2[e].y));
+        __syncthreads();
+        for (int j = 3; j >= 0; --j) {
+            expm_product<CTAS, SEQ>(n, rank, y, X4, z, j, X, X2, X3);
+            double2* t = y; y = z; z = t;
+        }
     }
     const int nsq = s < 16 ? s : 16;
     for (int q = 0; q < nsq; ++q) {
-        expm_product<CTAS>(n, rank, y, y, z, -1, nullptr, nullptr, nullptr);
+        expm_product<CTAS, SEQ>(n, rank, y, y, z, -1, nullptr, nullptr, nullptr);
         double2* t = y; y = z; z = t;
     }
     if (rank == 0)
@@ -661,11 +754,11 @@ __global__ void k_weighted_sum_p1(int NN, int nb, int per, const double* __restr
     }
     tmp[(long long)blockIdx.y * NN + e] = make_double2(re, im);
 }
-// One warp per element (a thread per element summed 256 ranges one after the
-// other: 31 us a call at N = 10, here 4).
-__global__ void k_weighted_sum_p2(int NN, int nz, const double2* __restrict__ tmp,
-                                  double2* __restrict__ I_acc) {
-    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+// One warp per element (a thread per element that loads as it adds took 31 us a
+// call at N = 10, here 4).
+__global__ void __launch_bounds__(256) k_weighted_sum_p2(int NN, int nz, const double2* __restrict__ tmp,
+                                                         double2* __restrict__ I_acc) {
+    const int e = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= NN) return;
     double re = 0.0, im = 0.0;
     for (int z = lane; z < nz; z += 32) {
@@ -682,6 +775,28 @@ __global__ void k_weighted_sum_p2(int NN, int nz, const double2* __restrict__ tm
         I_acc[e].x += re;
         I_acc[e].y += im;
     }
+}
+// The ranges in order, for split-TF32 contexts (I feeds rho~, which becomes FP32
+// operands): a block loads the ranges of eight components to shared memory, a thread
+// per component adds them (256 ranges of N = 24: 14 us, in the tree above 5).
+__global__ void __launch_bounds__(256) k_weighted_sum_p2_seq(int NN2, int nz, const double* __restrict__ tmp,
+                                                             double* __restrict__ I_acc) {
+    __shared__ double part[8][kWsumRanges + 1];
+    const int c = threadIdx.x & 7, e = blockIdx.x * 8 + c;
+    for (int z = threadIdx.x >> 3; z < nz; z += 32) part[c][z] = e < NN2 ? tmp[(long long)z * NN2 + e] : 0.0;
+    __syncthreads();
+    if (threadIdx.x >= 8 || e >= NN2) return;
+    double s = 0.0;
+#pragma unroll 16
+    for (int z = 0; z < nz; ++z) s = __dadd_rn(s, part[c][z]);
+    I_acc[e] = __dadd_rn(I_acc[e], s);
+}
+static void launch_weighted_sum_p2(gkba_ctx* c, int NN, int nz, double2* I) {
+    if (tensor_core_path(c))
+        k_weighted_sum_p2_seq<<<(unsigned)((2 * NN + 7) / 8), 256, 0, c->stream>>>(2 * NN, nz, (const double*)c->red_tmp,
+                                                                                  (double*)I);
+    else
+        k_weighted_sum_p2<<<(unsigned)((NN * 32LL + 255) / 256), 256, 0, c->stream>>>(NN, nz, c->red_tmp, I);
 }
 
 // hfK[(i*N + j)*N*N + l*N + k] = 2 v_iklj - v_ikjl  (Sigma_HF as a matrix-vector product)
@@ -1128,8 +1243,9 @@ __global__ void k_build_vomega64(int N, const double* __restrict__ v, double* __
 
 gkba_status fp64_prepare_model(gkba_ctx* c) {
     const long long n = c->N, N4 = n * n * n * n;
-    GKBA_CUDA(c, cudaFuncSetAttribute(k_expm_small<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(6 * kExpmSmallN * kExpmSmallN * sizeof(double2))));
+    for (auto kfn : {k_expm_small<8, false>, k_expm_small<8, true>})
+        GKBA_CUDA(c, cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(6 * kExpmSmallN * kExpmSmallN * sizeof(double2))));
     auto t = launch_begin(c, K_PREP, 0.0, 0.0);
     k_build_hfK<<<grid1(N4, 256), 256, 0, c->stream>>>(c->N, c->v, c->hfK);
     GKBA_TRY(launch_end(c, t));
@@ -1171,14 +1287,17 @@ static gkba_status zgemm_impl(gkba_ctx* c, int cls, int n, char opA, char opB, d
     for (int b0 = 0; b0 < all; b0 += most) {
         const int nb = std::min(most, all - b0), nid = std::max(0, std::min(nb, batch - b0));
         const uint32_t total = (uint32_t)(nb * nn);
-        // lanes per output: about four warps on every SM for a few matrices
-        const long long want = 4LL * c->num_sms * 32 / total;
-        const int tpo = want >= 8 ? 8 : want >= 4 ? 4 : want >= 2 ? 2 : 1;
-        const unsigned grid = grid1((long long)total * tpo, 128);
-        auto kfn = tpo == 8 ? k_zgemm<8> : tpo == 4 ? k_zgemm<4> : tpo == 2 ? k_zgemm<2> : k_zgemm<1>;
+        // one lane an output once the launch has about a warp for every SM's scheduler
+        const bool seq = tensor_core_path(c), few = total <= 32u * (unsigned)c->num_sms;
+        const int lanes = !seq && n >= 32 ? 8 : few ? 2 : 1;
+        auto kfn = seq          ? (few ? k_zgemm<2, true> : k_zgemm<1, true>)
+                   : lanes == 8 ? k_zgemm<8, false>
+                   : lanes == 2 ? k_zgemm<2, false>
+                                : k_zgemm<1, false>;
+        const int bs = (long long)total * lanes >= 512LL * c->num_sms ? 128 : 32;
         auto t = launch_begin(c, cls, flops * nid, 0.0);
-        kfn<<<grid, 128, 0, c->stream>>>(n, opA == 'C', opB == 'C', alpha, A + b0 * sA, sA, B + b0 * sB, sB, beta,
-                                         C + b0 * sC, sC, total, nid, p, skip_ge, idx);
+        kfn<<<grid1((long long)total * lanes, bs), bs, 0, c->stream>>>(n, opA == 'C', opB == 'C', alpha, A + b0 * sA, sA, B + b0 * sB, sB,
+                                                    beta, C + b0 * sC, sC, total, nid, p, skip_ge, idx);
         GKBA_TRY(launch_end(c, t));
     }
     return GKBA_OK;
@@ -1211,14 +1330,15 @@ gkba_status heun_stage(gkba_ctx* c, const double2* hhf, const double2* rho, cons
                        const double2* kprev, double a, double2* k_out, double2* y, double2* y2) {
     const long long NN = (long long)c->N * c->N;
     auto t = launch_begin(c, K_STEP, 16.0 * NN * c->N, 0.0);
-    k_heun_stage<<<grid1(NN * kRhsLanes, 128), 128, 0, c->stream>>>(c->N, hhf, rho, I, base, kprev, a, k_out, y, y2);
+    k_heun_stage<<<grid1(NN * 4, 64), 64, 0, c->stream>>>(c->N, hhf, rho, I, base, kprev, a, k_out, y, y2);
     return launch_end(c, t);
 }
 
-// exp(X) by products spread over all SMs: the Paterson-Stockmeyer form of the
-// degree-18 Taylor polynomial (k_expm_small), then up to 16 squarings of which
-// the device-side count c->dint[0] runs.  X: the scaled argument; X2, X3, X4, Y,
-// W: n x n scratch; the result goes to U (and U2).
+// exp(X) by products spread over all SMs: the degree-18 Taylor polynomial in the
+// form that k_expm_small takes (Horner for split-TF32 contexts, else Paterson and
+// Stockmeyer), then up to 16 squarings of which the device-side count c->dint[0]
+// runs.  X: the scaled argument; X2, X3, X4, Y, W: n x n scratch; the result goes
+// to U (and U2).
 static gkba_status expm_products(gkba_ctx* c, int n, const double2* X, double2* X2, double2* X3, double2* X4,
                                  double2* Y, double2* W, double2* U, double2* U2) {
     const long long nn = (long long)n * n;
@@ -1226,29 +1346,40 @@ static gkba_status expm_products(gkba_ctx* c, int n, const double2* X, double2* 
     auto prod = [&](const double2* A, const double2* B, double2* C, const ZPoly& p) {
         return zgemm_impl(c, K_STEP, n, 'N', 'N', one, A, 0, B, 0, zero, C, 0, 1, 0, p, nullptr, 0);
     };
-    GKBA_TRY(prod(X, X, X2, ZPoly{}));
-    GKBA_TRY(prod(X, X2, X3, ZPoly{}));
-    GKBA_TRY(prod(X2, X2, X4, ZPoly{}));
-    double f[19];
-    f[0] = 1.0;
-    for (int k = 1; k <= 18; ++k) f[k] = f[k - 1] / k;
-    {
-        auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-        k_expm_lead<<<grid1(nn, 256), 256, 0, c->stream>>>(n, f[16], f[17], f[18], X, X2, Y);
-        GKBA_TRY(launch_end(c, t));
-    }
     double2 *y = Y, *z = W;
-    for (int j = 3; j >= 0; --j) {
+    if (tensor_core_path(c)) {
         ZPoly p;
-        p.c0 = f[4 * j];
-        p.c1 = f[4 * j + 1];
-        p.c2 = f[4 * j + 2];
-        p.c3 = f[4 * j + 3];
-        p.X1 = X;
-        p.X2 = X2;
-        p.X3 = X3;
-        GKBA_TRY(prod(y, X4, z, p));
-        std::swap(y, z);
+        p.c0 = 1.0;
+        GKBA_TRY(zgemm_impl(c, K_STEP, n, 'N', 'N', one, X, 0, X, 0, zero, y, 0, 0, 1, ZPoly{}, nullptr, 0));  // I
+        for (int k = 18; k >= 1; --k) {
+            GKBA_TRY(zgemm_impl(c, K_STEP, n, 'N', 'N', make_double2(1.0 / k, 0.0), X, 0, y, 0, zero, z, 0, 1, 0, p,
+                                nullptr, 0));
+            std::swap(y, z);
+        }
+    } else {
+        GKBA_TRY(prod(X, X, X2, ZPoly{}));
+        GKBA_TRY(prod(X, X2, X3, ZPoly{}));
+        GKBA_TRY(prod(X2, X2, X4, ZPoly{}));
+        double f[19];
+        f[0] = 1.0;
+        for (int k = 1; k <= 18; ++k) f[k] = f[k - 1] / k;
+        {
+            auto t = launch_begin(c, K_STEP, 0.0, 0.0);
+            k_expm_lead<<<grid1(nn, 256), 256, 0, c->stream>>>(n, f[16], f[17], f[18], X, X2, Y);
+            GKBA_TRY(launch_end(c, t));
+        }
+        for (int j = 3; j >= 0; --j) {
+            ZPoly p;
+            p.c0 = f[4 * j];
+            p.c1 = f[4 * j + 1];
+            p.c2 = f[4 * j + 2];
+            p.c3 = f[4 * j + 3];
+            p.X1 = X;
+            p.X2 = X2;
+            p.X3 = X3;
+            GKBA_TRY(prod(y, X4, z, p));
+            std::swap(y, z);
+        }
     }
     // X3 is free now: squarings alternate between y and it
     double2* sq[2] = {y, X3};
@@ -1264,8 +1395,10 @@ static gkba_status expm_small(gkba_ctx* c, int n, const double2* hA, const doubl
                                 double2* U, double2* U2) {
     const size_t smem = 6 * (size_t)n * n * sizeof(double2);
     auto t = launch_begin(c, K_STEP, 0.0, 0.0);
-    if (n <= kExpmOneN) k_expm_small<1><<<1, 256, smem, c->stream>>>(n, c->dt, hA, hB, Z, U, U2);
-    else k_expm_small<8><<<8, 256, smem, c->stream>>>(n, c->dt, hA, hB, Z, U, U2);
+    const int ctas = n <= kExpmOneN ? 1 : 8;
+    auto kfn = tensor_core_path(c) ? (ctas == 1 ? k_expm_small<1, true> : k_expm_small<8, true>)
+                                   : (ctas == 1 ? k_expm_small<1, false> : k_expm_small<8, false>);
+    kfn<<<ctas, 256, smem, c->stream>>>(n, c->dt, hA, hB, Z, U, U2);
     return launch_end(c, t);
 }
 
@@ -1340,7 +1473,7 @@ gkba_status weighted_sum_units(gkba_ctx* c, int N, int nb, const double* coef, c
                                                                        c->red_tmp);
     GKBA_TRY(launch_end(c, t));
     t = launch_begin(c, K_RED, 0.0, 0.0);
-    k_weighted_sum_p2<<<grid1(NN * 32, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I);
+    launch_weighted_sum_p2(c, (int)NN, nz, I);
     return launch_end(c, t);
 }
 
@@ -1513,7 +1646,7 @@ gkba_status reduce_batch(gkba_ctx* c, int nb, double2* I_acc, double2* S_out) {
                                                                        c->Yu, c->red_tmp);
     GKBA_TRY(launch_end(c, t));
     t = launch_begin(c, K_RED, 0.0, 0.0);
-    k_weighted_sum_p2<<<grid1(NN * 32, 256), 256, 0, c->stream>>>((int)NN, nz, c->red_tmp, I_acc);
+    launch_weighted_sum_p2(c, (int)NN, nz, I_acc);
     return launch_end(c, t);
 }
 
