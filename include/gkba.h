@@ -63,7 +63,11 @@ typedef enum {
 } gkba_status;
 
 typedef enum {
-    GKBA_FP64 = 0,       /* every contraction in FP64 on the CUDA cores */
+    GKBA_FP64 = 0,       /* FP64 in and out.  The contractions of a general v run as exact
+                            products of 8-bit digits on the FP16 tensor cores where a
+                            result's error is then below about 3 2^-53 (rms) of the sum
+                            of its terms' absolute values, and as FP64 FMAs elsewhere:
+                            componentwise the accuracy of FMA chains */
     GKBA_SPLIT_TF32 = 1, /* contractions on tcgen05 tensor cores: FP32 data,
                             3 TF32 products (hi*hi + hi*lo + lo*hi), FP32
                             accumulation in short tensor-memory windows (see

@@ -1256,13 +1256,8 @@ gkba_status fp64_prepare_model(gkba_ctx* c) {
     t = launch_begin(c, K_PREP, 0.0, 0.0);
     k_build_vK64<<<grid1(N4, 256), 256, 0, c->stream>>>(c->N, c->v, c->vK64);
     GKBA_TRY(launch_end(c, t));
-    // stage S4 reads only the digit images of vK
     GKBA_TRY(oz_prepare(c));
-    GKBA_TRY(oz_slice(c, c->vK64, n * n * n, 0, c->N, n * n * n, 1, c->vKimg));
-    GKBA_CUDA(c, cudaStreamSynchronize(c->stream));
-    cudaFree(c->vK64);
-    c->vK64 = nullptr;
-    return GKBA_OK;
+    return oz_slice(c, c->vK64, n * n * n, 0, c->N, n * n * n, 1, c->vKimg);
 }
 
 gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz,
@@ -1273,7 +1268,7 @@ gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, l
     if (oz_img_bytes(Nc, Ktot) * nzB > c->ozimg_bytes)
         return fail(c, GKBA_ESTATE, "digit images of %d operands of %d x %lld do not fit", nzB, Nc, Ktot);
     GKBA_TRY(oz_slice(c, B, ldb, sBz, Nc, Ktot, nzB, c->ozimg));
-    return oz_gemm(c, cls, A, lda, sAz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
+    return oz_gemm(c, cls, A, lda, sAz, B, ldb, sBz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
 }
 
 static gkba_status zgemm_impl(gkba_ctx* c, int cls, int n, char opA, char opB, double2 alpha,
@@ -1700,7 +1695,7 @@ gkba_status fp64_final(gkba_ctx* c, int nb) {
     const StageMap m{0, 0, 1, 0, R, (int)R, 1, N};
     const long long max_z = (long long)(c->part_bytes / (N * R * 8));
     const int nz = oz_items(c, (int)R, N, N3, max_z);
-    GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m, fl, by));
+    GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m, fl, by));
     return reduce_partials_launch(c, nb, nz, N * R, R, c->part, false, c->Su);
 }
 

@@ -81,7 +81,7 @@ struct gkba_ctx {
 
     // FP64 contraction operands (natural N)
     double* wS64 = nullptr;  // [j][m][q][s] = w_mqsj
-    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn, until vKimg holds its digits
+    double* vK64 = nullptr;  // [i][n][r][p] = v_irpn
     bool oz = false;         // FP64 with a general v: digit images are needed (oz_gemm.cu)
     void* vKimg = nullptr;   // digit images of vK (oz)
 
@@ -237,8 +237,8 @@ gkba_status oz_prepare(gkba_ctx* c);
 gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz, int Nc, long long K, int nz,
                      void* img);
 int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items);
-gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const void* img,
-                    int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
+gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const double* B,
+                    long long ldb, long long sBz, const void* img, int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
                     long long sOitem, StageMap map, double flops, double bytes);
 // Stage S4 of the FP64 chain on the X3 of nb units in X13, with its reduction: S_u -> c->Su.
 gkba_status fp64_final(gkba_ctx* c, int nb);

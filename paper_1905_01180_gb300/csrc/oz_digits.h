@@ -10,9 +10,17 @@
 // of two windows are grouped by level l = i + j, weight 2^(96 - 8 l); a level's
 // sum over a window of at most 96 K is an integer below 7 96 2^14 < 2^24, exact
 // in the tensor core's FP32 accumulator.  Levels 0 .. 7 are kept (34 of the 49
-// digit products); the dropped ones are below 2^-60 of the window's largest
-// product, less than the rounding of X (2^-54 of the row's largest element).
-// Elements below 2^-1012 count as zero (the floor of E).
+// digit products); the dropped ones sum to at most 2^-57.6 of the window's largest
+// product a term (five digit products of up to 2^14 at level 8, of 2^108), less
+// than the rounding of X (2^-55 of the row's largest element).
+//
+// That error is normwise: 2^-55 of the largest elements times the other operand,
+// whatever the elements that meet.  Where small elements meet large ones, or zeros,
+// it can exceed the rounding of an FMA chain, which is relative to sum |x y|, by any
+// factor.  So every window result carries M = sum |d_0(x)| |d_0(y)| (one more MMA)
+// and is taken only if its error is small against M (oz_accept); the others are
+// summed again by FMAs.  Results that leave the normal range and rows with Inf, NaN
+// or nothing above 2^-958 go the same way.
 #pragma once
 
 #include <cmath>
@@ -54,6 +62,26 @@ GKBA_OZ_HD uint64_t oz_digits(uint32_t hi, uint32_t lo, uint32_t emax) {
     const uint64_t neg = (uint64_t)((int64_t)((uint64_t)hi << 32) >> 63);
     return (t ^ neg) + 0x8080808080808080ull;
 }
+
+// Magnitude of an element for M, as FP16 bits: |d_0|, its last bit set for every
+// element but zero, so that M = 0 means that no two nonzero elements meet.  d0: the
+// FP16 bits of d_0.
+GKBA_OZ_HD uint32_t oz_nonzero(uint32_t hi, uint32_t lo) {
+    const uint32_t any = (hi & 0x7FFFFFFFu) | lo;
+    return any < 1u ? any : 1u;
+}
+GKBA_OZ_HD uint32_t oz_magnitude(uint32_t d0, uint32_t nonzero) { return (d0 & 0x7FFFu) | nonzero; }
+
+// Acceptance of a window result.  With unit errors of 2^-55 / sqrt(3) an element its
+// error is e = 2^-55 / sqrt(3) sqrt(sx + sy) of the largest product, sx = sum (d_0(x) / 64)^2,
+// and |x|.|y| is M / 64^2 of it: M^2 >= c (sx + sy) bounds e by 2^-53 590 / sqrt(c) of
+// sum |x y|, 3.3 2^-53 here (an FMA chain's rms error is 0.5 to 2 2^-53 of it).  Well
+// scaled operands stay far below the bound (0.2 to 0.5) and nearly all of their results
+// are taken: of random ones at N = 10, 24 and 33 all but 6e-4, 2e-6 and 4e-7 in stage S1
+// and 2e-4, 0 and 0 in S2; twice the constant would turn down 4e-3 and 3e-3 at N = 10
+// and cost 20 % of its time.
+constexpr float kOzAccept = 32768.0f;
+GKBA_OZ_HD bool oz_accept(float M, float cs) { return M * M >= cs; }  // cs = c (sx + sy)
 
 // Digit i (0 = leading) of an oz_digits word.
 GKBA_OZ_HD int oz_digit(uint64_t t, int i) { return (int)((t >> (8 * (7 - i))) & 0xFF) - 128; }
@@ -128,8 +156,8 @@ GKBA_OZ_HD uint64_t oz_pack(uint32_t hi, uint32_t lo, int Es, const OzMul& k, ui
     return ((uint64_t)rh << 32) | (uint32_t)w;
 }
 GKBA_OZ_HD bool oz_packed(uint32_t ha, uint32_t e1) { return ha != 0u && e1 <= 2045u; }
-// W as FP64 in every case: Es >= kOzNonFinite / 2 (a non-finite operand) gives
-// NaN, results below the normal range zero.
+// W as FP64 in every case, to check the packing above against: Es >= kOzNonFinite / 2
+// (a non-finite operand) gives NaN, results below the normal range zero.
 GKBA_OZ_HD uint64_t oz_pack_any(uint32_t hi, uint32_t lo, int Es) {
     const uint32_t neg = (uint32_t)((int32_t)hi >> 31);
     hi ^= neg;

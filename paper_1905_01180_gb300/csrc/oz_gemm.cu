@@ -8,16 +8,21 @@
 // (k_gemm64_stage) is bound by them at 1.2 TFLOP/s.  Here every element is
 // split into seven 8-bit digits (oz_digits.h), the digit products run as FP16
 // MMAs whose FP32 sums are exact integers, and the epilogue puts a result
-// together with integer instructions only.  The result is closer to the exact
-// sum than the FMA chain's (tests/test_oz_digits.py; whole Heun steps and
-// self-energies: 1.1-2.0e-15 from 64-bit references where the FMA chain had
-// 1.2-2.8e-15).  Whole calls, FMA chain -> here: Heun step at N = 24, 301 points
-// 309 -> 15.8 ms; 40 self-energies at N = 33 78 -> 2.8 ms; Heun step at N = 10,
-// 501 points 23.8 -> 1.4 ms; three time-linear steps at N = 48 137 -> 11.4 ms.
+// together with integer instructions only.  Results whose error that would leave
+// large against sum |x y| (graded rows, blocks that hardly couple) are found by an
+// eighth MMA and summed again by FMAs, so that the path is as accurate as FMA chains
+// for operands of any scaling (oz_accept; tests/test_oz_graded.py).
 //
-// What bounds it: the integer instructions of the epilogue and the converter
-// (about 64 a result and 47 an element; at N = 24 the integer pipe is 52 % busy,
-// the tensor pipe 27 %, DRAM 25 %).
+// Whole calls, FMA chain -> here: Heun step at N = 24, 301 points 309 -> 18.2 ms; 40
+// self-energies at N = 33 78 -> 3.6 ms; Heun step at N = 10, 501 points 23.8 -> 1.7 ms.
+// Without the check of the results: 15.8, 2.8 and 1.4 ms.  What is summed again costs
+// most for matrices near a diagonal or nearly real (a propagation's start; three
+// time-linear steps at N = 48 137 -> 27 ms, 12 without the check) and at worst, N = 24
+// with imaginary parts of 1e-3, takes 0.6 of the FMA chain's time (50 -> 30 ms for 200
+// self-energies; 13 ms where rows and columns span 1e-6 .. 1e6).
+//
+// What bounds it: the latency of two chains of instructions that are each half busy,
+// the epilogue's (about 70 a result) and the converter's (about 53 an element).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -32,8 +37,10 @@ namespace {
 
 constexpr int kOzBM = 128;       // rows per tile (tensor-memory lanes)
 constexpr int kOzLbo = kOzBM * 16 + 32;  // bytes between the 8-wide K chunks of a digit plane of A
-constexpr int kOzMaxNB = 32;     // columns per accumulator: 8 levels x 32 = 256 TMEM columns
-constexpr int kOzSub = 6;        // 8-wide K chunks of one B pipeline stage (48 K)
+constexpr int kOzMaxNB = 24;     // columns per accumulator: (8 levels + M) x 24, at most 256 TMEM columns
+constexpr int kOzPlanes = kOzSlices + 1;  // of A: digits, magnitudes
+constexpr int kOzRows = kOzSlices + 2;    // of B's image, times NB: digits, zeros, magnitudes
+constexpr int kOzMaxSub = 6;     // 8-wide K chunks of one B pipeline stage, at most (48 K)
 constexpr int kOzRing = 8;       // exponent rings: more than the windows and accumulators in flight
 // Warps of the kernel: epilogue, converter, then producer, MMA issuer and two
 // that fill the warpgroup.
@@ -42,17 +49,20 @@ constexpr int oz_epi_warps(bool multi) { return multi ? 8 : 16; }
 constexpr int oz_threads(bool multi) { return 32 * (oz_epi_warps(multi) + kOzConvWarps + (multi ? 2 : 4)); }
 constexpr size_t kOzSmemMax = 227 * 1024;
 constexpr int kOzMaxCols = 256;  // 2 N, N <= 128
-// column offsets, row and column exponent rings, barriers
-constexpr int kOzMisc = kOzMaxCols * 4 + kOzRing * (kOzBM + kOzMaxNB) * 4 + 256;
+// column offsets, rings of row and column exponents and square sums, barriers
+constexpr int kOzMisc = kOzMaxCols * 4 + kOzRing * 2 * (kOzBM + kOzMaxNB) * 4 + 256;
 
-// Shape of one GEMM: column blocks of NB (a multiple of 8, at most 32) and K
-// windows of kw (a multiple of 16, at most 96).
+// Shape of one GEMM: column blocks of NB (a multiple of 8, at most 24) and K
+// windows of kw (a multiple of 16): one of at most 96, or several of at most 64,
+// which leave room for longer B stages (S4 at N = 24 and 48, windows of 96, 80 and
+// 64: 2.42, 2.48, 2.26 and 6.43, 6.59, 6.00 ms).
+constexpr int kOzLongKw = 64;
 struct OzGeom {
     int Nc, NB, nblk, kw, nwin;
     long long K;
-    long long win_bytes() const { return (long long)nblk * (kw / 8) * (8 * NB * 16); }  // digits of a window
-    long long img_bytes() const { return nwin * win_bytes(); }                        // of one z
-    long long exps() const { return (long long)nwin * nblk * NB; }                    // column exponents
+    long long win_bytes() const { return (long long)nblk * (kw / 8) * (kOzRows * NB * 16); }  // digits of a window
+    long long img_bytes() const { return nwin * win_bytes(); }                               // of one z
+    long long exps() const { return 2LL * nwin * nblk * NB; }  // column exponents and square sums
 };
 
 OzGeom oz_geom(int Nc, long long K) {
@@ -61,7 +71,8 @@ OzGeom oz_geom(int Nc, long long K) {
     g.K = K;
     g.nblk = (Nc + kOzMaxNB - 1) / kOzMaxNB;
     g.NB = ((Nc + g.nblk - 1) / g.nblk + 7) / 8 * 8;
-    g.nwin = (int)((K + kOzMaxKw - 1) / kOzMaxKw);
+    const int most = K <= kOzMaxKw ? kOzMaxKw : kOzLongKw;
+    g.nwin = (int)((K + most - 1) / most);
     g.kw = (int)(((K + g.nwin - 1) / g.nwin + 15) / 16 * 16);
     g.nwin = (int)((K + g.kw - 1) / g.kw);
     return g;
@@ -71,9 +82,11 @@ struct OzParams {
     const double* A;
     long long lda, sAz;
     int M;
-    const uint8_t* img;  // digit images of B: [z][window][block][chunk][8 NB rows][16 B]
+    const double* B;     // for the results that are summed again
+    long long ldb, sBz;
+    const uint8_t* img;  // digit images of B: [z][window][block][chunk][9 NB rows][16 B]
     long long img_z;     // bytes per z (0: shared)
-    const int* ecol;     // exponents of B's columns: [z][window][block NB]
+    const int* ecol;     // exponents and c x square sums of B's columns: [z][window][block][2][NB]
     long long ecol_z;
     double* out;
     long long sOz;
@@ -84,17 +97,25 @@ struct OzParams {
     int nitem, wper;     // split K: items per row tile, windows per item
     long long sOitem;
     long long tiles;     // z x item x row tile
-    uint32_t mma_id[kOzSlices], mma_col[kOzSlices];  // per digit of A: instruction descriptor, accumulator column
+    // per plane of A: instruction descriptor, accumulator column, first row of B
+    uint32_t mma_id[kOzPlanes], mma_col[kOzPlanes], mma_row[kOzPlanes];
     OzMul mul;
-    int na, nbs;         // A and B pipeline stages
+    int na, nbs, sub;    // A and B pipeline stages, chunks of a B stage
     int* err;
 };
+
+// c x the square sum of a row, infinite (nothing is accepted) for one at the
+// exponent's floor, whose digits lose more than the criterion knows of.
+__device__ __forceinline__ float oz_scaled_squares(float sq, uint32_t emax) {
+    return emax <= kOzExpMin ? __int_as_float(0x7F800000) : kOzAccept * sq;
+}
 
 // ---------------------------------------------------------------------------
 // Digit images of B.  One warp per (z, window, column): FP16 digits in the
 // K-major core-matrix layout the MMA reads (8 rows x 16 bytes, no swizzle):
 // row j NB + c holds digit j of column c of the block, rows 7 NB .. 8 NB - 1
-// are zero (they clear the accumulator's last level).  A window's K is
+// are zero (they clear the accumulator's last level), rows 8 NB .. 9 NB - 1 its
+// magnitudes (oz_magnitude).  A window's K is
 // permuted as the converter of A reads it: of the no chunks of the window,
 // chunk p holds k = p + no q, q = 0..7 (K odd), or the pairs 2 (p + no q) + {0, 1},
 // q = 0..3 (K even, 16-byte loads).
@@ -129,21 +150,35 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
             emax = max(emax, x[u][h].y & kOzExpMask);
         }
     emax = __reduce_max_sync(0xffffffffu, emax);
-    if (lane == 0) ecol[z * ecol_z + (long long)w * ncp + col] = oz_exponent(emax);
     const int blk = col / NB, c = col % NB;
-    uint8_t* o = img + z * img_z + ((long long)w * nblk + blk) * (kw / 8) * (8 * NB * 16);
+    uint8_t* o = img + z * img_z + ((long long)w * nblk + blk) * (kw / 8) * (kOzRows * NB * 16);
+    float sq = 0.0f;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
         const int p = (lane >> 2) + 8 * u;
         if (p >= no) continue;
         const uint64_t t0 = oz_digits(x[u][0].y, x[u][0].x, emax), t1 = oz_digits(x[u][1].y, x[u][1].x, emax);
-        uint8_t* op = o + (long long)p * (8 * NB * 16) + c * 16 + (lane & 3) * 4;
+        uint8_t* op = o + (long long)p * (kOzRows * NB * 16) + c * 16 + (lane & 3) * 4;
 #pragma unroll
         for (int j = 0; j < kOzSlices; ++j) {
             const __half2 d = __halves2half2(__int2half_rn(oz_digit(t0, j)), __int2half_rn(oz_digit(t1, j)));
             *reinterpret_cast<__half2*>(op + j * NB * 16) = d;
+            if (j > 0) continue;
+            const uint32_t b = *reinterpret_cast<const uint32_t*>(&d);
+            *reinterpret_cast<uint32_t*>(op + (kOzSlices + 1) * NB * 16) =
+                oz_magnitude(b, oz_nonzero(x[u][0].y, x[u][0].x)) |
+                oz_magnitude(b >> 16, oz_nonzero(x[u][1].y, x[u][1].x)) << 16;
+            const float d0 = (float)oz_digit(t0, 0) * (1.0f / 64.0f), d1 = (float)oz_digit(t1, 0) * (1.0f / 64.0f);
+            sq = fmaf(d0, d0, fmaf(d1, d1, sq));
         }
         *reinterpret_cast<uint32_t*>(op + kOzSlices * NB * 16) = 0u;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
+    if (lane == 0) {
+        int* e = ecol + z * ecol_z + ((long long)w * nblk + blk) * (2 * NB) + c;
+        e[0] = oz_exponent(emax);
+        e[NB] = __float_as_int(oz_scaled_squares(sq, emax));
     }
 }
 
@@ -158,17 +193,22 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
 // more of them (N = 33: 78 -> 68 us a self-energy).
 //
 // A: the converter reads a window's rows (FP64, through L1), takes the row's
-// largest exponent, and writes the seven digit planes [chunk][128 rows][16 B]
-// to shared memory (na stages).  The four lanes of a row read 64 contiguous
+// largest exponent, and writes the seven digit planes and the magnitudes
+// [chunk][128 rows][16 B] to shared memory (na stages).  The four lanes of a row read 64 contiguous
 // bytes; chunks are kOzLbo apart, 32 bytes off a multiple of 128, so that eight
 // lanes (two rows, four chunks) store to different banks.  B: bulk copies of pre-split images, one stage
-// per 48 K of a 32-column block (nbs stages).  Digit i of A times the stacked
+// per 16 to 48 K of a 24-column block (nbs stages).  Digit i of A times the stacked
 // digits 0 .. of B is one MMA of N = (digits) x NB columns at column offset
 // i NB of the accumulator: level l = i + j lands in columns [l NB, (l+1) NB),
-// so 34 digit products take seven MMAs per K step, none narrower than 32.
-// N is rounded up to 16, the columns past level 7 are never read.  The first
-// MMA covers all 8 NB columns (B's image ends in NB zero rows) and clears the
-// accumulator.  Two accumulators (TMEM columns 0 and 256).
+// so 34 digit products take seven MMAs per K step.  N is rounded up to 16, the 8
+// columns past level 7 that this adds to are never read.  The first MMA covers all 8 NB columns
+// (B's image has NB zero rows) and clears them.  An eighth MMA sums the magnitudes,
+// in NB columns from oz_mag_col on.  Two accumulators (TMEM columns 0 and 256).
+//
+// A result that oz_accept turns down, or that leaves the normal range, is summed
+// again by FMAs in the epilogue, from A and B in memory (oz_again: eight lanes a row;
+// with every lane on its own row a warp pays for 32 rows whenever one is wanted, and
+// the N = 48 propagation took 46 ms instead of 27).
 //
 // One window (K <= 96, stages S1-S3 up to N = 48): a row tile is converted
 // once and multiplied with every column block.  Longer K: per block and
@@ -242,6 +282,41 @@ __device__ __forceinline__ uint32_t desc_plain(uint32_t saddr, uint32_t lbo) {
     return ((saddr & 0x3FFFFu) >> 4) | (lbo >> 4) << 16;
 }
 
+// Accumulator column of the magnitudes' sums: past the levels and the columns that
+// an MMA of an odd number of 8-column groups adds to.
+__host__ __device__ constexpr int oz_mag_col(int NB) { return kOzLevels * NB + (NB & 8); }
+static_assert(oz_mag_col(kOzMaxNB) + 32 <= 256, "accumulator columns");
+
+// sum_k A[row][k] B[k] by FMAs for the rows (lanes) of a mask, four at a time: eight
+// lanes share a row's K, so that its loads are coalesced and the few rows of a warp do
+// not cost as much as all 32.  The result goes to the row's lane.
+__device__ __forceinline__ void oz_again(uint32_t rows, int lane, const double* __restrict__ a, long long lda,
+                                         const double* __restrict__ b, int Kw, uint64_t& r) {
+    while (rows != 0u) {
+        uint32_t pick[4], left = rows;
+        int mine = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            pick[i] = left != 0u ? (uint32_t)__ffs((int)left) - 1u : 32u;
+            left &= left - 1u;
+            if ((lane >> 3) == i) mine = (int)min(pick[i], 31u);
+        }
+        if (((rows >> mine) & 1u) == 0u) mine = (int)pick[0];
+        const double* ar = a + (long long)mine * lda;
+        double d = 0.0;
+#pragma unroll 2
+        for (int k = lane & 7; k < Kw; k += 8) d = fma(__ldg(ar + k), __ldg(b + k), d);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double x = __shfl_sync(0xffffffffu, d, 8 * i);
+            if (pick[i] == (uint32_t)lane) r = (uint64_t)__double_as_longlong(x);
+        }
+        rows = left;
+    }
+}
+
 // Position of a tile in a CTA's range (row tiles fastest, then split-K items,
 // then units), advanced without divisions.
 struct OzPos {
@@ -301,15 +376,16 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
     constexpr int kEpi = oz_epi_warps(MULTI), kWorkers = kEpi + kOzConvWarps;
     constexpr int KW = 8 * NO;                                    // K of a window
     constexpr uint32_t kPlane = (uint32_t)(NO * kOzLbo);          // one digit plane of A
-    constexpr uint32_t kAStage = kOzSlices * kPlane;
-    const uint32_t brow = (uint32_t)(8 * p.NB * 16);              // one 8-wide K chunk of a block's image
-    const uint32_t bstage = (uint32_t)(NO < kOzSub ? NO : kOzSub) * brow;
+    constexpr uint32_t kAStage = kOzPlanes * kPlane;
+    const uint32_t brow = (uint32_t)(kOzRows * p.NB * 16);        // one 8-wide K chunk of a block's image
+    const uint32_t bstage = (uint32_t)p.sub * brow;
     uint8_t* sA = smem;
     uint8_t* sB = sA + (size_t)p.na * kAStage;
     uint32_t* sCol = (uint32_t*)(sB + (size_t)p.nbs * bstage);  // output offset of each column
     int* sExp = (int*)(sCol + kOzMaxCols);
-    int* sEcol = sExp + kOzRing * kOzBM;  // column exponents of an accumulator
-    uint64_t* bars = (uint64_t*)(sEcol + kOzRing * kOzMaxNB);
+    float* sSq = (float*)(sExp + kOzRing * kOzBM);        // c x square sums of the rows
+    int* sEcol = (int*)(sSq + kOzRing * kOzBM);           // column exponents and square sums of an accumulator
+    uint64_t* bars = (uint64_t*)(sEcol + kOzRing * 2 * kOzMaxNB);
     constexpr int AFULL = 0, AEMPTY = 2, BFULL = 4, BEMPTY = 8, ACCF = 12, ACCE = 14, DRAIN = 16, NBARS = 17;
     uint32_t* tmem_slot = (uint32_t*)(bars + NBARS);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
@@ -389,39 +465,55 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
                     const int col0 = blk * p.NB + cb;
                     if (!MULTI) ++blk;
                     if (!MULTI && ab != grp) continue;
-                    const int* ec = sEcol + (accseq % kOzRing) * kOzMaxNB + cb;
+                    const int* ec = sEcol + (accseq % kOzRing) * 2 * kOzMaxNB + cb;
                     if (!oz_warp_wait(bar(ACCF + ab), (accseq >> 1) & 1, abort_flag, p.err, 41)) { ok = false; break; }
                     tc_fence_after();
                     const int Ea = sExp[(aseq % kOzRing) * kOzBM + q * 32 + lane] - 1014;
-                    uint32_t tc[kOzLevels];
+                    const float sqa = sSq[(aseq % kOzRing) * kOzBM + q * 32 + lane];
+                    uint32_t tc[kOzLevels + 1];
 #pragma unroll
-                    for (int l = 0; l < kOzLevels; ++l) tc[l] = lane_base + (uint32_t)(ab * 256 + cb + l * p.NB);
+                    for (int l = 0; l <= kOzLevels; ++l)
+                        tc[l] = lane_base + (uint32_t)(ab * 256 + cb + (l < kOzLevels ? l * p.NB : oz_mag_col(p.NB)));
 #pragma unroll(MULTI ? kOzMaxNB / 8 : 1)
                     for (int j = 0; j < (MULTI ? kOzMaxNB / 2 : half); j += 4) {  // four columns at a time
                         if (MULTI && j >= half) continue;
-                        uint32_t v[kOzLevels][4];
+                        uint32_t v[kOzLevels + 1][4];
 #pragma unroll
-                        for (int l = 0; l < kOzLevels; ++l) tmem_ld4(tc[l] + (uint32_t)j, v[l]);
+                        for (int l = 0; l <= kOzLevels; ++l) tmem_ld4(tc[l] + (uint32_t)j, v[l]);
                         const int4 e4 = *reinterpret_cast<const int4*>(ec + j);
+                        const float4 s4 = *reinterpret_cast<const float4*>(ec + p.NB + j);
                         const int Es[4] = {Ea + e4.x, Ea + e4.y, Ea + e4.z, Ea + e4.w};
+                        const float cs[4] = {sqa + s4.x, sqa + s4.y, sqa + s4.z, sqa + s4.w};
                         tmem_wait_ld();
                         // four independent chains; the rare cases in a second pass
-                        uint32_t hi[4], lo[4], hmin = 0xffffffffu, emax = 0u;
+                        uint32_t bad = 0u;
                         uint64_t r[4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             float a[kOzLevels];
 #pragma unroll
                             for (int l = 0; l < kOzLevels; ++l) a[l] = __uint_as_float(v[l][k]);
-                            uint32_t ha, e1;
-                            oz_sum(a, mul, hi[k], lo[k]);
-                            r[k] = oz_pack(hi[k], lo[k], Es[k], mul, ha, e1);
-                            hmin = min(hmin, ha);
-                            emax = max(emax, e1);
+                            uint32_t hi, lo, ha, e1;
+                            oz_sum(a, mul, hi, lo);
+                            r[k] = oz_pack(hi, lo, Es[k], mul, ha, e1);
+                            if (!(oz_packed(ha, e1) && oz_accept(__uint_as_float(v[kOzLevels][k]), cs[k]))) bad |= 1u << k;
                         }
-                        if (!oz_packed(hmin, emax)) {
+                        if (!rok) bad = 0u;
+                        if (__any_sync(0xffffffffu, bad != 0u)) {
+                            const long long k0 = MULTI ? (long long)(T.w0 + wi) * KW : 0;
+                            const int Kw = MULTI ? (int)min((long long)KW, p.K - k0) : (int)p.K;
+                            const double* ar = p.A + T.z * p.sAz + (long long)(T.mt * kOzBM + q * 32) * p.lda + k0;
+                            const double* br = p.B + T.z * p.sBz + (long long)(col0 + j) * p.ldb + k0;
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) r[k] = oz_pack_any(hi[k], lo[k], Es[k]);
+                            for (int k = 0; k < 4; ++k, br += p.ldb) {
+                                bool again = ((bad >> k) & 1u) != 0u && col0 + j + k < p.Nc;
+                                // M = 0: no two nonzero elements meet
+                                if (again && v[kOzLevels][k] == 0u && Es[k] < kOzNonFinite / 2) {
+                                    r[k] = 0ull;
+                                    again = false;
+                                }
+                                oz_again(__ballot_sync(0xffffffffu, again), lane, ar, p.lda, br, Kw, r[k]);
+                            }
                         }
                         if (MULTI) {
 #pragma unroll
@@ -550,9 +642,11 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const uint64_t d = oz_digits(x[i][q].y, x[i][q].x, E);
-                    x[i][q] = make_uint2((uint32_t)d, (uint32_t)(d >> 32));
+                    // the unused last byte says whether the element is zero
+                    x[i][q] = make_uint2(((uint32_t)d & 0xFFFFFF00u) | oz_nonzero(x[i][q].y, x[i][q].x), (uint32_t)(d >> 32));
                 }
             }
+            float S0 = 0.0f, S1 = 0.0f;  // square sums of the rows
             const int as = p.na == 2 ? (int)(aseq & 1) : 0;
             const uint32_t aph = (p.na == 2 ? aseq >> 1 : aseq) & 1;
             if (pass == 0 && !oz_warp_wait(bar(AEMPTY + as), aph ^ 1, abort_flag, p.err, 42)) break;
@@ -564,7 +658,8 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
                     const int rg = kBoth ? (c >= no ? 1 : 0) : pass;
                     const int pc = kBoth ? c - rg * no : c;
                     uint8_t* o = ap + pc * kOzLbo + rg * 128;
-// the same byte of two elements side by side, two digits at a
+                    uint32_t d0[4];
+                    // the same byte of two elements side by side, two digits at a
                     // time, then each digit as FP16 1024 + byte, minus 1152
 #pragma unroll
                     for (int w2 = 0; w2 < 4; ++w2) {  // bytes (7,6) (5,4) (3,2) (1,-)
@@ -579,18 +674,43 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
                         }
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {
-                            if (2 * w2 + k >= kOzSlices) continue;
                             uint32_t d[4];
+                            if (2 * w2 + k == kOzSlices) {  // magnitudes
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) d[q] = (d0[q] & 0x7FFF7FFFu) | (v[k][q] & 0x00010001u);
+                                *reinterpret_cast<uint4*>(o + kOzSlices * kPlane) = make_uint4(d[0], d[1], d[2], d[3]);
+                                continue;
+                            }
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 const __half2 hd = __hsub2(*reinterpret_cast<const __half2*>(&v[k][q]),
                                                            __half2half2(__ushort_as_half(0x6480)));
                                 d[q] = *reinterpret_cast<const uint32_t*>(&hd);
+                                if (2 * w2 + k == 0) d0[q] = d[q];
                             }
                             *reinterpret_cast<uint4*>(o + (2 * w2 + k) * kPlane) = make_uint4(d[0], d[1], d[2], d[3]);
                         }
                     }
+                    __half2 sq = __float2half2_rn(0.0f);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const __half2 h = *reinterpret_cast<const __half2*>(&d0[q]);
+                        sq = __hfma2(__hmul2(h, __float2half2_rn(1.0f / 4096.0f)), h, sq);
+                    }
+                    const float f = __low2float(sq) + __high2float(sq);
+                    if (kBoth && rg) S1 += f;
+                    else S0 += f;
                 }
+            }
+#pragma unroll
+            for (int d = 1; d < 4; d <<= 1) {
+                S0 += __shfl_xor_sync(0xffffffffu, S0, d);
+                if (kBoth) S1 += __shfl_xor_sync(0xffffffffu, S1, d);
+            }
+            if (s == 0) {
+                float* ss = sSq + (aseq % kOzRing) * kOzBM + 16 * cw + r8;
+                ss[kBoth ? 0 : 8 * pass] = oz_scaled_squares(S0, E0);
+                if (kBoth) ss[8] = oz_scaled_squares(S1, E1);
             }
             // next pass
             if (pass == NPASS - 1) {
@@ -632,17 +752,17 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
                         const int w = T.w0 + wi;
                         const int no = oz_chunks<NO, MULTI>(p, w);
                         const uint8_t* src = p.img + T.z * p.img_z + ((long long)w * p.nblk + blk) * NO * brow;
-                        for (int c0 = 0; c0 < no; c0 += kOzSub, ++bseq) {
+                        for (int c0 = 0; c0 < no; c0 += p.sub, ++bseq) {
                             const int st = (int)(bseq % (uint32_t)p.nbs);
                             if (!oz_wait(bar(BEMPTY + st), ((bseq / (uint32_t)p.nbs) & 1) ^ 1, abort_flag, p.err, 43, 300)) {
                                 ok = false;
                                 break;
                             }
-                            const uint32_t bytes = (uint32_t)min(kOzSub, no - c0) * brow;
-                            mbar_expect_tx(bar(BFULL + st), bytes + (c0 == 0 ? p.NB * 4u : 0u));
+                            const uint32_t bytes = (uint32_t)min(p.sub, no - c0) * brow;
+                            mbar_expect_tx(bar(BFULL + st), bytes + (c0 == 0 ? p.NB * 8u : 0u));
                             if (c0 == 0)
-                                bulk_load(smem_u32(sEcol + (accseq % kOzRing) * kOzMaxNB),
-                                          p.ecol + T.z * p.ecol_z + ((long long)w * p.nblk + blk) * p.NB, p.NB * 4u,
+                                bulk_load(smem_u32(sEcol + (accseq % kOzRing) * 2 * kOzMaxNB),
+                                          p.ecol + T.z * p.ecol_z + ((long long)w * p.nblk + blk) * (2 * p.NB), p.NB * 8u,
                                           bar(BFULL + st));
                             bulk_load(smem_u32(sB + (size_t)st * bstage), src + (size_t)c0 * brow, bytes, bar(BFULL + st));
                         }
@@ -680,21 +800,23 @@ __global__ void __launch_bounds__(oz_threads(MULTI), 1) k_oz_gemm(const __grid_c
                         const int ab = (int)(accseq & 1);
                         if (!oz_warp_wait(bar(ACCE + ab), ((accseq >> 1) & 1) ^ 1, abort_flag, p.err, 45)) { ok = false; break; }
 #pragma unroll 1
-                        for (int c0 = 0; c0 < no; c0 += kOzSub) {
+                        for (int c0 = 0; c0 < no; c0 += p.sub) {
                             if (!oz_warp_wait(bar(BFULL + st), bph, abort_flag, p.err, 46)) { ok = false; break; }
                             tc_fence_after();
                             const uint32_t ad = desc_plain(sA0 + as * kAStage + (uint32_t)c0 * kOzLbo, kOzLbo);
                             const uint32_t bd = desc_plain(sB0 + st * bstage, brow);
                             const uint32_t acc = tmem + (uint32_t)(ab * 256);
-                            const int ns = min(kOzSub, no - c0) / 2;
+                            const int ns = min(p.sub, no - c0) / 2;
 #pragma unroll
-                            for (int i = 0; i < kOzSlices; ++i) {
+                            for (int i = 0; i < kOzPlanes; ++i) {
                                 // digits of B this digit of A meets (digit 0's first step also
-                                // meets the zero rows, clearing level 7)
+                                // meets the zero rows, clearing level 7), then the magnitudes
+                                const int later = c0 | (i == kOzSlices ? 0 : i);
 #pragma unroll 1
                                 for (int ks = 0; ks < ns; ++ks)
                                     oz_mma(acc + p.mma_col[i], ad + (i * kPlane >> 4) + (uint32_t)ks * (2 * kOzLbo >> 4),
-                                           bd + (uint32_t)ks * (brow >> 3), p.mma_id[i], (c0 | i | ks) ? 1u : 0u);
+                                           bd + p.mma_row[i] + (uint32_t)ks * (brow >> 3), p.mma_id[i],
+                                           (later | ks) ? 1u : 0u);
                             }
                             oz_commit(bar(BEMPTY + st));
                             if (++st == (uint32_t)p.nbs) {
@@ -745,15 +867,21 @@ OzKernel oz_kernel(int kw, bool multi, bool vec) {
     return vec ? oz_kernel<false, true>(kw) : oz_kernel<false, false>(kw);
 }
 
-// A stages (1 or 2) and B stages (2 to 4) that fit the shared memory.
-void oz_stages(const OzGeom& g, int* na, int* nbs, size_t* smem) {
-    const size_t a = (size_t)kOzSlices * (g.kw / 8) * kOzLbo;
-    const size_t b = (size_t)std::min(kOzSub, g.kw / 8) * 8 * g.NB * 16;
-    *na = 2 * a + 2 * b + kOzMisc + 128 <= kOzSmemMax ? 2 : 1;
+// A stages (1 or 2), chunks of a B stage and B stages (2 to 4) that fit the shared
+// memory: two A stages if two whole B stages fit next to them, then the longest B
+// stage of which three fit (kw = 48, two A stages with B stages of 16 K or one with
+// 48 K: 2.55, 2.19 ms for S2 at N = 24).
+void oz_stages(const OzGeom& g, int* na, int* nbs, int* sub, size_t* smem) {
+    const size_t a = (size_t)kOzPlanes * (g.kw / 8) * kOzLbo, row = (size_t)kOzRows * g.NB * 16;
+    const size_t room = kOzSmemMax - kOzMisc - 128;
+    int c = std::min(kOzMaxSub, g.kw / 8);
+    *na = 2 * a + 2 * c * row <= room ? 2 : 1;
+    while (c > 2 && *na * a + 3 * c * row > room) c -= 2;
     int n = 2;
-    while (n < 4 && *na * a + (n + 1) * b + kOzMisc + 128 <= kOzSmemMax) ++n;
+    while (n < 4 && *na * a + (n + 1) * c * row <= room) ++n;
     *nbs = n;
-    *smem = *na * a + n * b + kOzMisc + 128;
+    *sub = c;
+    *smem = *na * a + n * c * row + kOzMisc + 128;
 }
 
 }  // namespace
@@ -763,11 +891,11 @@ size_t oz_img_bytes(int Nc, long long K) {
     return (size_t)g.img_bytes() + (size_t)g.exps() * 4;
 }
 
-// Windows are at most 96 K, the last one and the rounding of a window to 16 K pad.
+// The last window and the rounding of the others to 16 K pad.
 size_t oz_img_bound(int Nc, long long K) {
     const OzGeom g = oz_geom(Nc, 1);
-    const long long Kp = K + 16 * (K / kOzMaxKw + 1) + kOzMaxKw;
-    return (size_t)(g.nblk * g.NB) * (size_t)(16 * Kp + 4 * (Kp / 16));
+    const long long Kp = K + 16 * (K / kOzLongKw + 1) + kOzMaxKw;
+    return (size_t)(g.nblk * g.NB) * (size_t)(2 * kOzRows * Kp + 8 * (Kp / 16));
 }
 
 gkba_status oz_prepare(gkba_ctx* c) {
@@ -801,8 +929,8 @@ int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items) {
     return (int)((g.nwin + per - 1) / per);
 }
 
-gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const void* img,
-                    int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
+gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const double* B,
+                    long long ldb, long long sBz, const void* img, int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
                     long long sOitem, StageMap map, double flops, double bytes) {
     const OzGeom g = oz_geom(Nc, K);
     if (Nc > kOzMaxCols) return fail(c, GKBA_EINVAL, "oz_gemm: %d columns", Nc);
@@ -817,6 +945,9 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
     p.lda = lda;
     p.sAz = sAz;
     p.M = M;
+    p.B = B;
+    p.ldb = ldb;
+    p.sBz = sBz;
     p.img = (const uint8_t*)img;
     p.img_z = img_nz > 1 ? g.img_bytes() : 0;
     p.ecol = (const int*)((const char*)img + g.img_bytes() * img_nz);
@@ -835,17 +966,19 @@ gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long l
     if (p.nitem != nitem) return fail(c, GKBA_EINVAL, "oz_gemm: %d items for %d windows", nitem, g.nwin);
     p.sOitem = sOitem;
     p.mul = kOzMul;
-    for (int i = 0; i < kOzSlices; ++i) {
-        const int cnt = i == 0 ? 8 : std::min(kOzSlices, kOzLevels - i);
+    for (int i = 0; i < kOzPlanes; ++i) {
+        const bool mag = i == kOzSlices;
+        const int cnt = mag ? 1 : i == 0 ? 8 : std::min(kOzSlices, kOzLevels - i);
         const uint32_t n = (uint32_t)((cnt * p.NB + 15) & ~15);
         p.mma_id[i] = (1u << 4) | ((n >> 3) << 17) | ((uint32_t)(kOzBM >> 4) << 24);
-        p.mma_col[i] = (uint32_t)(i * p.NB);
+        p.mma_col[i] = (uint32_t)(mag ? oz_mag_col(p.NB) : i * p.NB);
+        p.mma_row[i] = mag ? (uint32_t)((kOzSlices + 1) * p.NB) : 0u;  // x 16 bytes, as the descriptor counts
     }
     p.tiles = (long long)nz * p.nitem * p.mtiles;
     if (p.tiles >= 1LL << 31) return fail(c, GKBA_EINVAL, "oz_gemm: %lld tiles", p.tiles);
     p.err = c->dint + 1;
     size_t smem = 0;
-    oz_stages(g, &p.na, &p.nbs, &smem);
+    oz_stages(g, &p.na, &p.nbs, &p.sub, &smem);
     const unsigned grid = (unsigned)std::min<long long>(p.tiles, c->num_sms);
     auto t = launch_begin(c, cls, flops, bytes);
     oz_kernel(g.kw, g.nwin > 1, vec)<<<grid, oz_threads(g.nwin > 1), smem, c->stream>>>(p);
