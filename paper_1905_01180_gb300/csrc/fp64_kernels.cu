@@ -671,13 +671,17 @@ __global__ void k_gkba_units(int N, int nk, int k0, int L, double dt, const doub
 // a fixed summation order (deterministic): pass 1 sums z-range zc of each
 // element into tmp[zc], pass 2 adds the z-ranges in order.  Partials are FP64
 // (FP64 path) or FP32 (tensor-core path); all sums are FP64.
-// Compensated (Kahan) running sum in the partials' own precision: the error
-// stays at a few ulps of the sum whatever the number of terms, and FP32 adds
-// run at full rate (GB300's FP64 rate is low).
+// FP32 partials are added in FP32 with compensation (Kahan): the error stays at a
+// few ulps of the sum whatever the number of terms, and FP32 adds run at full rate
+// (GB300's FP64 rate is low).  The few FP64 partials (oz_items) are plainly added.
 template <typename TP>
-struct KahanSum {
+struct PartialSum {
     TP s = 0, c = 0;
     __device__ __forceinline__ void add(TP x) {
+        if (sizeof(TP) == 8) {
+            s += x;
+            return;
+        }
         const TP y = x - c;
         const TP t = s + y;
         c = (t - s) - y;
@@ -698,7 +702,7 @@ __global__ void k_reduce_partials_p1(int N, int Np, int nb, int nz, int zper, lo
     const int i = rr / N, j = rr % N;
     const long long r_re = (long long)u * 2 * Np + j, r_im = r_re + Np;
     const int z0 = zc * zper, z1 = min(nz, z0 + zper);
-    KahanSum<TP> re[2], im[2];
+    PartialSum<TP> re[2], im[2];
     const TP* base = part + (long long)i * Rld;
     int z = z0;
     for (; z + 2 <= z1; z += 2) {
@@ -1693,8 +1697,8 @@ gkba_status fp64_final(gkba_ctx* c, int nb) {
     const double fl = 4.0 * (double)N4 * N * nb, by = 8.0 * (2 * N4 * nb + N4);
     const long long R = 2LL * N * nb;
     const StageMap m{0, 0, 1, 0, R, (int)R, 1, N};
-    const long long max_z = (long long)(c->part_bytes / (N * R * 8));
-    const int nz = oz_items(c, (int)R, N, N3, max_z);
+    const int nz = oz_items(N3);
+    if ((size_t)(8 * N * R * nz) > c->part_bytes) return fail(c, GKBA_ESTATE, "partial sums of %d units do not fit", nb);
     GKBA_TRY(oz_gemm(c, K_FIN, X13, N3, 0, c->vK64, N3, 0, c->vKimg, 1, N, N3, (double*)c->part, 0, (int)R, 1, nz, N * R, m, fl, by));
     return reduce_partials_launch(c, nb, nz, N * R, R, c->part, false, c->Su);
 }

@@ -105,7 +105,7 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const double form_bytes = !gen ? 0.0 : tc ? 4.0 * 2 * Np * Np * 4 : (2.0 * NN + 4.0 * NN) * 8;
     const double part_per_unit = !gen ? 0.0
                                  : tc ? (std::ceil((double)Np * Np * Np / kTcItemK) * Np * 2.0 * Np * 4)
-                                      : std::ceil((double)NN * N / 8192.0) * N * 2.0 * N * 8;
+                                      : (double)oz_items(NN * N) * N * 2.0 * N * 8;
     const double base_unit = 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
     // digit images of one stage's per-unit operands (the widest: S2 and S3)
     const double img_unit = c->oz ? (double)oz_img_bytes(2 * (int)N, 2 * N) : 0.0;
@@ -142,12 +142,7 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     size_t part_bytes;
     if (!gen) part_bytes = 0;
     else if (tc) part_bytes = tf32_part_bytes((int)Np, ub, c->acc_window);
-    // partial sums of oz_gemm: two items per SM of 128 rows if the cap allows them
-    // next to the units, at least one partial sum of every row
-    else {
-        const double want = (double)N * 8 * 2 * c->num_sms * 128, room = (double)cap - per_unit * ub;
-        part_bytes = (size_t)std::max(2.0 * N * N * 8 * ub, std::min(want, room));
-    }
+    else part_bytes = (size_t)(part_per_unit * ub);
     const size_t oPart = cv.take(part_bytes);
     // the time-linear accumulator's one operand is as long as all units' together
     const size_t ozimg_bytes = !c->oz ? 0

@@ -229,14 +229,14 @@ gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, l
                          long long sOz, int M, int Nc, long long Ktot, int nz, StageMap map,
                          double flops, double bytes);
 // Its parts (oz_gemm.cu).  B is given as digit images: oz_img_bytes(Nc, K) bytes per z, written by oz_slice.
-// K is split into nitem ranges of whole windows (out += item * sOitem);
-// oz_items proposes a number of them for M x Nc outputs, at most max_items.
+// K is split into nitem ranges of whole windows (out += item * sOitem), oz_items(K) for
+// stage S4.
 size_t oz_img_bytes(int Nc, long long K);
 size_t oz_img_bound(int Nc, long long K);  // of any K up to this one
 gkba_status oz_prepare(gkba_ctx* c);
 gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz, int Nc, long long K, int nz,
                      void* img);
-int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items);
+int oz_items(long long K);
 gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const double* B,
                     long long ldb, long long sBz, const void* img, int img_nz, int Nc, long long K, double* out, long long sOz, int M, int nz, int nitem,
                     long long sOitem, StageMap map, double flops, double bytes);

@@ -920,13 +920,18 @@ gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz,
     return launch_end(c, t);
 }
 
-int oz_items(gkba_ctx* c, int M, int Nc, long long K, long long max_items) {
-    const OzGeom g = oz_geom(Nc, K);
-    const long long mt = (M + kOzBM - 1) / kOzBM;
-    // about two items per SM: K is split only while there are fewer row tiles
-    const long long want = std::max(1LL, std::min({2LL * c->num_sms / mt, max_items, (long long)g.nwin}));
-    const long long per = (g.nwin + want - 1) / want;
-    return (int)((g.nwin + per - 1) / per);
+// Eight windows an item, three below 64 windows (N < 16: S4 of few units at N = 13,
+// eight and three 41 and 21 us), more where that were over 144 items (one an SM for
+// a single unit's one row tile, N >= 42).  By K alone: a unit's result does not depend
+// on the units it is computed with, nor on the memory that is free.  The partial sums
+// add 5 % to the traffic of X3 at N = 24 and 6 % at N = 48; splitting only where row
+// tiles were few took 2.27 instead of 1.77 ms for S4 at N = 24, 301 points.
+constexpr int kOzMaxItems = 144;
+int oz_items(long long K) {
+    const int nwin = oz_geom(1, K).nwin, windows = nwin < 64 ? 3 : 8;
+    const int want = std::min(kOzMaxItems, (nwin + windows - 1) / windows);
+    const int per = (nwin + want - 1) / want;
+    return (nwin + per - 1) / per;
 }
 
 gkba_status oz_gemm(gkba_ctx* c, int cls, const double* A, long long lda, long long sAz, const double* B,
