@@ -335,6 +335,12 @@ __global__ void k_set_identity(int N, int count, double2* __restrict__ A) {
     A[e] = make_double2((r / N) == (r % N) ? 1.0 : 0.0, 0.0);
 }
 
+// Halvings of an exponential's argument, and squarings of its result, at most: every
+// exponential takes as many of the one as of the other (with 30 and 16, arguments of a
+// norm above 2^15 gave a root of the exponential).  An argument left larger than 1/2
+// keeps the polynomial's accuracy up to a norm of 2^16 (0.5^19 / 19! becomes 1 / 19!).
+constexpr int kMaxSquarings = 16;
+
 // expm set-up: A = -i dt (hA + hB)/2; writes A into X, its 1-norm (max column
 // sum of |A_ij|) and the number of squarings s so that ||A||/2^s <= 1/2, then
 // scales X by 2^-s.  One block.
@@ -361,7 +367,7 @@ __global__ void k_expm_setup(int N, double dt, const double2* __restrict__ hA,
     }
     const double nrm = colmax[0];
     int s = 0;
-    while (s < 30 && ldexp(nrm, -s) > 0.5) ++s;
+    while (s < kMaxSquarings && ldexp(nrm, -s) > 0.5) ++s;
     const double scale = ldexp(1.0, -s);
     for (int e = tid; e < N * N; e += blockDim.x) {
         const double hr = 0.5 * (hA[e].x + hB[e].x), hi = 0.5 * (hA[e].y + hB[e].y);
@@ -378,7 +384,7 @@ __global__ void k_expm_setup(int N, double dt, const double2* __restrict__ hA,
 // (-i dt (hA + hB)/2, or a general matrix Z) scaled by 2^-s so that its 1-norm is
 // at most 1/2, the degree-18 Taylor polynomial as four Horner steps in X^4
 // (Paterson and Stockmeyer, SIAM J. Comput. 2, 1973: seven products instead of
-// eighteen), min(s, 16) squarings.  From kExpmOneN + 1 rows on a cluster of eight
+// eighteen), s squarings.  From kExpmOneN + 1 rows on a cluster of eight
 // CTAs shares every product: each keeps all matrices in shared memory, computes
 // an eighth and writes it to all eight (distributed shared memory, one cluster
 // barrier a product); below, one CTA is faster than the barriers.  One SM's FP64
@@ -492,7 +498,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(256)
     for (int j = 0; j < n; ++j) nrm = nrm < colsum[j] ? colsum[j] : nrm;
     if (!SEQ) nrm *= (TN)1.0001;
     int s = 0;
-    for (; s < 30 && nrm > (TN)0.5; ++s) nrm *= (TN)0.5;
+    for (; s < kMaxSquarings && nrm > (TN)0.5; ++s) nrm *= (TN)0.5;
     const double scale = __hiloint2double((1023 - s) << 20, 0);
     for (int e = tid; e < nn; e += 256) {
         X[e] = make_double2(scale * X[e].x, scale * X[e].y);
@@ -529,8 +535,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(256)
             double2* t = y; y = z; z = t;
         }
     }
-    const int nsq = s < 16 ? s : 16;
-    for (int q = 0; q < nsq; ++q) {
+    for (int q = 0; q < s; ++q) {
         expm_product<CTAS, SEQ>(n, rank, y, y, z, -1, nullptr, nullptr, nullptr);
         double2* t = y; y = z; z = t;
     }
@@ -548,12 +553,12 @@ __global__ void k_expm_lead(int n, double c16, double c17, double c18, const dou
     Y[e] = make_double2(fma(c17, X[e].x, c18 * X2[e].x) + (e / n == e % n ? c16 : 0.0),
                         fma(c17, X[e].y, c18 * X2[e].y));
 }
-// The result of *s squarings (at most 16) that alternated between two buffers.
+// The result of *s squarings that alternated between two buffers.
 __global__ void k_expm_select(long long n, const int* __restrict__ s, const double2* __restrict__ even,
                               const double2* __restrict__ odd, double2* __restrict__ U, double2* __restrict__ U2) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
-    const double2 x = (min(*s, 16) & 1) ? odd[e] : even[e];
+    const double2 x = (*s & 1) ? odd[e] : even[e];
     U[e] = x;
     if (U2) U2[e] = x;
 }
@@ -1157,7 +1162,7 @@ __global__ void k_expm_setup_general(int n, const double2* __restrict__ Z, doubl
     }
     const double nrm = colmax[0];
     int s = 0;
-    while (s < 16 && ldexp(nrm, -s) > 0.5) ++s;
+    while (s < kMaxSquarings && ldexp(nrm, -s) > 0.5) ++s;
     const double scale = ldexp(1.0, -s);
     for (int e = threadIdx.x; e < n * n; e += blockDim.x)
         X[e] = make_double2(scale * Z[e].x, scale * Z[e].y);
@@ -1335,8 +1340,8 @@ gkba_status heun_stage(gkba_ctx* c, const double2* hhf, const double2* rho, cons
 
 // exp(X) by products spread over all SMs: the degree-18 Taylor polynomial in the
 // form that k_expm_small takes (Horner for split-TF32 contexts, else Paterson and
-// Stockmeyer), then up to 16 squarings of which the device-side count c->dint[0]
-// runs.  X: the scaled argument; X2, X3, X4, Y, W: n x n scratch; the result goes
+// Stockmeyer), then kMaxSquarings squarings of which the device-side count
+// c->dint[0] runs.  X: the scaled argument; X2, X3, X4, Y, W: n x n scratch; the result goes
 // to U (and U2).
 static gkba_status expm_products(gkba_ctx* c, int n, const double2* X, double2* X2, double2* X3, double2* X4,
                                  double2* Y, double2* W, double2* U, double2* U2) {
@@ -1382,7 +1387,7 @@ static gkba_status expm_products(gkba_ctx* c, int n, const double2* X, double2* 
     }
     // X3 is free now: squarings alternate between y and it
     double2* sq[2] = {y, X3};
-    for (int i = 0; i < 16; ++i)
+    for (int i = 0; i < kMaxSquarings; ++i)
         GKBA_TRY(zgemm_impl(c, K_STEP, n, 'N', 'N', one, sq[i & 1], 0, sq[i & 1], 0, zero, sq[(i + 1) & 1], 0, 1, 0,
                             ZPoly{}, c->dint + 0, i));
     auto t = launch_begin(c, K_STEP, 0.0, 0.0);
