@@ -113,7 +113,10 @@ typedef struct {
     void* cuda_stream; /* cudaStream_t to run on; NULL = the library creates one */
     size_t workspace_bytes; /* cap on the contraction workspace (0 = default 64 GiB, at most
                                85 % of the free device memory);
-                               the batch of (t_k, component) units is sized to fit */
+                               the batch of (t_k, component) units is sized to fit (to
+                               within 4 KiB of alignment, in FP64 at N <= 3 64 KiB more).
+                               The model's tensors (about 60 N^4 bytes in FP64) and the
+                               history store are outside it */
     int device;        /* CUDA device ordinal (-1 = current device) */
     int timing;        /* nonzero: time every contraction kernel with CUDA events
                           (see gkba_get_stats) */

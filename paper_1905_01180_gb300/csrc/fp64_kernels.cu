@@ -1273,11 +1273,16 @@ gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, l
                          const double* B, long long ldb, long long sBz, double* out,
                          long long sOz, int M, int Nc, long long Ktot, int nz, StageMap map,
                          double flops, double bytes) {
-    const int nzB = sBz ? nz : 1;
-    if (oz_img_bytes(Nc, Ktot) * nzB > c->ozimg_bytes)
-        return fail(c, GKBA_ESTATE, "digit images of %d operands of %d x %lld do not fit", nzB, Nc, Ktot);
-    GKBA_TRY(oz_slice(c, B, ldb, sBz, Nc, Ktot, nzB, c->ozimg));
-    return oz_gemm(c, cls, A, lda, sAz, B, ldb, sBz, c->ozimg, nzB, Nc, Ktot, out, sOz, M, nz, 1, 0, map, flops, bytes);
+    const long long fit = (long long)(c->ozimg_bytes / oz_img_bytes(Nc, Ktot));
+    if (fit < 1) return fail(c, GKBA_ESTATE, "the digit image of an operand of %d x %lld does not fit", Nc, Ktot);
+    const int most = sBz ? (int)std::min<long long>(fit, nz) : nz;
+    for (int z = 0; z < nz; z += most) {
+        const int n = std::min(most, nz - z), nB = sBz ? n : 1;
+        GKBA_TRY(oz_slice(c, B + z * sBz, ldb, sBz, Nc, Ktot, nB, c->ozimg));
+        GKBA_TRY(oz_gemm(c, cls, A + z * sAz, lda, sAz, B + z * sBz, ldb, sBz, c->ozimg, nB, Nc, Ktot, out + z * sOz, sOz,
+                         M, n, 1, 0, map, flops * n / nz, bytes * n / nz));
+    }
+    return GKBA_OK;
 }
 
 static gkba_status zgemm_impl(gkba_ctx* c, int cls, int n, char opA, char opB, double2 alpha,

@@ -102,14 +102,14 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const bool gen = c->kind == GKBA_V_GENERAL;  // structured kinds need no stage buffers
     const long long Np = c->Np;
     const double x_bytes = !gen ? 0.0 : tc ? 2.0 * Np * Np * Np * Np * 4 : 2.0 * NN * NN * 8;
-    const double form_bytes = !gen ? 0.0 : tc ? 4.0 * 2 * Np * Np * 4 : (2.0 * NN + 4.0 * NN) * 8;
-    const double part_per_unit = !gen ? 0.0
-                                 : tc ? (std::ceil((double)Np * Np * Np / kTcItemK) * Np * 2.0 * Np * 4)
-                                      : (double)oz_items(NN * N) * N * 2.0 * N * 8;
-    const double base_unit = 2 * x_bytes + form_bytes + part_per_unit + (4.0 + kReduceSplit) * NN * 16 + 8;
-    // digit images of one stage's per-unit operands (the widest: S2 and S3)
-    const double img_unit = c->oz ? (double)oz_img_bytes(2 * (int)N, 2 * N) : 0.0;
-    const double per_unit = base_unit + img_unit;
+    // FP64: the real forms of up to three matrices; stage S4's partial sums share X2,
+    // the digit images the reduction scratch and S Gbar the forms of S1, none of which
+    // is in use at the same time
+    const double form_bytes = !gen ? 0.0 : tc ? 4.0 * 2 * Np * Np * 4 : (2.0 * NN + 4.0 * NN + 4.0 * NN) * 8;
+    const double part_per_unit =
+        !gen || !tc ? 0.0 : (std::ceil((double)Np * Np * Np / kTcItemK) * Np * 2.0 * Np * 4);
+    const double per_unit =
+        2 * x_bytes + form_bytes + part_per_unit + ((c->oz ? 3.0 : 4.0) + kReduceSplit) * NN * 16 + 8;
     size_t cap = c->ws_cap;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
@@ -118,11 +118,9 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     }
     long long fit = (long long)((double)cap / per_unit);
     fit -= fit & 1;
-    // a cap that holds two units without their images is met up to the images
-    if (fit < 2 && (double)cap >= 2 * base_unit) fit = 2;
     if (fit < 2)
         return fail(c, GKBA_ENOMEM, "workspace cap %.3g GB holds fewer than 2 units (%.3g GB each)",
-                    cap / 1e9, base_unit / 1e9);
+                    cap / 1e9, per_unit / 1e9);
     int ub = (int)std::min<long long>(fit, want_units);
     if (c->ws && ub <= c->ub_cap) {
         c->ub = ub;
@@ -139,17 +137,8 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const size_t x13_bytes = (size_t)std::max(x_bytes * ub, std::floor(x3_blocked));
     const size_t oX13 = cv.take(x13_bytes);
     const size_t oX2 = cv.take((size_t)(x_bytes * ub));
-    size_t part_bytes;
-    if (!gen) part_bytes = 0;
-    else if (tc) part_bytes = tf32_part_bytes((int)Np, ub, c->acc_window);
-    else part_bytes = (size_t)(part_per_unit * ub);
+    const size_t part_bytes = gen && tc ? tf32_part_bytes((int)Np, ub, c->acc_window) : 0;
     const size_t oPart = cv.take(part_bytes);
-    // the time-linear accumulator's one operand is as long as all units' together
-    const size_t ozimg_bytes = !c->oz ? 0
-                               : std::max((size_t)(img_unit * ub), c->history == GKBA_HISTORY_TIME_LINEAR
-                                                                       ? oz_img_bound(2 * (int)N, 2LL * N * ub)
-                                                                       : 0);
-    const size_t oImg = cv.take(ozimg_bytes);
     const size_t oB1 = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 2 * Np * Np * ub * 4) : (size_t)(2LL * NN * ub * 8));
     const size_t oG = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 4 * Np * Np * ub * 4) : (size_t)(4LL * NN * ub * 8));
     const size_t oG3 = cv.take(!gen ? 0 : tc ? (size_t)(2LL * 4 * Np * Np * ub * 4) : (size_t)(4LL * NN * ub * 8));
@@ -157,8 +146,16 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     const size_t oMb = cv.take((size_t)(ub * NN * 16));
     const size_t oCoef = cv.take((size_t)ub * 8);
     const size_t oSu = cv.take((size_t)(ub * NN * 16));
-    const size_t oYu = cv.take((size_t)(ub * NN * 16));
-    const size_t oRed = cv.take((size_t)(kReduceSplit * ub * NN * 16));
+    const size_t oYu = cv.take(c->oz ? 0 : (size_t)(ub * NN * 16));
+    size_t red_bytes = (size_t)(kReduceSplit * ub * NN * 16);
+    if (c->oz) {
+        // images of all units fit from N = 4 on; smaller bases run in batches of what
+        // fits 64 KiB.  The time-linear accumulator's operand is one of all units.
+        red_bytes = std::max(red_bytes, std::min(oz_img_bytes(2 * (int)N, 2 * N) * ub, (size_t)64 << 10));
+        if (c->history == GKBA_HISTORY_TIME_LINEAR)
+            for (int nb = 2; nb <= ub; nb += 2) red_bytes = std::max(red_bytes, oz_img_bytes(2 * (int)N, 2LL * N * nb));
+    }
+    const size_t oRed = cv.take(red_bytes);
     void* ws = nullptr;
     if (cudaMalloc(&ws, cv.off) != cudaSuccess) {
         cudaGetLastError();
@@ -172,10 +169,10 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     c->X13 = b + oX13;
     c->x13_bytes = x13_bytes;
     c->X2 = b + oX2;
-    c->part = b + oPart;
-    c->part_bytes = part_bytes;
-    c->ozimg = b + oImg;
-    c->ozimg_bytes = ozimg_bytes;
+    c->part = b + (c->oz ? oX2 : oPart);
+    c->part_bytes = c->oz ? (size_t)(x_bytes * ub) : part_bytes;
+    c->ozimg = b + oRed;
+    c->ozimg_bytes = c->oz ? red_bytes : 0;
     c->formsB1 = b + oB1;
     c->formsG = b + oG;
     c->formsG3 = b + oG3;
@@ -183,7 +180,7 @@ gkba_status ensure_workspace(gkba_ctx* c, int want_units) {
     c->Mb = (double2*)(b + oMb);
     c->coef = (double*)(b + oCoef);
     c->Su = (double2*)(b + oSu);
-    c->Yu = (double2*)(b + oYu);
+    c->Yu = (double2*)(b + (c->oz ? oB1 : oYu));
     c->red_tmp = (double2*)(b + oRed);
     return GKBA_OK;
 }

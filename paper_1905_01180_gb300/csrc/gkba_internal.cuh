@@ -126,13 +126,13 @@ struct gkba_ctx {
     void* X13 = nullptr;
     size_t x13_bytes = 0;
     void* X2 = nullptr;
-    void* part = nullptr;
+    void* part = nullptr;        // partial sums of S4 (oz: in X2)
     size_t part_bytes = 0;
     double2* PQ = nullptr;       // P and Q for ub/2 history points: 2 * (ub/2) * N*N
     void* formsB1 = nullptr;     // per-unit B operand of S1
     void* formsG = nullptr;      // per-unit B operand of S2/S3
     void* formsG3 = nullptr;     // per-unit B operand of S3 when its slot differs (sep_A)
-    void* ozimg = nullptr;       // digit images of one stage's B operands (oz)
+    void* ozimg = nullptr;       // digit images of one stage's B operands (oz), in red_tmp
     size_t ozimg_bytes = 0;
     double2* vjp = nullptr;      // adjoint scratch: 10 blocks of vjp_units N*N units
     int vjp_units = 0;
@@ -149,7 +149,7 @@ struct gkba_ctx {
     double2* Mb = nullptr;       // per-unit Gbar (= the right factor of S.Gbar), ub * N*N
     double* coef = nullptr;      // per-unit weight (+-c_k), ub
     double2* Su = nullptr;       // per-unit S, ub * N*N
-    double2* Yu = nullptr;       // per-unit coef * S . Gbar, ub * N*N
+    double2* Yu = nullptr;       // per-unit coef * S . Gbar, ub * N*N (oz: in formsB1)
     double2* red_tmp = nullptr;  // split-K reduction scratch: kReduceSplit * ub * N*N
 
     // time-linear history (GKBA_HISTORY_TIME_LINEAR): T(t_n, t_k) = Ucal_n Ucal_k^+
@@ -232,7 +232,6 @@ gkba_status gemm64_stage(gkba_ctx* c, int cls, const double* A, long long lda, l
 // K is split into nitem ranges of whole windows (out += item * sOitem), oz_items(K) for
 // stage S4.
 size_t oz_img_bytes(int Nc, long long K);
-size_t oz_img_bound(int Nc, long long K);  // of any K up to this one
 gkba_status oz_prepare(gkba_ctx* c);
 gkba_status oz_slice(gkba_ctx* c, const double* B, long long ldb, long long sBz, int Nc, long long K, int nz,
                      void* img);

@@ -891,13 +891,6 @@ size_t oz_img_bytes(int Nc, long long K) {
     return (size_t)g.img_bytes() + (size_t)g.exps() * 4;
 }
 
-// The last window and the rounding of the others to 16 K pad.
-size_t oz_img_bound(int Nc, long long K) {
-    const OzGeom g = oz_geom(Nc, 1);
-    const long long Kp = K + 16 * (K / kOzLongKw + 1) + kOzMaxKw;
-    return (size_t)(g.nblk * g.NB) * (size_t)(2 * kOzRows * Kp + 8 * (Kp / 16));
-}
-
 gkba_status oz_prepare(gkba_ctx* c) {
     for (int kw = 16; kw <= kOzMaxKw; kw += 16)
         for (int m = 0; m < 4; ++m)
