@@ -304,7 +304,7 @@ __device__ __forceinline__ void oz_again(uint32_t rows, int lane, const double* 
         if (((rows >> mine) & 1u) == 0u) mine = (int)pick[0];
         const double* ar = a + (long long)mine * lda;
         double d = 0.0;
-#pragma unroll 2
+#pragma unroll 4
         for (int k = lane & 7; k < Kw; k += 8) d = fma(__ldg(ar + k), __ldg(b + k), d);
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
