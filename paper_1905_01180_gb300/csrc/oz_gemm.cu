@@ -13,13 +13,13 @@
 // eighth MMA and summed again by FMAs, so that the path is as accurate as FMA chains
 // for operands of any scaling (oz_accept; tests/test_oz_graded.py).
 //
-// Whole calls, FMA chain -> here: Heun step at N = 24, 301 points 309 -> 18.2 ms; 40
-// self-energies at N = 33 78 -> 3.6 ms; Heun step at N = 10, 501 points 23.8 -> 1.7 ms.
+// Whole calls, FMA chain -> here: Heun step at N = 24, 301 points 309 -> 17.2 ms; 40
+// self-energies at N = 33 78 -> 3.5 ms; Heun step at N = 10, 501 points 23.8 -> 1.6 ms.
 // Without the check of the results: 15.8, 2.8 and 1.4 ms.  What is summed again costs
 // most for matrices near a diagonal or nearly real (a propagation's start; three
-// time-linear steps at N = 48 137 -> 27 ms, 12 without the check) and at worst, N = 24
+// time-linear steps at N = 48 137 -> 30 ms, 12 without the check) and at worst, N = 24
 // with imaginary parts of 1e-3, takes 0.6 of the FMA chain's time (50 -> 30 ms for 200
-// self-energies; 13 ms where rows and columns span 1e-6 .. 1e6).
+// self-energies; 14 ms where rows and columns span 1e-6 .. 1e6).
 //
 // What bounds it: the latency of two chains of instructions that are each half busy,
 // the epilogue's (about 70 a result) and the converter's (about 53 an element).
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ B, 
 // A result that oz_accept turns down, or that leaves the normal range, is summed
 // again by FMAs in the epilogue, from A and B in memory (oz_again: eight lanes a row;
 // with every lane on its own row a warp pays for 32 rows whenever one is wanted, and
-// the N = 48 propagation took 46 ms instead of 27).
+// the N = 48 propagation took 46 ms instead of 30).
 //
 // One window (K <= 96, stages S1-S3 up to N = 48): a row tile is converted
 // once and multiplied with every column block.  Longer K: per block and
